@@ -113,8 +113,8 @@ struct amr_ctx {
   bool classified = false;               // cls holds the classes of the last refinement's adjacent cells
   int prev_levels = -1;                  // levels of the kept previous hierarchy (-1: none kept)
   // adjoint
-  DevBuf idx, vert_off, vert_corners, face_off, face_links, sort_keys, grad_face, sort_scratch, group_cnt, lvl_ptrs;
-  bool vert_groups = false, face_groups = false;
+  DevBuf idx, vert_off, vert_corners, face_key, face_acc, face_lines, grad_face, sort_scratch, group_cnt, lvl_ptrs;
+  bool vert_groups = false;
   int64_t n_links = 0;
   // misc layout: [0..CNT_N) u64 counters, then u32 err word, u32 work, u64 totals[4]
   unsigned long long* counters = nullptr;
@@ -477,7 +477,7 @@ void amr_ctx_free(amr_ctx* ctx) {
                    &ctx->count,     &ctx->offsets,      &ctx->ids,        &ctx->payload,    &ctx->scratch,
                    &ctx->misc,      &ctx->scal,         &ctx->adj_cell,   &ctx->adj_off,    &ctx->adj_ids,
                    &ctx->link_cell, &ctx->link_dir,     &ctx->link_q,     &ctx->link_face,  &ctx->link_stage, &ctx->idx,
-                   &ctx->vert_off,  &ctx->vert_corners, &ctx->face_off,   &ctx->face_links, &ctx->sort_keys,
+                   &ctx->vert_off,  &ctx->vert_corners, &ctx->face_key,   &ctx->face_acc,   &ctx->face_lines,
                    &ctx->grad_face, &ctx->sort_scratch, &ctx->group_cnt,  &ctx->lvl_ptrs,   &ctx->table,
                    &ctx->face_gid,  &ctx->fstat,        &ctx->spill,      &ctx->calg,       &ctx->defer};
   for (DevBuf* b : all) release(ctx, *b);
@@ -1218,7 +1218,7 @@ amr_status amr_geom_load(amr_ctx* ctx, const float* coords, int64_t n_verts, con
   if (n_faces > 0 && !coords) return fail(ctx, AMR_EINVAL, "null coordinates");
   if (idx && n_verts <= 0 && n_faces > 0) return fail(ctx, AMR_EINVAL, "indexed input needs n_verts > 0");
   ctx->loaded = ctx->binned = ctx->refined = false;
-  ctx->vert_groups = ctx->face_groups = false;
+  ctx->vert_groups = false;
   ctx->nf = n_faces;
   ctx->nv = idx ? n_verts : 0;
   ctx->indexed = idx != nullptr;
@@ -1341,7 +1341,6 @@ amr_status amr_refine_near_wall(amr_ctx* ctx, const amr_refine_params* prm, amr_
   }
   ctx->refined = false;
   ctx->classified = false;
-  ctx->face_groups = false;
   ctx->n_links = 0;
   ctx->last.n_levels = 0;  // until this refinement succeeds
   GeomParams& g = ctx->geoms[0];
@@ -1400,11 +1399,6 @@ amr_status group_by_key(amr_ctx* ctx, const uint32_t* keys, int64_t n, int64_t n
 amr_status amr_backward(amr_ctx* ctx, const float* grad_q, float* grad_out) {
   const int D = ctx->dom.dim;
   const int64_t nl = ctx->n_links, nf = ctx->nf;
-  if (!ctx->face_groups) {
-    TRY(group_by_key(ctx, static_cast<const uint32_t*>(ctx->link_face.p), nl, nf, ctx->face_off, ctx->face_links,
-                     "adjoint_group_links"));
-    ctx->face_groups = true;
-  }
   const bool indexed = ctx->indexed;
   if (indexed && !ctx->vert_groups) {
     TRY(group_by_key(ctx, static_cast<const uint32_t*>(ctx->idx.p), nf * D, ctx->nv, ctx->vert_off,
@@ -1424,13 +1418,21 @@ amr_status amr_backward(amr_ctx* ctx, const float* grad_q, float* grad_out) {
   a.face_gid = ctx->multi ? static_cast<const uint32_t*>(ctx->face_gid.p) : nullptr;
   a.level_blocks = static_cast<const int32_t* const*>(ctx->lvl_ptrs.p);
   a.X = static_cast<const float*>(ctx->X.p);
-  a.nrm = static_cast<const float*>(ctx->nrm.p);
-  a.face_off = static_cast<const uint32_t*>(ctx->face_off.p);
-  a.face_links = static_cast<const uint32_t*>(ctx->face_links.p);
+  a.rec = static_cast<const FaceRec3*>(ctx->frec.p);
+  TRY(ensure(ctx, ctx->face_key, sizeof(uint32_t) * (size_t)(nf > 0 ? nf : 1)));
+  TRY(ensure(ctx, ctx->face_acc, sizeof(unsigned long long) * (size_t)(D + 1) * (size_t)(nf > 0 ? nf : 1)));
+  TRY(ensure(ctx, ctx->face_lines, sizeof(FaceLines) * (size_t)(nf > 0 ? nf : 1)));
+  a.blocks = static_cast<const int32_t*>(ctx->lv[ctx->geoms[0].n_levels - 1].blocks.p);
+  a.face_lines = static_cast<FaceLines*>(ctx->face_lines.p);
+  a.n_links = nl;
+  a.count_bits = key_bits(nl);
+  a.face_key = static_cast<uint32_t*>(ctx->face_key.p);
+  a.face_acc = static_cast<unsigned long long*>(ctx->face_acc.p);
   a.grad_q = grad_q;
   a.link_cell = static_cast<const uint32_t*>(ctx->link_cell.p);
   a.link_dir = static_cast<const uint8_t*>(ctx->link_dir.p);
   a.link_q = static_cast<const float*>(ctx->link_q.p);
+  a.link_face = static_cast<const uint32_t*>(ctx->link_face.p);
   a.adj_cell = static_cast<const uint32_t*>(ctx->adj_cell.p);
   a.grad_face = gface;
   cudaStream_t st = ctx->stream;
@@ -1541,7 +1543,6 @@ amr_status amr_fluid_links(amr_ctx* ctx, amr_refine_result* out) {
     CK(cudaMemcpyAsync(lf, ctx->tl_face.p, sizeof(uint32_t) * kept, cudaMemcpyDeviceToDevice, st));
     ctx->n_links = (int64_t)kept;
   }
-  ctx->face_groups = false;
   ctx->last.n_links = ctx->n_links;
   *out = ctx->last;
   return AMR_OK;
@@ -1836,7 +1837,7 @@ amr_status batch_gather(amr_batch* b) {
   CK(cudaGetLastError());
   ctx->loaded = true;
   ++ctx->load_gen;
-  ctx->vert_groups = ctx->face_groups = false;
+  ctx->vert_groups = false;
   return AMR_OK;
 }
 
@@ -1981,7 +1982,6 @@ amr_status amr_batch_run(amr_batch* b, const amr_refine_params* prm, amr_refine_
     }
   }
   ctx->refined = false;
-  ctx->face_groups = false;
   TRY(batch_gather(b));
   TRY(amr_bin_all(ctx));
   amr_refine_result r{};

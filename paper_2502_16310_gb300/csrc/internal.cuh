@@ -353,6 +353,39 @@ __device__ __forceinline__ T warp_inclusive_scan(T v) {
   return v;
 }
 
+// --- lattice directions ------------------------------------------------------
+// D3Q19 direction i (1..18), component a: 1..6 = +x,-x,+y,-y,+z,-z; 7..18 =
+// the xy, xz and yz plane diagonals, each as (+,+), (-,-), (+,-), (-,+).
+__host__ __device__ constexpr int d3q19_c(int i, int a) {
+  if (i <= 6) return ((i - 1) >> 1) == a ? ((i & 1) ? 1 : -1) : 0;
+  const int p = (i - 7) >> 2, j = (i - 7) & 3;
+  const int a1 = p == 2 ? 1 : 0;  // first axis of the plane
+  const int a2 = p == 0 ? 1 : 2;  // second axis
+  if (a == a1) return (j == 0 || j == 2) ? 1 : -1;
+  if (a == a2) return (j == 0 || j == 3) ? 1 : -1;
+  return 0;
+}
+// D2Q9 direction i (1..8), component a: +x, +y, -x, -y, then (+,+), (-,+), (-,-), (+,-).
+__host__ __device__ constexpr int d2q9_c(int i, int a) {
+  if (i <= 4) return ((i - 1) & 1) == a ? (i <= 2 ? 1 : -1) : 0;
+  return a == 0 ? (i == 5 || i == 8 ? 1 : -1) : (i <= 6 ? 1 : -1);
+}
+// D3Q19 components packed two bits per direction (value + 1), for lanes that
+// each hold a different direction.
+__host__ __device__ constexpr uint64_t pack_dir_axis(int a) {
+  uint64_t k = 0;
+  for (int i = 1; i <= 18; ++i) k |= (uint64_t)(d3q19_c(i, a) + 1) << (2 * i);
+  return k;
+}
+constexpr uint64_t kDirX = pack_dir_axis(0), kDirY = pack_dir_axis(1), kDirZ = pack_dir_axis(2);
+__device__ __forceinline__ float dir_comp(uint64_t k, int i) { return (float)((int)((k >> (2 * i)) & 3ull) - 1); }
+constexpr uint64_t pack_dir2_axis(int a) {
+  uint64_t k = 0;
+  for (int i = 1; i <= 8; ++i) k |= (uint64_t)(d2q9_c(i, a) + 1) << (2 * i);
+  return k;
+}
+constexpr uint64_t kDir2X = pack_dir2_axis(0), kDir2Y = pack_dir2_axis(1);
+
 // ---------------------------------------------------------------------------
 // Launchers (host side).  All are asynchronous on `st` and return the number
 // of kernels they launched.  Sizes marked "device" are read by the kernels
@@ -629,21 +662,35 @@ int launch_links(const LinkArgs& a, void* scratch, int num_sms, cudaStream_t st)
 int launch_advance(const uint64_t* level_tot, const uint64_t* n_links, uint64_t* run, uint32_t* adj_off,
                    int64_t cap_cells, unsigned* err, bool close, cudaStream_t st);
 
+// What a face's links share in the adjoint (see k_face_lines).
+struct __align__(16) FaceLines {
+  float v0[3];
+  int extent;
+  float inv[9];
+  float pad[3];
+};
+static_assert(sizeof(FaceLines) == 64, "one record is two sectors");
+
 struct AdjointArgs {
   int dim;
   int64_t nf;
   GeomParams g0;
   const GeomParams* table;
   const uint32_t* face_gid;    // nullable
-  const int32_t* const* level_blocks;  // device array of per-level block pointers
+  const int32_t* const* level_blocks;  // device array of per-level block pointers (batches)
+  const int32_t* blocks;       // single geometry: the finest level's blocks
   const float* X;
-  const float* nrm;
-  const uint32_t* face_off;    // [nf + 1]
-  const uint32_t* face_links;  // link indices grouped by face, ascending within a face
+  const FaceRec3* rec;         // 3D face records
+  int64_t n_links;
+  int count_bits;              // n_links <= 2^count_bits
+  FaceLines* face_lines;       // [nf]
+  uint32_t* face_key;          // [nf] scale of each face's sums (see k_face_scale)
+  unsigned long long* face_acc;  // [nf][dim + 1] sums of each face's terms, fixed point
   const float* grad_q;
   const uint32_t* link_cell;
   const uint8_t* link_dir;
   const float* link_q;
+  const uint32_t* link_face;
   const uint32_t* adj_cell;
   float* grad_face;            // [nf][D][D]
 };
@@ -653,6 +700,7 @@ size_t radix_sort_scratch_bytes(int64_t n);
 int launch_stable_sort(const uint32_t* keys, int64_t n, int key_bits, uint32_t* sorted_keys, uint32_t* sorted_vals,
                        const uint32_t* vals_in, void* scratch, uint64_t* total, unsigned* err, cudaStream_t st);
 int launch_count_keys(const uint32_t* keys, int64_t n, uint32_t* cnt, cudaStream_t st);
+// Gradient of every face's corners from its links (zero without links); returns the launch count.
 int launch_face_grad(const AdjointArgs& a, cudaStream_t st);
 int launch_vertex_grad(int dim, const float* grad_face, const uint32_t* vert_off, const uint32_t* vert_corners,
                        int64_t nv, float* out, cudaStream_t st);

@@ -38,17 +38,6 @@ static_assert(kLThreads == kLRows, "phase 0 and 2 map thread i to row i");
 
 __constant__ int c_d2q9[9][2] = {{0, 0}, {1, 0}, {0, 1}, {-1, 0}, {0, -1}, {1, 1}, {-1, 1}, {-1, -1}, {1, -1}};
 
-// D3Q19 direction i (1..18), component a: 1..6 = +x,-x,+y,-y,+z,-z; 7..18 =
-// the xy, xz and yz plane diagonals, each as (+,+), (-,-), (+,-), (-,+).
-__host__ __device__ constexpr int d3q19_c(int i, int a) {
-  if (i <= 6) return ((i - 1) >> 1) == a ? ((i & 1) ? 1 : -1) : 0;
-  const int p = (i - 7) >> 2, j = (i - 7) & 3;
-  const int a1 = p == 2 ? 1 : 0;  // first axis of the plane
-  const int a2 = p == 0 ? 1 : 2;  // second axis
-  if (a == a1) return (j == 0 || j == 2) ? 1 : -1;
-  if (a == a2) return (j == 0 || j == 3) ? 1 : -1;
-  return 0;
-}
 static_assert(d3q19_c(1, 0) == 1 && d3q19_c(2, 0) == -1 && d3q19_c(5, 2) == 1 && d3q19_c(6, 2) == -1, "axes");
 static_assert(d3q19_c(7, 0) == 1 && d3q19_c(7, 1) == 1 && d3q19_c(8, 0) == -1 && d3q19_c(8, 1) == -1, "xy");
 static_assert(d3q19_c(9, 0) == 1 && d3q19_c(9, 1) == -1 && d3q19_c(10, 0) == -1 && d3q19_c(10, 1) == 1, "xy");
@@ -175,16 +164,6 @@ struct LinkTiles {
   uint8_t* stage_row;            // their row within the tile
   int64_t stage_cap;
 };
-
-// D3Q19 components packed two bits per direction (value + 1), for lanes that
-// each hold a different direction.
-__host__ __device__ constexpr uint64_t pack_dir_axis(int a) {
-  uint64_t k = 0;
-  for (int i = 1; i <= 18; ++i) k |= (uint64_t)(d3q19_c(i, a) + 1) << (2 * i);
-  return k;
-}
-constexpr uint64_t kDirX = pack_dir_axis(0), kDirY = pack_dir_axis(1), kDirZ = pack_dir_axis(2);
-__device__ __forceinline__ float dir_comp(uint64_t k, int i) { return (float)((int)((k >> (2 * i)) & 3ull) - 1); }
 
 // Per-pair quantities the direction tests share (one record per lane, 7 x 16 B
 // so that lanes reading different records hit different banks).
