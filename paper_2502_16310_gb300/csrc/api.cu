@@ -614,6 +614,8 @@ struct Plan {
   bool fin_at[AMR_MAX_LEVELS];      // some geometry ends at this level
   bool cont_after[AMR_MAX_LEVELS];  // some geometry continues below this level
   bool face_at[AMR_MAX_LEVELS];     // some geometry's blocks of the level are marked face by face
+  bool unit_at[AMR_MAX_LEVELS];     // ... with d the cell size (kFaceUnit)
+  bool plain_at[AMR_MAX_LEVELS];    // ... with another d or predicate
   bool walk_at[AMR_MAX_LEVELS];     // some geometry's blocks of the level are walked
   bool adjacency, links;
   int lattice, warps, pred, search, propagate;
@@ -672,11 +674,15 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
       if (ok && p->face_pass == AMR_FACE_PASS_AUTO) ok = face_cells(ctx, g, L, emean, 1.0) <= kAutoFaceCells;
       if (ok) bits |= 1u << L;
     }
+    // the inflated box is the 3^D cells around a cell exactly when d is the cell size on every level
+    const bool unit = P.pred == AMR_PRED_BOX && g.d_abs == 0.0 && g.d_rel == 1.0;
+    if (bits && unit) bits |= kFaceUnit;
     g.face_levels = bits;
     for (int L = 0; L < g.n_levels; ++L) {
-      if ((bits >> L) & 1u)
+      if ((bits >> L) & 1u) {
         P.face_at[L] = true;
-      else
+        (unit ? P.unit_at : P.plain_at)[L] = true;
+      } else
         P.walk_at[L] = true;
     }
     sig = (sig ^ bits) * 1099511628211ull;
@@ -801,9 +807,8 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
       m.rec = static_cast<const FaceRec3*>(ctx->frec.p);
       m.face_gid = ctx->multi ? static_cast<const uint32_t*>(ctx->face_gid.p) : nullptr;
       for (int l = 0; l < L; ++l) m.first_child[l] = static_cast<const int32_t*>(ctx->lv[l].first.p);
-      // faces per work fetch: enough warps to fill the GPU (24 resident per SM)
-      const int64_t warps = (int64_t)ctx->num_sms * 24;
-      m.batch = (int)std::max<int64_t>(1, std::min<int64_t>(kFaceBatch, ctx->nf / (2 * warps)));
+      m.unit = P.unit_at[L];
+      m.plain = P.plain_at[L];
       if (a.blockcnt) CK(cudaMemsetAsync(a.blockcnt, 0, sizeof(uint64_t) * (size_t)(lb.cap > 0 ? lb.cap : 1), st));
       timed(ctx, st, "mark_faces", [&] { return launch_mark_faces(m, ctx->num_sms, st); });
       if (P.walk_at[L]) {

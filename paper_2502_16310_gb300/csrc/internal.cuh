@@ -40,6 +40,8 @@ enum : int {
   CNT_N = 11,
 };
 
+constexpr uint32_t kFaceUnit = 1u << 31;        // flag in GeomParams::face_levels
+
 // Per-geometry parameters.  A launch may cover the blocks (faces) of many
 // geometries; each block (face) then carries its geometry id and reads its
 // row of this table.  Single-geometry launches pass one row by value.
@@ -56,6 +58,7 @@ struct GeomParams {
   int n_levels;
   int root[3];
   uint32_t face_levels;  // bit L: this geometry's mask-only blocks of level L are marked face by face
+                         // (kFaceUnit: d is the cell size, so by widening the cells that a face meets)
   int64_t bin_base;
   int64_t root_base;   // first level-0 block of this geometry in the concatenated list
   int64_t face_base;   // first face of this geometry in the concatenated face arrays
@@ -518,9 +521,10 @@ struct MarkArgs {
   // per level l < lv.level: the first-child index of each block (-1: none), so that a
   // block of this level is found from its root by one step per level
   const int32_t* first_child[kMaxLevels];
-  int batch;            // faces a warp takes per work fetch (1..kFaceBatch)
+  int batch;            // faces a warp takes per work fetch (set by the launcher)
+  bool unit, plain;     // some geometry's faces of the level have kFaceUnit / do not have it
 };
-constexpr int kFaceBatch = 8;  // most faces a warp takes per work fetch
+constexpr int kFaceBatch = 8;  // most faces a warp of the general kernel takes per work fetch
 int launch_mark_faces(const MarkArgs& m, int num_sms, cudaStream_t st);
 
 // The algorithmic cell-face test count of one level (single geometry): per cell

@@ -19,6 +19,9 @@
 // Decisions are exact: each FP32 axis test carries a forward error bound; a
 // (cell, face) pair whose sign is not certified on every axis is re-evaluated
 // in FP64 (and counted).  Block-level culls only use certified separations.
+#include <algorithm>
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace amr {
@@ -194,15 +197,17 @@ struct BlockFrame {
 // Per-face setup (one lane): edges, projections of the face on every axis in
 // the block frame, the cell-level intervals [tmin - r|a|_1, tmax + r|a|_1] and
 // their error bounds.  Returns false when some axis certifiably separates the
-// face from the whole inflated block.
+// face from the whole inflated block.  Without kCull (face-by-face marking, which has no block) the face is
+// kept whatever the block would say; returns 16 u (P + O + r) then, the error bound of a unit axis.
 //
 // Error bound per axis a: every computed projection, interval end and cell
 // coordinate differs from its exact value by at most a few unit roundoffs of
 // (P + O + r) |a|_1, where P bounds the vertex offsets in the frame (this also
 // covers the rounding of the frame origin, of the edges when they are not
 // exact and of the FP32 normal relative to the FP64 one).  eps = 16 u (P+O+r)|a|_1.
-template <int D>
-__device__ __forceinline__ bool setup_face(const float* V, const float* nh, const BlockFrame<D>& F, Surv<D>& S) {
+template <int D, bool kCull = true>
+__device__ __forceinline__ auto setup_face(const float* V, const float* nh, const BlockFrame<D>& F, Surv<D>& S)
+    -> std::conditional_t<kCull, bool, float> {
   float p[3][3];
   float P = 0.f;
 #pragma unroll
@@ -228,6 +233,12 @@ __device__ __forceinline__ bool setup_face(const float* V, const float* nh, cons
       tmax = fmaxf(tmax, s);
     }
     const float eps = scale * A1;
+    if constexpr (!kCull) {
+      const float R = F.r * A1;
+      const float lo = tmin - R, hi = tmax + R;
+      S.t[ai] = make_float4(lo - eps, hi + eps, lo + eps, hi - eps);
+      return true;
+    }
     const float xb = D == 3 ? fmaf(F.cB[2], az, fmaf(F.cB[1], ay, F.cB[0] * ax)) : fmaf(F.cB[1], ay, F.cB[0] * ax);
     const float RB = F.rb * A1;
     // block interval [xb - RB, xb + RB] vs face interval [tmin, tmax]
@@ -265,7 +276,10 @@ __device__ __forceinline__ bool setup_face(const float* V, const float* nh, cons
     S.e[0] = e0;
     S.e[1] = e1;
   }
-  return true;
+  if constexpr (kCull)
+    return true;
+  else
+    return scale;
 }
 
 // Cell tests of the lane's two cells against one survivor: 0 = separated,
@@ -451,6 +465,64 @@ __device__ __noinline__ bool resolve_fp64(const RefineLevel& a, uint32_t gid, ui
   const double m = a.pred == 1 ? point_dist_fp64(V, xc, D) - G.d : margin_fp64_2(V, xc, r);
   if (fabs(m) <= kBandRel * G.h) ++*band;
   return m <= 0.0;
+}
+
+// sat_adjacent_fp64_3 by a whole warp, an axis per lane (the same operations in the same order per axis,
+// so the same decision and band): an FP64 operation takes tens of cycles here, and one pair's 13 axes in
+// a row held its warp for tens of microseconds, which on a small mesh is longer than the rest of a level.
+// Every lane passes the same arguments and gets the decision.
+__device__ __noinline__ bool resolve_sat_warp(const RefineLevel& a, uint32_t gid, uint32_t face, int b0, int b1, int b2,
+                                              int cell_local, bool* band) {
+  const int lane = threadIdx.x & 31;
+  const GeomParams& P = a.table ? a.table[gid] : a.g0;
+  const double h = scalbn(P.h0, -a.level);
+  const double d = __dadd_rn(P.d_abs, __dmul_rn(P.d_rel, h));
+  const double r = __dadd_rn(0.5 * h, d), tol = kBandRel * h;
+  const int b[3] = {b0, b1, b2};
+  double p[3][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double xc = __dadd_rn(P.origin[c], __dmul_rn((double)(4 * b[c] + ((cell_local >> (2 * c)) & 3)) + 0.5, h));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) p[k][c] = __dsub_rn((double)a.X[(int64_t)(3 * k + c) * a.nf + face], xc);
+  }
+  double a0 = lane == 0 ? 1.0 : 0.0, a1 = lane == 1 ? 1.0 : 0.0, a2 = lane == 2 ? 1.0 : 0.0;
+  if (lane == 3) {
+    const double u0 = __dsub_rn(p[1][0], p[0][0]), u1 = __dsub_rn(p[1][1], p[0][1]), u2 = __dsub_rn(p[1][2], p[0][2]);
+    const double w0 = __dsub_rn(p[2][0], p[0][0]), w1 = __dsub_rn(p[2][1], p[0][1]), w2 = __dsub_rn(p[2][2], p[0][2]);
+    a0 = __dsub_rn(__dmul_rn(u1, w2), __dmul_rn(u2, w1));
+    a1 = __dsub_rn(__dmul_rn(u2, w0), __dmul_rn(u0, w2));
+    a2 = __dsub_rn(__dmul_rn(u0, w1), __dmul_rn(u1, w0));
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int k1 = (k + 1) % 3;
+    if (lane >= 4 + 3 * k && lane < 7 + 3 * k) {
+      const double ex = __dsub_rn(p[k1][0], p[k][0]), ey = __dsub_rn(p[k1][1], p[k][1]),
+                   ez = __dsub_rn(p[k1][2], p[k][2]);
+      const int i = lane - 4 - 3 * k;
+      a0 = i == 0 ? 0.0 : (i == 1 ? ez : -ey);
+      a1 = i == 0 ? -ez : (i == 1 ? 0.0 : ex);
+      a2 = i == 0 ? ey : (i == 1 ? -ex : 0.0);
+    }
+  }
+  const double l2sq = __dadd_rn(__dadd_rn(__dmul_rn(a0, a0), __dmul_rn(a1, a1)), __dmul_rn(a2, a2));
+  double lo = 1e300, hi = -1e300;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const double s = __dadd_rn(__dadd_rn(__dmul_rn(p[k][0], a0), __dmul_rn(p[k][1], a1)), __dmul_rn(p[k][2], a2));
+    lo = fmin(lo, s);
+    hi = fmax(hi, s);
+  }
+  const double R = __dmul_rn(r, __dadd_rn(__dadd_rn(fabs(a0), fabs(a1)), fabs(a2)));
+  const double g = fmax(__dsub_rn(lo, R), __dsub_rn(-R, hi));
+  const bool axis = lane < 13 && l2sq != 0.0;
+  const bool small = __dmul_rn(g, g) <= __dmul_rn(tol * tol, l2sq);
+  const unsigned sep = __ballot_sync(0xffffffffu, axis && g > 0.0);
+  const unsigned big = __ballot_sync(0xffffffffu, axis && g > 0.0 && !small);
+  const unsigned near0 = __ballot_sync(0xffffffffu, axis && !(g > 0.0) && small);
+  *band = sep ? big == 0u : near0 != 0u;
+  return sep == 0u;
 }
 
 // Shared walk of one block: bins of the query box, canonical-bin dedup,
@@ -675,6 +747,21 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
             t1 = D == 3 ? point_test<D>(S, o1, R2) : 0;
           } else {
             cell_test2<D>(S, o0, o1, t0, t1);
+          }
+        }
+        if constexpr (D == 3 && !kPoint) {
+          for (uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h0) && t0 == 2) |
+                            ((uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h1) && t1 == 2) << 32);
+               u; u &= u - 1) {
+            const int cell = __ffsll((long long)u) - 1;
+            bool in_band;
+            const int t = resolve_sat_warp(a, gid, S.face, b[0], b[1], b[2], cell, &in_band) ? 1 : 0;
+            if (lane == 0) {
+              ++wc.fb;
+              wc.band += in_band ? 1ull : 0ull;
+            }
+            if (cell == lane) t0 = t;
+            if (cell == lane + 32) t1 = t;
           }
         }
         bool r0 = false, r1 = false;
@@ -927,16 +1014,6 @@ struct GroupCounters {
   uint32_t fb = 0, band = 0, cand = 0, surv = 0, big = 0;
 };
 
-// FP64 decision of one (cell, face) pair of a group (the per-block walk's resolution).
-__device__ __noinline__ bool resolve_group(const RefineLevel& a, uint32_t gid, uint32_t face, const int* b,
-                                           int cell_local, GroupCounters& wc) {
-  unsigned long long fb = 0, band = 0;
-  const bool r = resolve_fp64<3>(a, gid, face, b, cell_local, &fb, &band);
-  wc.fb += (uint32_t)fb;
-  wc.band += (uint32_t)band;
-  return r;
-}
-
 // One parent group: walk, culls and cell tests.  kMark: only the masks are
 // wanted (the walk ends once every cell of the 8 children is marked); else the
 // per-cell counts and the survivor records of the finest level are kept.
@@ -1073,15 +1150,21 @@ __device__ __forceinline__ void walk_group(const RefineLevel& a, const GeomParam
           int t0 = 0, t1 = 0;
           cell_test2<3>(S, o0, o1, t0, t1);
           const int bj[3] = {c0[0] + cx, c0[1] + cy, c0[2] + cz};  // child j's block coordinates
-          bool r0 = false, r1 = false;
-          if (!m0) {
-            if (t0 == 2) t0 = resolve_group(a, gid, S.face, bj, lane, wc) ? 1 : 0;
-            r0 = t0 != 0;
+          // pairs not certified in FP32, one after another by the whole warp
+          for (uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !m0 && t0 == 2) |
+                            ((uint64_t)__ballot_sync(0xffffffffu, !m1 && t1 == 2) << 32);
+               u; u &= u - 1) {
+            const int cell = __ffsll((long long)u) - 1;
+            bool in_band;
+            const int t = resolve_sat_warp(a, gid, S.face, bj[0], bj[1], bj[2], cell, &in_band) ? 1 : 0;
+            if (lane == 0) {
+              ++wc.fb;
+              wc.band += in_band ? 1u : 0u;
+            }
+            if (cell == lane) t0 = t;
+            if (cell == lane + 32) t1 = t;
           }
-          if (!m1) {
-            if (t1 == 2) t1 = resolve_group(a, gid, S.face, bj, lane + 32, wc) ? 1 : 0;
-            r1 = t1 != 0;
-          }
+          const bool r0 = !m0 && t0 != 0, r1 = !m1 && t1 != 0;
           hb0 |= (uint32_t)r0 << j;
           hb1 |= (uint32_t)r1 << j;
           if constexpr (kMark) {
@@ -1717,6 +1800,13 @@ __device__ __forceinline__ int cell_test1(const Surv<D>& S, const float* o) {
   return sep ? 0 : (in ? 1 : 2);
 }
 
+// Table row of a geometry; a single geometry's row is a kernel argument (read in place, not copied).
+template <bool MULTI>
+__device__ __forceinline__ const GeomParams& row(const RefineLevel& a, uint32_t gid) {
+  if constexpr (MULTI) return a.table[gid];
+  return a.g0;
+}
+
 // setup_face without the block cull, lane-parallel: lane ai < 13 (2D: 3)
 // computes axis ai with setup_face's arithmetic; lane 0 stores the edges.
 template <int D>
@@ -1817,7 +1907,7 @@ __device__ __forceinline__ void setup_face_lanes(const float* V, const float* nh
 constexpr int kMarkWarps = 4;  // warps per CTA of k_mark_faces
 constexpr int kMarkSlots = 64;  // blocks of a face's range looked up once per face (more: per cell)
 
-template <int D, int PRED>
+template <int D, int PRED, bool MULTI>
 __global__ void __launch_bounds__(kMarkWarps * 32, 6) k_mark_faces(MarkArgs m) {
   const RefineLevel& a = m.lv;
   __shared__ Surv<D> s_surv[kMarkWarps];
@@ -1843,9 +1933,9 @@ __global__ void __launch_bounds__(kMarkWarps * 32, 6) k_mark_faces(MarkArgs m) {
       if (f >= a.nf) break;
       // the face's geometry: only geometries marked face by face on this level (their blocks of the
       // level have the mask as the only output; the walk does the others)
-      const uint32_t gid = a.table ? __ldg(m.face_gid + f) : 0u;
-      const GeomParams& P = a.table ? a.table[gid] : a.g0;
-      if (!((P.face_levels >> a.level) & 1u)) continue;
+      const uint32_t gid = MULTI ? __ldg(m.face_gid + f) : 0u;
+      const GeomParams& P = row<MULTI>(a, gid);
+      if (!((P.face_levels >> a.level) & 1u) || (P.face_levels & kFaceUnit)) continue;
       const FastGeom g = fast_geom(P, a.level);
       const float hf = g.h_hi;
       const float inv_h = 1.0f / hf;
@@ -2004,6 +2094,416 @@ __global__ void __launch_bounds__(kMarkWarps * 32, 6) k_mark_faces(MarkArgs m) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same marking where d is the cell size itself (d_abs = 0, d_rel = 1, the
+// default) and the predicate the box one.  A cell's inflated box is then the
+// 3^D block of cells around it, so a face meets it exactly when the face meets
+// one of those cells: a face is tested against the few cells that its own AABB
+// reaches (r = h / 2), and the cells it meets are widened by one cell with bit
+// operations on the block masks.  On the largest workload that leaves 16 cells
+// per face and level to test instead of 84.
+//
+// The decisions stay those of the definition.  A certified overlap with a cell
+// is far beyond FP64's rounding, so the inflated boxes of its neighbours meet
+// the face; a face certified apart from all 3^D cells of an inflated box has a
+// distance from it that FP64 sees.  Where the test of a cell is not certified,
+// its 3^D neighbours are tested with their own inflated boxes, as everywhere
+// else (FP32, then FP64).  Cells of one layer outside the domain are tested as
+// well, for they widen into it.  A cell that a face meets lies in a block of
+// the level: the cell above it was marked.
+//
+// A warp takes up to kCellFaces faces in four steps: a lane per face (cell range,
+// axis thresholds), a lane per block of the ranges (index), a lane per cell, a
+// lane per block again (widening, then one atomic for its new marks), each packed
+// over all the faces.  Bound by instructions and the latency of the block
+// lookups.  Against a warp per face testing every inflated cell (k_mark_faces):
+// the five levels of 1.3 M faces 10.6 -> 2.36 ms, the four of 82 K 0.76 -> 0.29,
+// the three of 20 K 0.22 -> 0.13 (the uncertified cells' tests by one lane in a
+// row: 4.5, 1.0 and 0.53 ms).
+// ---------------------------------------------------------------------------
+template <int D>
+struct MarkFace {
+  float shift[3];              // frame corner's rounding error
+  float h_hi, h_lo;
+  float inv_n0, inv_n1, inv_b0, inv_b1;
+  int lo[3], blo[3];           // first cell of the range, first block of the widened range
+  int n0, n1, nb0, nb1, nb2;   // cells and blocks per axis
+  int total, nslot;
+  uint32_t slot, face, gid;    // first slot of the range's blocks
+};
+
+constexpr int kCellWarps = 4;    // warps per CTA of k_mark_cells
+constexpr int kCellBlocks = 5;   // CTAs per SM (shared memory)
+constexpr int kCellFaces = 16;   // faces a warp takes per work fetch
+constexpr int kCellPool = 160;   // blocks of the ranges of a group of faces
+
+template <int D>
+struct CellSmem {
+  Surv<D> surv[kCellFaces];
+  MarkFace<D> f[kCellFaces];
+  alignas(8) uint32_t met[kCellPool][2];    // per block: its cells that the face meets, then widened
+  uint64_t tmp[kCellPool];
+  uint32_t more[kCellPool][2];   // cells marked by their own test
+  int32_t bi[kCellPool];         // the block's index (-1: absent)
+  uint8_t own[kCellPool];        // its face
+};
+
+// Owner of item k0 + lane among items numbered through consecutive ranges: lanes [g0, g1) (own) hold
+// their ranges' first items; returns the owner's lane.
+__device__ __forceinline__ int range_owner(uint32_t first, bool own, int g0, uint32_t k0, int lane) {
+  const unsigned before = __popc(__ballot_sync(0xffffffffu, own && first < k0));
+  const unsigned heads = __reduce_or_sync(0xffffffffu, own && first - k0 < 32u ? 1u << (first - k0) : 0u);
+  return g0 + (int)(before + __popc(heads & (0xffffffffu >> (31 - lane)))) - 1;
+}
+
+// cell_test1 for the cell's box widened by grow: the thresholds move by grow |a|_1, and the
+// certificates by the rounding of that.
+template <int D>
+__device__ __noinline__ int cell_test_grown(const Surv<D>& S, const float* o, float grow) {
+  bool sep = false, in = true;
+  auto upd = [&](float x, float A1, const float4& t) {
+    const float g = grow * A1, e = kEpsK * kU32 * g;
+    sep |= (x < (t.x - g) - e) | (x > (t.y + g) + e);
+    in &= (x > (t.z - g) + e) & (x < (t.w + g) - e);
+  };
+  if constexpr (D == 3) {
+#pragma unroll
+    for (int ai = 0; ai < 3; ++ai) upd(o[ai], 1.f, S.t[ai]);
+    const float4 q0 = S.en[0], q1 = S.en[1], q2 = S.en[2];
+    const float e[3][3] = {{q0.x, q0.y, q0.z}, {q0.w, q1.x, q1.y}, {q1.z, q1.w, q2.x}};
+    upd(fmaf(o[2], q2.w, fmaf(o[1], q2.z, o[0] * q2.y)), fabsf(q2.y) + fabsf(q2.z) + fabsf(q2.w), S.t[3]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float ex = e[k][0], ey = e[k][1], ez = e[k][2];
+      upd(fmaf(o[2], ey, -o[1] * ez), fabsf(ey) + fabsf(ez), S.t[4 + 3 * k]);
+      upd(fmaf(o[0], ez, -o[2] * ex), fabsf(ex) + fabsf(ez), S.t[5 + 3 * k]);
+      upd(fmaf(o[1], ex, -o[0] * ey), fabsf(ex) + fabsf(ey), S.t[6 + 3 * k]);
+    }
+  } else {
+    upd(o[0], 1.f, S.t[0]);
+    upd(o[1], 1.f, S.t[1]);
+    upd(fmaf(o[1], S.e[0], -o[0] * S.e[1]), fabsf(S.e[0]) + fabsf(S.e[1]), S.t[2]);
+  }
+  return sep ? 0 : (in ? 1 : 2);
+}
+
+// A block mask widened by one cell along axis AX: its own cells, and the neighbours' facing layers
+// (prev / next: the masks of the blocks before and after it on that axis).
+template <int AX>
+__device__ __forceinline__ uint64_t widen(uint64_t m, uint64_t prev, uint64_t next) {
+  constexpr int s = 2 * AX == 0 ? 1 : (AX == 1 ? 4 : 16);
+  constexpr uint64_t first = AX == 0 ? 0x1111111111111111ull : (AX == 1 ? 0x000f000f000f000full : 0xffffull);
+  constexpr uint64_t last = first << (3 * s);
+  return m | ((m << s) & ~first) | ((m >> s) & ~last) | ((prev >> (3 * s)) & first) | ((next << (3 * s)) & last);
+}
+
+template <int D, bool MULTI>
+__global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(MarkArgs m) {
+  const RefineLevel& a = m.lv;
+  __shared__ __align__(16) CellSmem<D> s_all[kCellWarps];
+  const int lane = threadIdx.x & 31;
+  CellSmem<D>& sm = s_all[threadIdx.x >> 5];
+  const int64_t nblk = launch_count(a.n_blocks, a.n_dev, a.err);
+  const int batch = m.batch > 0 ? (m.batch < kCellFaces ? m.batch : kCellFaces) : 1;
+  // k = a + n b (0 <= a < n, k < 2^20): b = floor((k + 1/2) / n), exactly, from an FP32
+  // reciprocal (the quotient is at least 1/(2n) from an integer; the error is below 2^-21 k / n)
+  auto divn = [](int k, float inv) { return (int)(((float)k + 0.5f) * inv); };
+  // index of the level's block with coordinates b, or -1 when the level does not have it: its
+  // root by the root order, then per level the ancestor's first child plus the slot (the
+  // coordinates' bit of that level per axis); the upper levels' arrays stay in cache
+  auto find = [&](uint32_t g, const int* b) -> int32_t {
+    const GeomParams& Q = row<MULTI>(a, g);
+    const int L = a.level;
+#pragma unroll
+    for (int c = 0; c < D; ++c)
+      if (b[c] < 0 || b[c] >= (Q.root[c] << L)) return -1;
+    int64_t i = Q.root_base + (b[0] >> L) + (int64_t)Q.root[0] * ((b[1] >> L) + (int64_t)Q.root[1] * (b[2] >> L));
+    for (int l = 1; l <= L && i >= 0; ++l) {
+      const int sh = L - l;
+      const int slot = ((b[0] >> sh) & 1) | (((b[1] >> sh) & 1) << 1) | (D == 3 ? ((b[2] >> sh) & 1) << 2 : 0);
+      const int32_t c = __ldg(m.first_child[l - 1] + i);
+      i = c >= 0 ? (int64_t)c + slot : -1;
+    }
+    return i < nblk ? (int32_t)i : -1;
+  };
+  WarpCounters wc;
+  unsigned long long n_tests = 0;
+  for (;;) {
+    unsigned base = 0;
+    if (lane == 0) base = atomicAdd(a.work, (unsigned)batch);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if ((int64_t)base >= a.nf) break;
+    // a lane per face: its cell range and thresholds
+    const int64_t f = (int64_t)base + lane;
+    bool use = lane < batch && f < a.nf;
+    const uint32_t gid = MULTI && use ? __ldg(m.face_gid + f) : 0u;
+    const GeomParams& P = row<MULTI>(a, gid);
+    use = use && ((P.face_levels >> a.level) & 1u) && (P.face_levels & kFaceUnit);
+    MarkFace<D> M;
+    BlockFrame<D> F;
+    float V[D * D], nh[3] = {0.f, 0.f, 0.f};
+    if (use) {
+      const FastGeom g = fast_geom(P, a.level);
+      const float hf = g.h_hi, inv_h = 1.0f / hf;
+      if constexpr (D == 3) {
+        const float4* R = reinterpret_cast<const float4*>(m.rec + f);
+        const float4 r0 = __ldg(R), r1 = __ldg(R + 1), r2 = __ldg(R + 2);
+        V[0] = r0.x; V[1] = r0.y; V[2] = r0.z; V[3] = r0.w; V[4] = r1.x;
+        V[5] = r1.y; V[6] = r1.z; V[7] = r1.w; V[8] = r2.x;
+        nh[0] = r2.y; nh[1] = r2.z; nh[2] = r2.w;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) V[j] = __ldg(a.X + (int64_t)j * a.nf + f);
+      }
+      // cells that can meet the face's AABB (a superset: the margin covers the FP32 error of the
+      // cell coordinate), down to one layer outside the domain; the blocks of that range widened
+      int n[3] = {1, 1, 1}, nb[3] = {1, 1, 1};
+      float O = 0.f;
+      M.lo[2] = M.blo[2] = 0;
+      M.shift[2] = 0.f;
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        const int ncell = (4 * P.root[c]) << a.level;
+        float vmin = V[c], vmax = V[c];
+#pragma unroll
+        for (int k = 1; k < D; ++k) {
+          vmin = fminf(vmin, V[D * k + c]);
+          vmax = fmaxf(vmax, V[D * k + c]);
+        }
+        const float margin = 1e-3f + 16.0f * kU32 * (fmaxf(fabsf(vmin), fabsf(vmax)) + fabsf(P.org_hi[c])) * inv_h;
+        const float xl = (vmin - P.org_hi[c]) * inv_h, xh = (vmax - P.org_hi[c]) * inv_h;
+        if (!(xl <= xh)) use = false;  // also a non-finite coordinate
+        const float tl = floorf(xl - margin), th = floorf(xh + margin);
+        const int il = tl < -1.f ? -1 : (tl > (float)ncell ? ncell + 1 : (int)tl);
+        const int ih = th < -1.f ? -2 : (th > (float)ncell ? ncell : (int)th);
+        if (ih < il) use = false;
+        M.lo[c] = il;
+        n[c] = ih - il + 1;
+        M.blo[c] = (il - 1) >> 2;
+        nb[c] = ((ih + 1) >> 2) - M.blo[c] + 1;
+        float flo;
+        df_position(P.org_hi[c], P.org_lo[c], (float)il, g.h_hi, g.h_lo, F.Xb[c], flo);
+        M.shift[c] = flo;
+        F.cB[c] = 0.f;
+        // the frame holds the range and the neighbours of its cells
+        O = fmaxf(O, (float)(n[c] + 2) * hf + 2.0f * fabsf(flo));
+      }
+      F.h = hf;
+      F.r = 0.5f * hf;
+      F.rb = 0.f;
+      F.O = O;
+      // the host keeps every range below 2^15 cells (largest face of the binning); a
+      // larger one here means inconsistent inputs: reported, not tested
+      const int64_t wide = (int64_t)(n[0] + 2) * (n[1] + 2) * (D == 3 ? n[2] + 2 : 1);
+      if (use && wide > (1 << 20)) {
+        atomicOr(a.err, ERR_OVERFLOW);
+        use = false;
+      }
+      const int nslot = nb[0] * nb[1] * nb[2];
+      if (nslot > kMarkSlots) {  // too many blocks: every cell of the widened range by its own test
+#pragma unroll
+        for (int c = 0; c < D; ++c) {
+          n[c] += 2;
+          M.lo[c] -= 1;
+        }
+      }
+      M.total = n[0] * n[1] * n[2];
+      M.nslot = nslot;
+      M.n0 = n[0], M.n1 = n[1], M.nb0 = nb[0], M.nb1 = nb[1], M.nb2 = nb[2];
+      M.inv_n0 = 1.0f / (float)n[0], M.inv_n1 = 1.0f / (float)n[1];
+      M.inv_b0 = 1.0f / (float)nb[0], M.inv_b1 = 1.0f / (float)nb[1];
+      M.h_hi = g.h_hi, M.h_lo = g.h_lo;
+      M.slot = 0u, M.face = (uint32_t)f, M.gid = gid;
+    }
+    const unsigned valid = __ballot_sync(0xffffffffu, use);
+    const int nv = __popc(valid);
+    if (use) {
+      wc.cand++;
+      const int i = __popc(valid & ((1u << lane) - 1u));
+      setup_face<D, false>(V, nh, F, sm.surv[i]);
+      sm.f[i] = M;
+    }
+    __syncwarp();
+    const int my_total = lane < nv ? sm.f[lane].total : 0;
+    const int my_slots = lane < nv ? sm.f[lane].nslot : 0;
+    for (int g0 = 0; g0 < nv;) {
+      // a run of faces whose blocks fit the slots, or one face with too many blocks
+      const bool slots = sm.f[g0].nslot <= kMarkSlots;
+      const uint32_t ns = lane >= g0 && lane < nv ? (my_slots <= kMarkSlots ? my_slots : kCellPool + 1) : 0u;
+      const uint32_t sincl = warp_inclusive_scan<uint32_t>(ns);
+      const int g1 = slots ? g0 + __popc(__ballot_sync(0xffffffffu, ns && sincl <= (uint32_t)kCellPool)) : g0 + 1;
+      const bool own = lane >= g0 && lane < g1;
+      const uint32_t nsl = slots ? __shfl_sync(0xffffffffu, sincl, g1 - 1) : 0u;
+      const uint32_t sfirst = sincl - ns;
+      if (own) sm.f[lane].slot = sfirst;
+      __syncwarp();
+      for (uint32_t k0 = 0; k0 < nsl; k0 += 32) {
+        const int j = range_owner(sfirst, own, g0, k0, lane);
+        const uint32_t s = k0 + lane;
+        if (s < nsl) {
+          const MarkFace<D>& Q = sm.f[j];
+          const int k = (int)(s - Q.slot);
+          const int k1 = divn(k, Q.inv_b0), k2 = divn(k1, Q.inv_b1);
+          const int b[3] = {Q.blo[0] + k - k1 * Q.nb0, Q.blo[1] + k1 - k2 * Q.nb1, Q.blo[2] + k2};
+          sm.bi[s] = find(Q.gid, b);
+          sm.own[s] = (uint8_t)j;
+          sm.met[s][0] = sm.met[s][1] = 0u;
+          sm.more[s][0] = sm.more[s][1] = 0u;
+        }
+      }
+      __syncwarp();
+      // cell x of face j by its own inflated box: FP32, then FP64
+      auto inflated = [&](const MarkFace<D>& Q, int j, const int* x, const float* o) -> bool {
+        const int t = cell_test_grown<D>(sm.surv[j], o, Q.h_hi);
+        if (t != 2) return t != 0;
+        const int b[3] = {x[0] >> 2, x[1] >> 2, x[2] >> 2};
+        const int local = (x[0] & 3) | ((x[1] & 3) << 2) | (D == 3 ? (x[2] & 3) << 4 : 0);
+        return resolve_fp64<D>(a, Q.gid, Q.face, b, local, &wc.fb, &wc.band);
+      };
+      const uint32_t nc = own ? (uint32_t)my_total : 0u;
+      const uint32_t cincl = warp_inclusive_scan<uint32_t>(nc);
+      const uint32_t cfirst = cincl - nc, ncell = __shfl_sync(0xffffffffu, cincl, 31);
+      // cell (i + dd) of face j's range: its coordinates and its centre in the face's frame, whose corner
+      // is the range's first cell (one further in where the range was widened)
+      auto centre = [&](const MarkFace<D>& Q, const int* i, int d0, int d1, int d2, int* x, float* o) {
+        const int dd[3] = {d0, d1, d2};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          x[q] = Q.lo[q] + i[q] + dd[q];
+          const float l = (float)(i[q] + dd[q] - (slots ? 0 : 1)) + 0.5f;
+          o[q] = q < D ? fmaf(l, Q.h_hi, fmaf(l, Q.h_lo, Q.shift[q])) : 0.f;
+        }
+      };
+      auto cell_of = [&](const MarkFace<D>& Q, int idx, int* i) {
+        const int j1 = divn(idx, Q.inv_n0), j2 = D == 3 ? divn(j1, Q.inv_n1) : 0;
+        i[0] = idx - j1 * Q.n0;
+        i[1] = D == 3 ? j1 - j2 * Q.n1 : j1;
+        i[2] = j2;
+      };
+      auto local_of = [](const int* x) { return (x[0] & 3) | ((x[1] & 3) << 2) | (D == 3 ? (x[2] & 3) << 4 : 0); };
+      auto slot_of = [](const MarkFace<D>& Q, const int* x) {
+        return Q.slot + (uint32_t)(((x[0] >> 2) - Q.blo[0]) +
+                                   Q.nb0 * (((x[1] >> 2) - Q.blo[1]) + Q.nb1 * ((x[2] >> 2) - Q.blo[2])));
+      };
+      for (uint32_t k0 = 0; k0 < ncell; k0 += 32) {
+        const int j = range_owner(cfirst, own, g0, k0, lane);
+        const int idx = (int)(k0 + lane - __shfl_sync(0xffffffffu, cfirst, j));
+        bool unsure = false;
+        if (k0 + lane < ncell) {
+          const MarkFace<D>& Q = sm.f[j];
+          int i[3], x[3];
+          float o[3];
+          cell_of(Q, idx, i);
+          centre(Q, i, 0, 0, 0, x, o);
+          ++n_tests;
+          if (slots) {
+            const int t = cell_test1<D>(sm.surv[j], o);
+            if (t == 1) atomicOr(&sm.met[slot_of(Q, x)][local_of(x) >> 5], 1u << (local_of(x) & 31));
+            unsure = t == 2;
+          } else {
+            const int b[3] = {x[0] >> 2, x[1] >> 2, x[2] >> 2};
+            const int32_t bi = find(Q.gid, b);
+            if (bi >= 0 && !((a.mask[bi] >> local_of(x)) & 1ull) && inflated(Q, j, x, o)) {
+              atomicOr(reinterpret_cast<unsigned long long*>(a.mask + bi), 1ull << local_of(x));
+              a.flag[bi] = 1;
+            }
+          }
+        }
+        // a cell whose test is not certified: its neighbours by their own inflated boxes, a lane each
+        // (FP64 takes thousands of cycles: in parallel, and not for cells that are marked already)
+        for (unsigned ub = __ballot_sync(0xffffffffu, unsure); ub; ub &= ub - 1) {
+          const int src = __ffs(ub) - 1;
+          const int ju = __shfl_sync(0xffffffffu, j, src), iu = __shfl_sync(0xffffffffu, idx, src);
+          int t = 0, x[3] = {0, 0, 0};
+          if (lane < (D == 3 ? 27 : 9)) {
+            const MarkFace<D>& Q = sm.f[ju];
+            int i[3];
+            float o[3];
+            cell_of(Q, iu, i);
+            centre(Q, i, lane % 3 - 1, lane / 3 % 3 - 1, D == 3 ? lane / 9 - 1 : 0, x, o);
+            const uint32_t s = slot_of(Q, x);
+            const int32_t bi = sm.bi[s];
+            if (bi >= 0) {
+              const uint64_t now = __ldcg(reinterpret_cast<const unsigned long long*>(a.mask + bi));
+              if (!((now >> local_of(x)) & 1ull)) t = cell_test_grown<D>(sm.surv[ju], o, Q.h_hi);
+            }
+            if (D == 2 && t == 2) {
+              const int b[3] = {x[0] >> 2, x[1] >> 2, 0};
+              t = resolve_fp64<D>(a, Q.gid, Q.face, b, local_of(x), &wc.fb, &wc.band) ? 1 : 0;
+            }
+            if (t == 1) atomicOr(&sm.more[s][local_of(x) >> 5], 1u << (local_of(x) & 31));
+          }
+          if constexpr (D == 3) {
+            for (unsigned vb = __ballot_sync(0xffffffffu, t == 2); vb; vb &= vb - 1) {
+              const int e = __ffs(vb) - 1;
+              const MarkFace<D>& Q = sm.f[ju];
+              int y[3];
+#pragma unroll
+              for (int q = 0; q < 3; ++q) y[q] = __shfl_sync(0xffffffffu, x[q], e);
+              bool in_band;
+              const bool adj = resolve_sat_warp(a, Q.gid, Q.face, y[0] >> 2, y[1] >> 2, y[2] >> 2, local_of(y), &in_band);
+              if (lane == 0) {
+                ++wc.fb;
+                wc.band += in_band ? 1ull : 0ull;
+                if (adj) atomicOr(&sm.more[slot_of(Q, y)][local_of(y) >> 5], 1u << (local_of(y) & 31));
+              }
+            }
+          }
+          __syncwarp();
+        }
+      }
+      __syncwarp();
+      // widen along each axis, a lane per block (met -> tmp -> met -> tmp)
+      uint64_t* met = reinterpret_cast<uint64_t*>(&sm.met[0][0]);
+      auto pass = [&](auto ax, const uint64_t* in, auto put) {
+        constexpr int AX = decltype(ax)::value;
+        for (uint32_t s = lane; s < nsl; s += 32) {
+          const MarkFace<D>& Q = sm.f[sm.own[s]];
+          const int k = (int)(s - Q.slot), k1 = divn(k, Q.inv_b0), k2 = divn(k1, Q.inv_b1);
+          const int at = AX == 0 ? k - k1 * Q.nb0 : (AX == 1 ? k1 - k2 * Q.nb1 : k2);
+          const int n = AX == 0 ? Q.nb0 : (AX == 1 ? Q.nb1 : Q.nb2);
+          const int step = AX == 0 ? 1 : (AX == 1 ? Q.nb0 : Q.nb0 * Q.nb1);
+          put(s, widen<AX>(in[s], at > 0 ? in[s - step] : 0ull, at + 1 < n ? in[s + step] : 0ull));
+        }
+        __syncwarp();
+      };
+      // the last pass sends a block's new marks with one atomic
+      auto send = [&](uint32_t s, uint64_t w) {
+        const int32_t bi = sm.bi[s];
+        const uint64_t all = (w | sm.more[s][0] | ((uint64_t)sm.more[s][1] << 32)) & (D == 3 ? ~0ull : 0xffffull);
+        if (bi >= 0 && all) {
+          const uint64_t now = __ldcg(reinterpret_cast<const unsigned long long*>(a.mask + bi));
+          if (all & ~now) {
+            atomicOr(reinterpret_cast<unsigned long long*>(a.mask + bi), (unsigned long long)all);
+            if (now == 0) a.flag[bi] = 1;
+          }
+        }
+      };
+      pass(std::integral_constant<int, 0>{}, met, [&](uint32_t s, uint64_t w) { sm.tmp[s] = w; });
+      if constexpr (D == 3) {
+        pass(std::integral_constant<int, 1>{}, sm.tmp, [&](uint32_t s, uint64_t w) { met[s] = w; });
+        pass(std::integral_constant<int, 2>{}, met, send);
+      } else {
+        pass(std::integral_constant<int, 1>{}, sm.tmp, send);
+      }
+      g0 = g1;
+    }
+    __syncwarp();  // the next faces reuse the records
+  }
+  unsigned long long v[4] = {wc.fb, wc.band, wc.cand, n_tests};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+  }
+  if (lane == 0) {
+    if (v[0]) atomicAdd(&a.counters[CNT_FALLBACK], v[0]);
+    if (v[1]) atomicAdd(&a.counters[CNT_BAND], v[1]);
+    if (v[2]) atomicAdd(&a.counters[CNT_FACE_SETUPS], v[2]);
+    if (v[3]) atomicAdd(&a.counters[CNT_FACE_TESTS], v[3]);
+  }
+}
+
 // Warps per SM kept resident: 32 (CTAs of `warps` warps).
 int grid_warps(int num_sms, int64_t n, int warps, bool persistent) {
   const int64_t cap = (int64_t)num_sms * (32 / warps > 0 ? 32 / warps : 1);
@@ -2080,21 +2580,36 @@ int launch_adjacency(const EmitArgs& a, int num_sms, cudaStream_t st) {
 
 int launch_mark_faces(const MarkArgs& m, int num_sms, cudaStream_t st) {
   if (m.lv.nf <= 0) return 0;
-  constexpr int kWarps = kMarkWarps;
-  const int batch = m.batch > 0 ? m.batch : kFaceBatch;
-  int64_t need = (m.lv.nf + batch - 1) / batch;  // warps with work
-  int64_t g = (need + kWarps - 1) / kWarps;
-  const int64_t cap = (int64_t)num_sms * (32 / kWarps);
-  if (g > cap) g = cap;
-  if (g < 1) g = 1;
-  const int mode = m.lv.pred == 1 ? 1 : 0;
-  if (m.lv.dim == 3)
-    mode == 1 ? k_mark_faces<3, 1><<<(unsigned)g, kWarps * 32, 0, st>>>(m)
-              : k_mark_faces<3, 0><<<(unsigned)g, kWarps * 32, 0, st>>>(m);
-  else
-    mode == 1 ? k_mark_faces<2, 1><<<(unsigned)g, kWarps * 32, 0, st>>>(m)
-              : k_mark_faces<2, 0><<<(unsigned)g, kWarps * 32, 0, st>>>(m);
-  return 1;
+  const bool point = m.lv.pred == 1, multi = m.lv.table != nullptr;
+  int k = 0;
+  // `per` faces at most per fetch, fewer where that would leave warps without work
+  auto go = [&](auto kernel, int per, int64_t fetches, int64_t resident, int warps) {
+    MarkArgs x = m;
+    x.batch = (int)std::max<int64_t>(1, std::min<int64_t>(per, m.lv.nf / fetches));
+    const int64_t need = (m.lv.nf + (int64_t)x.batch * warps - 1) / ((int64_t)x.batch * warps);
+    if (k++) cudaMemsetAsync(m.lv.work, 0, sizeof(unsigned), st);
+    kernel<<<(unsigned)std::min<int64_t>(need, resident), warps * 32, 0, st>>>(x);
+  };
+  auto cells = [&](auto kernel) {
+    const int64_t grid = (int64_t)num_sms * kCellBlocks;
+    go(kernel, kCellFaces, grid * kCellWarps, grid, kCellWarps);
+  };
+  auto faces = [&](auto kernel) { go(kernel, kFaceBatch, (int64_t)num_sms * 48, (int64_t)num_sms * 8, kMarkWarps); };
+  if (m.unit) {
+    if (m.lv.dim == 3)
+      multi ? cells(k_mark_cells<3, true>) : cells(k_mark_cells<3, false>);
+    else
+      multi ? cells(k_mark_cells<2, true>) : cells(k_mark_cells<2, false>);
+  }
+  if (m.plain) {
+    if (m.lv.dim == 3)
+      point ? (multi ? faces(k_mark_faces<3, 1, true>) : faces(k_mark_faces<3, 1, false>))
+            : (multi ? faces(k_mark_faces<3, 0, true>) : faces(k_mark_faces<3, 0, false>));
+    else
+      point ? (multi ? faces(k_mark_faces<2, 1, true>) : faces(k_mark_faces<2, 1, false>))
+            : (multi ? faces(k_mark_faces<2, 0, true>) : faces(k_mark_faces<2, 0, false>));
+  }
+  return k;
 }
 
 size_t children_scratch_bytes(int64_t n) {
