@@ -48,6 +48,7 @@ struct TimingSlot {
 
 struct LevelBufs {
   DevBuf blocks, gid, parent, mask, flag, cellcnt, blockcnt, base, desc;
+  DevBuf info, rfirst;    // records left by the faces: per block its records and pairs, its first record
   DevBuf first;           // per block: index of its first child in the next level, -1 without children
   DevBuf prev, n2o, o2n;  // previous call's blocks (kept on request) and the re-adaptation maps
   int64_t n_prev = 0;
@@ -60,6 +61,7 @@ constexpr int SC_TOT = 16;   // [16] adjacency totals per level (pairs | cells <
 constexpr int SC_NL = 32;    // [16] links per level
 constexpr int SC_RUN = 48;   // [3] running cells, pairs, links
 constexpr int SC_REC = 52;   // [16] survivor records handed out per level
+constexpr int SC_RTOT = 68;    // records placed (the record scan's total)
 constexpr int SC_WORDS = 72;
 
 // A captured graph stays valid while no buffer it uses was reallocated
@@ -104,7 +106,7 @@ struct amr_ctx {
   bool multi = false;
   DevBuf table, face_gid;
   // buffers
-  DevBuf X, nrm, frec, recs, hkeys, hvals, mkeys, mvals, cls, flbase, tl_cell, tl_dir, tl_q, tl_face, stage_a, stage_b, frange, count, offsets, ids, payload, scratch, misc, scal;
+  DevBuf X, nrm, frec, recs, staged, hkeys, hvals, mkeys, mvals, cls, flbase, tl_cell, tl_dir, tl_q, tl_face, stage_a, stage_b, frange, count, offsets, ids, payload, scratch, misc, scal;
   LevelBufs lv[AMR_MAX_LEVELS];
   DevBuf adj_cell, adj_off, adj_ids, link_cell, link_dir, link_q, link_face, link_stage;
   int64_t cap_cells = 0, cap_pairs = 0, cap_links = 0;
@@ -348,6 +350,20 @@ amr_status read_scalar(amr_ctx* ctx, cudaStream_t st, int slot, uint64_t* v, uns
   return AMR_OK;
 }
 
+// Two of them.
+amr_status read_scalars(amr_ctx* ctx, cudaStream_t st, int slot0, uint64_t* v0, int slot1, uint64_t* v1,
+                        unsigned* err_out) {
+  char* h = static_cast<char*>(ctx->h_pinned);
+  TRY(small_copy(ctx, st, {{ctx->h_dev + 128, ctx->d_scal + slot0, sizeof(uint64_t)},
+                      {ctx->h_dev + 136, ctx->d_scal + slot1, sizeof(uint64_t)},
+                      {ctx->h_dev + 64, ctx->d_err, sizeof(unsigned)}}));
+  TRY(sync_check(ctx, st));
+  *v0 = *reinterpret_cast<uint64_t*>(h + 128);
+  *v1 = *reinterpret_cast<uint64_t*>(h + 136);
+  *err_out = *reinterpret_cast<unsigned*>(h + 64);
+  return AMR_OK;
+}
+
 amr_status device_error(amr_ctx* ctx, unsigned e) {
   if (!e) return AMR_OK;
   // clear it so the context stays usable after the report
@@ -472,7 +488,7 @@ amr_status amr_ctx_init(amr_ctx* ctx) {
 void amr_ctx_free(amr_ctx* ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   drop_graph(ctx);
-  DevBuf* all[] = {&ctx->X, &ctx->frec, &ctx->recs, &ctx->hkeys, &ctx->hvals, &ctx->mkeys, &ctx->mvals, &ctx->cls, &ctx->flbase,
+  DevBuf* all[] = {&ctx->X, &ctx->frec, &ctx->recs, &ctx->staged, &ctx->hkeys, &ctx->hvals, &ctx->mkeys, &ctx->mvals, &ctx->cls, &ctx->flbase,
                    &ctx->tl_cell, &ctx->tl_dir, &ctx->tl_q, &ctx->tl_face, &ctx->nrm,          &ctx->stage_a,    &ctx->stage_b,    &ctx->frange,
                    &ctx->count,     &ctx->offsets,      &ctx->ids,        &ctx->payload,    &ctx->scratch,
                    &ctx->misc,      &ctx->scal,         &ctx->adj_cell,   &ctx->adj_off,    &ctx->adj_ids,
@@ -484,7 +500,8 @@ void amr_ctx_free(amr_ctx* ctx) {
   for (int L = 0; L < AMR_MAX_LEVELS; ++L) {
     LevelBufs& l = ctx->lv[L];
     DevBuf* lb[] = {&l.blocks, &l.gid,  &l.parent, &l.mask, &l.flag, &l.cellcnt,
-                    &l.blockcnt, &l.base, &l.desc,   &l.prev, &l.n2o,  &l.o2n, &l.first};
+                    &l.blockcnt, &l.base, &l.desc,   &l.prev, &l.n2o,  &l.o2n, &l.first,
+                    &l.info,     &l.rfirst};
     for (DevBuf* b : lb) release(ctx, *b);
   }
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
@@ -616,6 +633,7 @@ struct Plan {
   bool face_at[AMR_MAX_LEVELS];     // some geometry's blocks of the level are marked face by face
   bool unit_at[AMR_MAX_LEVELS];     // ... with d the cell size (kFaceUnit)
   bool plain_at[AMR_MAX_LEVELS];    // ... with another d or predicate
+  bool rec_at[AMR_MAX_LEVELS];      // the faces leave the records of every geometry that ends at the level
   bool walk_at[AMR_MAX_LEVELS];     // some geometry's blocks of the level are walked
   bool adjacency, links;
   int lattice, warps, pred, search, propagate;
@@ -630,6 +648,12 @@ constexpr double kMaxFaceCells = 32768.0;
 // Automatic choice: face by face where the geometry's mean face covers at most
 // this many cells of the level (the block walk is cheaper once faces span many cells).
 constexpr double kAutoFaceCells = 1024.0;
+// The same in 3D where d is the cell size, for mask-only levels and for the records of a last level
+// (k_mark_cells: a face of 17 cells across takes as long as the walk; measured on 32^3 roots, 4 levels,
+// last level by faces / by the walk: 2.2 cells 1.06 / 1.94 ms for the refinement, 8.6 cells 0.48 / 0.61,
+// 13.8 cells 0.41 / 0.51, 19.6 cells 0.54 / 0.52).  In 2D the walk of the last level is never dearer than
+// the records' launches (0.33 / 0.35 ms for 20,000 edges).
+constexpr double kAutoUnitCells = 8192.0;
 
 // Cells of level L in the range of a face of geometry g whose largest AABB side
 // is ext root cells: (ext 2^L + 2 d_L / h_L + pad) per axis (pad 4 bounds the
@@ -663,19 +687,31 @@ Plan make_plan(const amr_ctx* ctx, const amr_refine_params* p) {
 // which of the two launches a level needs.  Returns a signature of the choice.
 uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
   uint64_t sig = 1469598103934665603ull;
+  auto unit_of = [&](const GeomParams& g) { return P.pred == AMR_PRED_BOX && g.d_abs == 0.0 && g.d_rel == 1.0; };
+  // face by face on level L: at most `most` cells for the geometry's largest face, `mean` for its mean face
+  auto small_faces = [&](size_t gi, int L, double most, double mean) {
+    const double emax = gi < ctx->face_ext_max.size() ? ctx->face_ext_max[gi] : INFINITY;
+    const double emean = gi < ctx->face_ext_mean.size() ? ctx->face_ext_mean[gi] : INFINITY;
+    return face_cells(ctx, ctx->geoms[gi], L, emax, 4.0) <= most &&
+           (p->face_pass != AMR_FACE_PASS_AUTO || face_cells(ctx, ctx->geoms[gi], L, emean, 1.0) <= mean);
+  };
+  const bool any = p->face_pass != AMR_FACE_PASS_OFF && P.search == AMR_SEARCH_QUERY_BOX;
+  // levels where geometries end: from the faces when that suits every one of them
+  for (int L = 0; L < P.NL; ++L) P.rec_at[L] = any && P.adjacency && P.fin_at[L] && ctx->dom.dim == 3;
+  for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
+    const int L = ctx->geoms[gi].n_levels - 1;
+    if (P.rec_at[L]) P.rec_at[L] = unit_of(ctx->geoms[gi]) && small_faces(gi, L, kMaxFaceCells, kAutoUnitCells);
+  }
   for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
     GeomParams& g = ctx->geoms[gi];
     uint32_t bits = 0;
-    const double emax = gi < ctx->face_ext_max.size() ? ctx->face_ext_max[gi] : INFINITY;
-    const double emean = gi < ctx->face_ext_mean.size() ? ctx->face_ext_mean[gi] : INFINITY;
-    for (int L = 0; L < g.n_levels && p->face_pass != AMR_FACE_PASS_OFF; ++L) {
-      bool ok = P.search == AMR_SEARCH_QUERY_BOX && (L < g.n_levels - 1 || !P.adjacency);
-      ok = ok && face_cells(ctx, g, L, emax, 4.0) <= kMaxFaceCells;
-      if (ok && p->face_pass == AMR_FACE_PASS_AUTO) ok = face_cells(ctx, g, L, emean, 1.0) <= kAutoFaceCells;
-      if (ok) bits |= 1u << L;
+    for (int L = 0; any && L < g.n_levels; ++L) {
+      const bool mask_only = L < g.n_levels - 1 || !P.adjacency;
+      const double mean = unit_of(g) && ctx->dom.dim == 3 ? kAutoUnitCells : kAutoFaceCells;
+      if (mask_only ? small_faces(gi, L, kMaxFaceCells, mean) : P.rec_at[L]) bits |= 1u << L;
     }
     // the inflated box is the 3^D cells around a cell exactly when d is the cell size on every level
-    const bool unit = P.pred == AMR_PRED_BOX && g.d_abs == 0.0 && g.d_rel == 1.0;
+    const bool unit = unit_of(g);
     if (bits && unit) bits |= kFaceUnit;
     g.face_levels = bits;
     for (int L = 0; L < g.n_levels; ++L) {
@@ -713,7 +749,9 @@ RefineLevel level_args(amr_ctx* ctx, const Plan& P, int L) {
   a.mask = static_cast<uint64_t*>(ctx->lv[L].mask.p);
   a.flag = static_cast<uint8_t*>(ctx->lv[L].flag.p);
   if (P.fin_at[L] && P.adjacency) {
-    a.cellcnt = static_cast<uint16_t*>(ctx->lv[L].cellcnt.p);
+    a.cellcnt = P.rec_at[L] ? nullptr : static_cast<uint16_t*>(ctx->lv[L].cellcnt.p);
+    a.staged = P.rec_at[L] ? static_cast<StagedRec*>(ctx->staged.p) : nullptr;
+    a.info = P.rec_at[L] ? static_cast<uint64_t*>(ctx->lv[L].info.p) : nullptr;
     a.blockcnt = static_cast<uint64_t*>(ctx->lv[L].blockcnt.p);
     a.recs = static_cast<SurvRec*>(ctx->recs.p);
     a.cap_recs = ctx->cap_recs;
@@ -778,7 +816,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
       TRY(ensure(ctx, lb.mask, sizeof(uint64_t) * n1));
       TRY(ensure(ctx, lb.flag, n1));
       if (P.fin_at[L] && P.adjacency) {
-        TRY(ensure(ctx, lb.cellcnt, sizeof(uint16_t) * NCell * n1));
+        if (!P.rec_at[L]) TRY(ensure(ctx, lb.cellcnt, sizeof(uint16_t) * NCell * n1));
         TRY(ensure(ctx, lb.blockcnt, sizeof(uint64_t) * n1));
         TRY(ensure(ctx, lb.base, sizeof(uint64_t) * n1));
         TRY(ensure(ctx, lb.desc, sizeof(uint64_t) * n1));
@@ -788,14 +826,20 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
           TRY(ensure(ctx, ctx->recs, sizeof(SurvRec) * (size_t)want));
           ctx->cap_recs = want;
         }
+        if (P.rec_at[L]) {
+          TRY(ensure(ctx, ctx->staged, sizeof(StagedRec) * (size_t)ctx->cap_recs));
+          TRY(ensure(ctx, lb.info, sizeof(uint64_t) * n1));
+          TRY(ensure(ctx, lb.rfirst, sizeof(uint64_t) * n1));
+        }
         // blocks with more survivor records than shared memory stages were seen: a spill area for
         // every warp the refine launch can hold (32 per SM)
         // (a level marked by parent groups always stages a group's records past shared memory there)
-        if (ctx->want_spill || refine_by_groups(D, L, P.pred, P.search))
+        if (ctx->want_spill || (!P.rec_at[L] && refine_by_groups(D, L, P.pred, P.search)))
           TRY(ensure(ctx, ctx->spill, sizeof(SurvRec) * (size_t)kSpillCap * 32 * (size_t)ctx->num_sms));
       }
     }
     RefineLevel a = level_args(ctx, P, L);
+    MarkArgs marks{};
     CK(cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned), st));
     if (P.face_at[L]) {
       // face by face: masks and flags start clear; deeper levels find their blocks by descending
@@ -810,6 +854,8 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
       m.unit = P.unit_at[L];
       m.plain = P.plain_at[L];
       if (a.blockcnt) CK(cudaMemsetAsync(a.blockcnt, 0, sizeof(uint64_t) * (size_t)(lb.cap > 0 ? lb.cap : 1), st));
+      if (a.info) CK(cudaMemsetAsync(a.info, 0, sizeof(uint64_t) * (size_t)(lb.cap > 0 ? lb.cap : 1), st));
+      marks = m;
       timed(ctx, st, "mark_faces", [&] { return launch_mark_faces(m, ctx->num_sms, st); });
       if (P.walk_at[L]) {
         // the other geometries' blocks: the walk (it also records the faces of those that end here)
@@ -882,18 +928,44 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
     }
     if (P.fin_at[L] && P.adjacency) {
       if (eager) TRY(ensure(ctx, ctx->scratch, scan_u64_scratch_bytes(lb.cap)));
-      timed(ctx, st, "adj_scan", [&] {
-        return launch_scan_u64(static_cast<const uint64_t*>(lb.blockcnt.p), static_cast<uint64_t*>(lb.base.p), lb.cap,
-                               ctx->d_scal + SC_N + L, ctx->d_scal + SC_TOT + L, ctx->scratch.p, ctx->d_err,
-                               ctx->num_sms, st);
-      });
       int64_t cells = 0, pairs = 0;
-      if (eager) {
+      uint64_t tot = 0;
+      for (int attempt = 0; attempt < 2; ++attempt) {
+        timed(ctx, st, "adj_scan", [&] {
+          int k = 0;
+          uint64_t* n_rec = static_cast<uint64_t*>(lb.desc.p);  // (the descriptors take their place)
+          if (P.rec_at[L]) {
+            k += launch_record_counts(a, n_rec, ctx->num_sms, st);
+            k += launch_scan_u64(n_rec, static_cast<uint64_t*>(lb.rfirst.p), lb.cap, ctx->d_scal + SC_N + L,
+                                 ctx->d_scal + SC_RTOT, ctx->scratch.p, ctx->d_err, ctx->num_sms, st);
+          }
+          return k + launch_scan_u64(static_cast<const uint64_t*>(lb.blockcnt.p), static_cast<uint64_t*>(lb.base.p),
+                                     lb.cap, ctx->d_scal + SC_N + L, ctx->d_scal + SC_TOT + L, ctx->scratch.p,
+                                     ctx->d_err, ctx->num_sms, st);
+        });
+        if (!eager) break;
         CK(cudaGetLastError());
-        uint64_t tot = 0;
+        uint64_t n_rec = 0;
         unsigned e = 0;
-        TRY(read_scalar(ctx, st, SC_TOT + L, &tot, &e));
+        TRY(read_scalars(ctx, st, SC_TOT + L, &tot, SC_REC + L, &n_rec, &e));
         TRY(device_error(ctx, e));
+        if (!P.rec_at[L] || (int64_t)n_rec <= ctx->cap_recs) break;
+        // the faces left more records than there was room for: again, with room for all
+        ctx->cap_recs = (int64_t)(n_rec + n_rec / 4 + 1024);
+        TRY(ensure(ctx, ctx->recs, sizeof(SurvRec) * (size_t)ctx->cap_recs));
+        TRY(ensure(ctx, ctx->staged, sizeof(StagedRec) * (size_t)ctx->cap_recs));
+        a = level_args(ctx, P, L);
+        marks.lv = a;
+        CK(cudaMemsetAsync(a.info, 0, sizeof(uint64_t) * (size_t)(lb.cap > 0 ? lb.cap : 1), st));
+        CK(cudaMemsetAsync(a.rec_count, 0, sizeof(uint64_t), st));
+        CK(cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned), st));
+        timed(ctx, st, "mark_faces", [&] { return launch_mark_faces(marks, ctx->num_sms, st); });
+      }
+      if (P.rec_at[L])
+        timed(ctx, st, "place_records", [&] {
+          return launch_place_records(a, static_cast<const uint64_t*>(lb.rfirst.p), ctx->num_sms, st);
+        });
+      if (eager) {
         cells = (int64_t)(tot >> 32);
         pairs = (int64_t)(tot & 0xffffffffull);
         if (run_pairs + pairs >= (int64_t)0xffffffffll)

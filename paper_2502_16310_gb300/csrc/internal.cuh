@@ -461,6 +461,16 @@ struct __align__(16) SurvRec {
   uint32_t pad;
   uint64_t cells;
 };
+// The same left by a face (see k_mark_cells), before the records are placed by block.
+struct StagedRec {
+  uint64_t cells;
+  uint32_t face, block;
+  uint32_t rank;                // among the block's records
+  uint32_t pad;
+};
+constexpr int kInfoShift = 29;  // RefineLevel::info: records | pairs << kInfoShift (a face leaves a block one record)
+constexpr uint64_t kInfoMask = (1ull << kInfoShift) - 1;
+static_assert(kMaxFaces <= 1 << kInfoShift, "a block's records fit");
 constexpr int kRecCap = 64;     // records of a block staged in shared memory
 constexpr int kSpillCap = 960;  // more, up to this many, go to the warp's spill area (when given);
                                 // a block with still more records is walked again for its lists
@@ -481,12 +491,14 @@ struct RefineLevel {
   int64_t nf;
   uint64_t* mask;
   uint8_t* flag;
-  uint16_t* cellcnt;           // per cell face count, blocks whose geometry ends at this level
+  uint16_t* cellcnt;           // per cell face count, blocks whose geometry ends at this level (null: from the records)
   uint64_t* blockcnt;          // per block pairs | adjacent cells << 32 (0 for the others)
   SurvRec* recs;               // survivor records (nullable), capacity cap_recs
   int64_t cap_recs;
   uint64_t* rec_count;         // device: records handed out on this level
-  uint64_t* rec_desc;          // per block: offset << 16 | count, or ~0 (records incomplete)
+  uint64_t* rec_desc;          // per block: offset << kInfoShift | count, or ~0 (records incomplete)
+  StagedRec* staged;           // nullable: records left by the faces, capacity cap_recs; then also:
+  uint64_t* info;              // per block: its records | pairs << kInfoShift (zeroed before)
   SurvRec* spill;              // nullable: kSpillCap records per warp of the launch (records past kRecCap)
   unsigned long long* counters;
   unsigned* work;              // dynamic work counter (zeroed before launch)
@@ -526,6 +538,11 @@ struct MarkArgs {
 };
 constexpr int kFaceBatch = 8;  // most faces a warp of the general kernel takes per work fetch
 int launch_mark_faces(const MarkArgs& m, int num_sms, cudaStream_t st);
+// A level whose records the faces left (lv.staged): blockcnt and the blocks' record counts; then, with
+// first = the exclusive scan of n_rec, the records by block and their descriptors (ERR_OVERFLOW when
+// more were left than cap_recs).
+int launch_record_counts(const RefineLevel& a, uint64_t* n_rec, int num_sms, cudaStream_t st);
+int launch_place_records(const RefineLevel& a, const uint64_t* first, int num_sms, cudaStream_t st);
 
 // The algorithmic cell-face test count of one level (single geometry): per cell
 // of its blocks, the distinct faces in the bins its inflated box overlaps,

@@ -809,7 +809,7 @@ __device__ __noinline__ void spill_record(SurvRec* spill, uint32_t i, uint32_t f
 
 // The block's K survivor records (staged in shared memory, past kRecCap in the
 // warp's spill area) into a contiguous range of the level's record array, and
-// its descriptor: offset << 16 | K, 0 for none, ~0 when they are incomplete (the
+// its descriptor: offset << kInfoShift | K, 0 for none, ~0 when they are incomplete (the
 // adjacency pass then walks the block again).  Whole warp.
 template <int D>
 __device__ __forceinline__ void store_records(const RefineLevel& a, WarpSmem<D>& sm, uint32_t K, unsigned blk,
@@ -851,7 +851,7 @@ __device__ __forceinline__ void store_records(const RefineLevel& a, WarpSmem<D>&
       a.recs[base + i] = r;
     }
   }
-  if (lane == 0) a.rec_desc[blk] = K == 0 ? 0ull : (base == ~0ull ? ~0ull : (base << 16) | K);
+  if (lane == 0) a.rec_desc[blk] = K == 0 ? 0ull : (base == ~0ull ? ~0ull : (base << kInfoShift) | K);
   __syncwarp();
 }
 
@@ -1210,7 +1210,7 @@ __device__ __forceinline__ void walk_group(const RefineLevel& a, const GeomParam
 
 // The group's K records into a contiguous range of the level's record array,
 // grouped by child (each child's records in the order they were found), and
-// every child's descriptor: offset << 16 | count, 0 for none, ~0 when the
+// every child's descriptor: offset << kInfoShift | count, 0 for none, ~0 when the
 // records are incomplete (the adjacency pass then walks the block again).
 __device__ __noinline__ void store_group_records(const RefineLevel& a, GroupSmem& sm, const SurvRec* spill,
                                                   uint32_t K, unsigned blk0, int lane) {
@@ -1241,7 +1241,7 @@ __device__ __noinline__ void store_group_records(const RefineLevel& a, GroupSmem
   }
   const uint32_t incl = warp_inclusive_scan<uint32_t>(lane < 8 ? cntj : 0u);
   const uint32_t first = incl - (lane < 8 ? cntj : 0u);
-  if (lane < 8) a.rec_desc[blk0 + lane] = cntj == 0 ? 0ull : ((base + first) << 16) | cntj;
+  if (lane < 8) a.rec_desc[blk0 + lane] = cntj == 0 ? 0ull : ((base + first) << kInfoShift) | cntj;
   uint32_t run = first;  // lane j < 8: next position of child j
   for (uint32_t i0 = 0; i0 < K; i0 += 32) {
     const uint32_t i = i0 + (uint32_t)lane;
@@ -1473,8 +1473,38 @@ __device__ __forceinline__ void emit_block(const EmitArgs& a, unsigned blk, uint
     const uint64_t base = pre ? pre[0] : a.block_base[blk];
     const uint64_t pair_base = run_pairs + (base & 0xffffffffull);
     const uint64_t cell_base = run_cells + (base >> 32);
-    const uint32_t n0 = lane < NC ? a.lv.cellcnt[(int64_t)blk * NC + lane] : 0u;
-    const uint32_t n1 = D == 3 ? (uint32_t)a.lv.cellcnt[(int64_t)blk * NC + 32 + lane] : 0u;
+    const uint64_t desc = pre ? pre[1] : (a.lv.recs ? a.lv.rec_desc[blk] : ~0ull);
+    const uint32_t K = (uint32_t)(desc & kInfoMask);  // (desc != ~0: the block's records)
+    const uint64_t rec0 = desc >> kInfoShift;
+    // MODE 0: its records, two per lane
+    uint32_t f[2] = {0xffffffffu, 0xffffffffu};
+    uint64_t cm[2] = {0ull, 0ull};
+    const bool held = MODE == 0 && desc != ~0ull && K <= (uint32_t)kRecCap;
+    if (held) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t i = (uint32_t)lane + 32u * h;
+        if (i < K) {
+          const SurvRec r = a.lv.recs[rec0 + i];
+          f[h] = r.face;
+          cm[h] = r.cells;
+        }
+      }
+    }
+    // faces per cell: as the walk counted them, or (a level marked from the faces) from the records
+    uint32_t n0 = 0, n1 = 0;
+    auto count = [&](uint64_t m) {
+      n0 += (uint32_t)(m >> lane) & 1u;
+      n1 += D == 3 ? (uint32_t)(m >> (lane + 32)) & 1u : 0u;
+    };
+    if (a.lv.cellcnt) {
+      n0 = lane < NC ? a.lv.cellcnt[(int64_t)blk * NC + lane] : 0u;
+      n1 = D == 3 ? (uint32_t)a.lv.cellcnt[(int64_t)blk * NC + 32 + lane] : 0u;
+    } else if (held) {
+      for (uint32_t j = 0; j < K; ++j) count(__shfl_sync(0xffffffffu, j < 32 ? cm[0] : cm[1], (int)(j & 31u)));
+    } else {
+      for (uint32_t j = 0; j < K; ++j) count(a.lv.recs[rec0 + j].cells);
+    }
     // exclusive prefixes over cells in bit order (cells 0..31 then 32..63)
     const uint32_t i0 = warp_inclusive_scan<uint32_t>(n0);
     const uint32_t tot0 = __shfl_sync(0xffffffffu, i0, 31);
@@ -1524,26 +1554,12 @@ __device__ __forceinline__ void emit_block(const EmitArgs& a, unsigned blk, uint
         }
       }
     };
-    const uint64_t desc = pre ? pre[1] : (a.lv.recs ? a.lv.rec_desc[blk] : ~0ull);
     constexpr uint32_t kSortRecs = pow2_floor(sort_region_bytes<D>() / 12);  // key + payload per record
     constexpr uint32_t kSortKeys = pow2_floor(sort_region_bytes<D>() / 4);
     if constexpr (MODE == 0) {
-    if (desc != ~0ull && (uint32_t)(desc & 0xffffu) <= (uint32_t)kRecCap) {
+    if (held) {
       // the refine pass left this block's surviving faces with their cell masks:
       // rank them by face id, then every lane lists its cells' faces in that order
-      const uint32_t K = (uint32_t)(desc & 0xffffu);
-      const uint64_t r0 = desc >> 16;
-      uint32_t f[2] = {0xffffffffu, 0xffffffffu};
-      uint64_t cm[2] = {0ull, 0ull};
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t i = (uint32_t)lane + 32u * h;
-        if (i < K) {
-          const SurvRec r = a.lv.recs[r0 + i];
-          f[h] = r.face;
-          cm[h] = r.cells;
-        }
-      }
       uint32_t rank[2] = {0u, 0u};
       for (uint32_t j = 0; j < K; ++j) {
         const uint32_t fj = __shfl_sync(0xffffffffu, j < 32 ? f[0] : f[1], (int)(j & 31u));
@@ -1580,13 +1596,10 @@ __device__ __forceinline__ void emit_block(const EmitArgs& a, unsigned blk, uint
       }
       return;
     } else {
-    if (desc != ~0ull && (uint32_t)(desc & 0xffffu) > (uint32_t)kRecCap &&
-        (uint32_t)(desc & 0xffffu) <= kSortRecs) {
+    if (desc != ~0ull && K > (uint32_t)kRecCap && K <= kSortRecs) {
       // many records: sort them by face id in shared memory, then list the cells' faces in that order
-      const uint32_t K = (uint32_t)(desc & 0xffffu);
-      const uint64_t r0 = desc >> 16;
       uint32_t* sf = reinterpret_cast<uint32_t*>(&sm);
-      const uint64_t* sk = sort_records(a.lv.recs + r0, K, sf, lane);
+      const uint64_t* sk = sort_records(a.lv.recs + rec0, K, sf, lane);
       for (uint32_t j = 0; j < K; ++j) {
         const uint64_t mj = sk[j];
         put(lane < NC && ((mj >> lane) & 1ull), D == 3 && ((mj >> (lane + 32)) & 1ull), sf[j]);
@@ -1771,32 +1784,45 @@ __global__ void __launch_bounds__(kChThreads) k_children(ChildrenArgs a, uint64_
 // only the frame's offset bounds P and O), and the same FP64 resolution.
 // ---------------------------------------------------------------------------
 
-// One cell's SAT test against a survivor: the projections of cell_test2.
+// One cell's SAT test against a survivor: the projections of cell_test2, the box axes and the face
+// normal (in 2D, all) first, then the edge axes.
+__device__ __forceinline__ void cell_axis(float x, const float4& t, bool& sep, bool& in) {
+  sep |= (x < t.x) | (x > t.y);
+  in &= (x > t.z) & (x < t.w);
+}
+
 template <int D>
-__device__ __forceinline__ int cell_test1(const Surv<D>& S, const float* o) {
-  bool sep = false, in = true;
-  auto upd = [&](float x, const float4& t) {
-    sep |= (x < t.x) | (x > t.y);
-    in &= (x > t.z) & (x < t.w);
-  };
-  if constexpr (D == 3) {
+__device__ __forceinline__ void cell_axes_face(const Surv<D>& S, const float* o, bool& sep, bool& in) {
 #pragma unroll
-    for (int ai = 0; ai < 3; ++ai) upd(o[ai], S.t[ai]);
+  for (int ai = 0; ai < D; ++ai) cell_axis(o[ai], S.t[ai], sep, in);
+  if constexpr (D == 3) {
+    const float4 q2 = S.en[2];
+    cell_axis(fmaf(o[2], q2.w, fmaf(o[1], q2.z, o[0] * q2.y)), S.t[3], sep, in);
+  } else {
+    cell_axis(fmaf(o[1], S.e[0], -o[0] * S.e[1]), S.t[2], sep, in);
+  }
+}
+
+template <int D>
+__device__ __forceinline__ void cell_axes_edges(const Surv<D>& S, const float* o, bool& sep, bool& in) {
+  if constexpr (D == 3) {
     const float4 q0 = S.en[0], q1 = S.en[1], q2 = S.en[2];
     const float e[3][3] = {{q0.x, q0.y, q0.z}, {q0.w, q1.x, q1.y}, {q1.z, q1.w, q2.x}};
-    upd(fmaf(o[2], q2.w, fmaf(o[1], q2.z, o[0] * q2.y)), S.t[3]);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const float ex = e[k][0], ey = e[k][1], ez = e[k][2];
-      upd(fmaf(o[2], ey, -o[1] * ez), S.t[4 + 3 * k]);
-      upd(fmaf(o[0], ez, -o[2] * ex), S.t[5 + 3 * k]);
-      upd(fmaf(o[1], ex, -o[0] * ey), S.t[6 + 3 * k]);
+      cell_axis(fmaf(o[2], ey, -o[1] * ez), S.t[4 + 3 * k], sep, in);
+      cell_axis(fmaf(o[0], ez, -o[2] * ex), S.t[5 + 3 * k], sep, in);
+      cell_axis(fmaf(o[1], ex, -o[0] * ey), S.t[6 + 3 * k], sep, in);
     }
-  } else {
-    upd(o[0], S.t[0]);
-    upd(o[1], S.t[1]);
-    upd(fmaf(o[1], S.e[0], -o[0] * S.e[1]), S.t[2]);
   }
+}
+
+template <int D>
+__device__ __forceinline__ int cell_test1(const Surv<D>& S, const float* o) {
+  bool sep = false, in = true;
+  cell_axes_face<D>(S, o, sep, in);
+  cell_axes_edges<D>(S, o, sep, in);
   return sep ? 0 : (in ? 1 : 2);
 }
 
@@ -2112,40 +2138,57 @@ __global__ void __launch_bounds__(kMarkWarps * 32, 6) k_mark_faces(MarkArgs m) {
 // well, for they widen into it.  A cell that a face meets lies in a block of
 // the level: the cell above it was marked.
 //
-// A warp takes up to kCellFaces faces in four steps: a lane per face (cell range,
-// axis thresholds), a lane per block of the ranges (index), a lane per cell, a
-// lane per block again (widening, then one atomic for its new marks), each packed
-// over all the faces.  Bound by instructions and the latency of the block
-// lookups.  Against a warp per face testing every inflated cell (k_mark_faces):
-// the five levels of 1.3 M faces 10.6 -> 2.36 ms, the four of 82 K 0.76 -> 0.29,
-// the three of 20 K 0.22 -> 0.13 (the uncertified cells' tests by one lane in a
-// row: 4.5, 1.0 and 0.53 ms).
+// A warp takes up to kCellFaces faces in steps, each packed over all the faces: a
+// lane per face (cell range, axis thresholds), a lane per block of the ranges
+// (index), where the ranges are long a lane per x-row (the part of it that no
+// axis separates), a lane per cell, a lane per block again (widening, then one
+// atomic for its new marks).  A face with more blocks than kCellPool is taken in
+// tiles.  Bound by instructions and the latency of the block lookups.  Against a
+// warp per face testing every inflated cell (k_mark_faces): the five levels of
+// 1.3 M faces 10.6 -> 2.36 ms, the four of 82 K 0.76 -> 0.29, the three of 20 K
+// 0.22 -> 0.13 (the uncertified cells' tests by one lane in a row: 4.5, 1.0 and
+// 0.53 ms).
+//
+// REC: the level is the last of its geometries and their adjacency is wanted.  A
+// face's widened cells of a block are then the block's survivor record, so the
+// face leaves it (staged, with its rank among the block's records) and
+// k_place_records brings the records together by block: no block walks its bins.
+// Marks and records of the finest level, 1.3 M faces of 9 cells edge on 11 M
+// blocks: 15.5 ms by the parents' walk (k_refine_groups), 4.3 + 1.1 ms; 82 K on
+// 0.76 M: 0.98 -> 0.41 + 0.05.  Without the rows' cut the faces took 5.6 ms; 8
+// faces per warp and 7 blocks per SM 5.9.
 // ---------------------------------------------------------------------------
 template <int D>
 struct MarkFace {
   float shift[3];              // frame corner's rounding error
   float h_hi, h_lo;
   float inv_n0, inv_n1, inv_b0, inv_b1;
-  int lo[3], blo[3];           // first cell of the range, first block of the widened range
+  int lo[3], off[3];           // first cell of the range; its place from the frame's corner, in cells
+  int blo[3];                  // first block of the widened range
   int n0, n1, nb0, nb1, nb2;   // cells and blocks per axis
   int total, nslot;
   uint32_t slot, face, gid;    // first slot of the range's blocks
+  uint8_t c0[3], c1[3];        // blocks of the range (from blo) whose marks are sent
 };
 
 constexpr int kCellWarps = 4;    // warps per CTA of k_mark_cells
 constexpr int kCellBlocks = 5;   // CTAs per SM (shared memory)
 constexpr int kCellFaces = 16;   // faces a warp takes per work fetch
 constexpr int kCellPool = 160;   // blocks of the ranges of a group of faces
+constexpr uint32_t kCellRow = 3; // mean cells per x-row above which rows are cut first
+constexpr int kCellTile = 3;     // a face with more blocks is taken in tiles of 3 per axis and their rims
+static_assert((kCellTile + 2) * (kCellTile + 2) * (kCellTile + 2) <= kCellPool, "a tile and its rim fit");
 
 template <int D>
 struct CellSmem {
   Surv<D> surv[kCellFaces];
   MarkFace<D> f[kCellFaces];
-  alignas(8) uint32_t met[kCellPool][2];    // per block: its cells that the face meets, then widened
+  alignas(8) uint32_t met[kCellPool][2];  // per block: its cells that the face meets, then widened
   uint64_t tmp[kCellPool];
   uint32_t more[kCellPool][2];   // cells marked by their own test
   int32_t bi[kCellPool];         // the block's index (-1: absent)
   uint8_t own[kCellPool];        // its face
+  int whole[4][3];               // a face taken in tiles: lo, n, blo, nb of its range
 };
 
 // Owner of item k0 + lane among items numbered through consecutive ranges: lanes [g0, g1) (own) hold
@@ -2187,6 +2230,43 @@ __device__ __noinline__ int cell_test_grown(const Surv<D>& S, const float* o, fl
   return sep ? 0 : (in ? 1 : 2);
 }
 
+// The part of an x-row (iy, iz) of a face's range that no axis separates from the face: first cell and
+// count.  The projection of a cell centre on an axis is linear along the row, so each axis leaves an
+// interval; it is kept a little too wide (the cells left are tested), which also covers the rounding of
+// the projection at the row's start.  An axis with hardly any x part cuts nothing.
+__device__ __forceinline__ void row_part(const Surv<3>& S, const MarkFace<3>& Q, int iy, int iz, int& ix, uint32_t& n) {
+  const float lx = (float)Q.off[0] + 0.5f, ly = (float)(Q.off[1] + iy) + 0.5f, lz = (float)(Q.off[2] + iz) + 0.5f;
+  const float ox = fmaf(lx, Q.h_hi, fmaf(lx, Q.h_lo, Q.shift[0])), oy = fmaf(ly, Q.h_hi, fmaf(ly, Q.h_lo, Q.shift[1])),
+              oz = fmaf(lz, Q.h_hi, fmaf(lz, Q.h_lo, Q.shift[2]));
+  float lo = 0.f, hi = (float)(Q.n0 - 1);
+  auto cut = [&](float s, float ax, const float4& t) {
+    const float g = ax * Q.h_hi;
+    if (fabsf(g) > 1e-35f) {
+      const float r = __fdividef(1.0f, g), a = (t.x - s) * r, b = (t.y - s) * r;
+      lo = fmaxf(lo, fminf(a, b));
+      hi = fminf(hi, fmaxf(a, b));
+    }
+  };
+  cut(ox, 1.f, S.t[0]);
+  const float4 q0 = S.en[0], q1 = S.en[1], q2 = S.en[2];
+  cut(fmaf(oz, q2.w, fmaf(oy, q2.z, ox * q2.y)), q2.y, S.t[3]);
+  const float e[3][3] = {{q0.x, q0.y, q0.z}, {q0.w, q1.x, q1.y}, {q1.z, q1.w, q2.x}};
+  bool out = (oy < S.t[1].x) | (oy > S.t[1].y) | (oz < S.t[2].x) | (oz > S.t[2].y);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float ex = e[k][0], ey = e[k][1], ez = e[k][2];
+    const float s = fmaf(oz, ey, -oy * ez);
+    const float4 t = S.t[4 + 3 * k];
+    out |= (s < t.x) | (s > t.y);
+    cut(fmaf(ox, ez, -oz * ex), ez, S.t[5 + 3 * k]);
+    cut(fmaf(oy, ex, -ox * ey), -ey, S.t[6 + 3 * k]);
+  }
+  const int i0 = (int)fmaxf(0.f, ceilf(lo - 1e-3f)), i1 = (int)fminf((float)(Q.n0 - 1), floorf(hi + 1e-3f));
+  ix = i0;
+  n = !out && i1 >= i0 ? (uint32_t)(i1 - i0 + 1) : 0u;
+}
+__device__ __forceinline__ void row_part(const Surv<2>&, const MarkFace<2>&, int, int, int&, uint32_t&) {}
+
 // A block mask widened by one cell along axis AX: its own cells, and the neighbours' facing layers
 // (prev / next: the masks of the blocks before and after it on that axis).
 template <int AX>
@@ -2197,7 +2277,7 @@ __device__ __forceinline__ uint64_t widen(uint64_t m, uint64_t prev, uint64_t ne
   return m | ((m << s) & ~first) | ((m >> s) & ~last) | ((prev >> (3 * s)) & first) | ((next << (3 * s)) & last);
 }
 
-template <int D, bool MULTI>
+template <int D, bool MULTI, bool REC>
 __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(MarkArgs m) {
   const RefineLevel& a = m.lv;
   __shared__ __align__(16) CellSmem<D> s_all[kCellWarps];
@@ -2225,6 +2305,13 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
       i = c >= 0 ? (int64_t)c + slot : -1;
     }
     return i < nblk ? (int32_t)i : -1;
+  };
+  auto set_range = [](MarkFace<D>& M, const int* n, const int* nb) {
+    M.total = n[0] * n[1] * n[2];
+    M.nslot = nb[0] * nb[1] * nb[2];
+    M.n0 = n[0], M.n1 = n[1], M.nb0 = nb[0], M.nb1 = nb[1], M.nb2 = nb[2];
+    M.inv_n0 = 1.0f / (float)n[0], M.inv_n1 = 1.0f / (float)n[1];
+    M.inv_b0 = 1.0f / (float)nb[0], M.inv_b1 = 1.0f / (float)nb[1];
   };
   WarpCounters wc;
   unsigned long long n_tests = 0;
@@ -2299,21 +2386,15 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
         atomicOr(a.err, ERR_OVERFLOW);
         use = false;
       }
-      const int nslot = nb[0] * nb[1] * nb[2];
-      if (nslot > kMarkSlots) {  // too many blocks: every cell of the widened range by its own test
 #pragma unroll
-        for (int c = 0; c < D; ++c) {
-          n[c] += 2;
-          M.lo[c] -= 1;
-        }
+      for (int c = 0; c < 3; ++c) {
+        M.off[c] = 0;
+        M.c0[c] = 0;
+        M.c1[c] = (uint8_t)(nb[c] < 255 ? nb[c] : 255);
       }
-      M.total = n[0] * n[1] * n[2];
-      M.nslot = nslot;
-      M.n0 = n[0], M.n1 = n[1], M.nb0 = nb[0], M.nb1 = nb[1], M.nb2 = nb[2];
-      M.inv_n0 = 1.0f / (float)n[0], M.inv_n1 = 1.0f / (float)n[1];
-      M.inv_b0 = 1.0f / (float)nb[0], M.inv_b1 = 1.0f / (float)nb[1];
       M.h_hi = g.h_hi, M.h_lo = g.h_lo;
       M.slot = 0u, M.face = (uint32_t)f, M.gid = gid;
+      set_range(M, n, nb);
     }
     const unsigned valid = __ballot_sync(0xffffffffu, use);
     const int nv = __popc(valid);
@@ -2324,16 +2405,67 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
       sm.f[i] = M;
     }
     __syncwarp();
-    const int my_total = lane < nv ? sm.f[lane].total : 0;
-    const int my_slots = lane < nv ? sm.f[lane].nslot : 0;
+    int my_total = lane < nv ? sm.f[lane].total : 0;
+    int my_slots = lane < nv ? sm.f[lane].nslot : 0;
+    int tile = 0;            // tiles of the face g0 already taken, where it has too many blocks
     for (int g0 = 0; g0 < nv;) {
-      // a run of faces whose blocks fit the slots, or one face with too many blocks
-      const bool slots = sm.f[g0].nslot <= kMarkSlots;
-      const uint32_t ns = lane >= g0 && lane < nv ? (my_slots <= kMarkSlots ? my_slots : kCellPool + 1) : 0u;
+      // a run of faces whose blocks fit the slots, or a tile of one face with more
+      bool big = tile > 0;
+      if (tile == 0) {
+        const MarkFace<D>& Q = sm.f[g0];
+        big = Q.nslot > kCellPool;
+        if (big) {
+          const int wn[3] = {Q.n0, Q.n1, Q.total / (Q.n0 * Q.n1)}, wb[3] = {Q.nb0, Q.nb1, Q.nb2};
+          if (lane == 0) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+              sm.whole[0][q] = Q.lo[q];
+              sm.whole[1][q] = wn[q];
+              sm.whole[2][q] = Q.blo[q];
+              sm.whole[3][q] = wb[q];
+            }
+          }
+          __syncwarp();
+        }
+      }
+      int g1 = g0 + 1;
+      if (big) {
+        int nt[3], t[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) nt[q] = (sm.whole[3][q] + kCellTile - 1) / kCellTile;
+        t[0] = tile % nt[0], t[1] = tile / nt[0] % nt[1], t[2] = tile / (nt[0] * nt[1]);
+        __syncwarp();
+        MarkFace<D> M = sm.f[g0];
+        int n[3], nb[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          // its blocks, one more around them (for the cells that widen into them), and of the face's
+          // range the cells within one of its own
+          const int b0 = t[q] * kCellTile, b1 = min(b0 + kCellTile, sm.whole[3][q]);
+          const int h0 = max(b0 - 1, 0), h1 = min(b1 + 1, sm.whole[3][q]);
+          const int lo = max(sm.whole[0][q], 4 * (sm.whole[2][q] + b0) - 1);
+          const int hi = min(sm.whole[0][q] + sm.whole[1][q] - 1, 4 * (sm.whole[2][q] + b1));
+          M.lo[q] = q < D ? lo : 0;
+          n[q] = q < D ? hi - lo + 1 : 1;
+          M.off[q] = q < D ? lo - sm.whole[0][q] : 0;
+          M.blo[q] = sm.whole[2][q] + h0;
+          nb[q] = h1 - h0;
+          M.c0[q] = (uint8_t)(b0 - h0), M.c1[q] = (uint8_t)(b1 - h0);
+        }
+        if (n[0] <= 0 || n[1] <= 0 || n[2] <= 0) n[0] = n[1] = n[2] = 0;
+        set_range(M, n, nb);
+        __syncwarp();  // every lane has read the face
+        if (lane == 0) sm.f[g0] = M;
+        __syncwarp();
+        if (lane == g0) my_total = M.total, my_slots = M.nslot;
+        if (++tile == nt[0] * nt[1] * nt[2]) tile = 0;
+      }
+      const bool last_tile = tile == 0;
+      const uint32_t ns = lane >= g0 && lane < nv ? (uint32_t)min(my_slots, kCellPool + 1) : 0u;
       const uint32_t sincl = warp_inclusive_scan<uint32_t>(ns);
-      const int g1 = slots ? g0 + __popc(__ballot_sync(0xffffffffu, ns && sincl <= (uint32_t)kCellPool)) : g0 + 1;
+      if (!big) g1 = g0 + __popc(__ballot_sync(0xffffffffu, ns && sincl <= (uint32_t)kCellPool));
       const bool own = lane >= g0 && lane < g1;
-      const uint32_t nsl = slots ? __shfl_sync(0xffffffffu, sincl, g1 - 1) : 0u;
+      const uint32_t nsl = __shfl_sync(0xffffffffu, sincl, g1 - 1);
       const uint32_t sfirst = sincl - ns;
       if (own) sm.f[lane].slot = sfirst;
       __syncwarp();
@@ -2352,25 +2484,16 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
         }
       }
       __syncwarp();
-      // cell x of face j by its own inflated box: FP32, then FP64
-      auto inflated = [&](const MarkFace<D>& Q, int j, const int* x, const float* o) -> bool {
-        const int t = cell_test_grown<D>(sm.surv[j], o, Q.h_hi);
-        if (t != 2) return t != 0;
-        const int b[3] = {x[0] >> 2, x[1] >> 2, x[2] >> 2};
-        const int local = (x[0] & 3) | ((x[1] & 3) << 2) | (D == 3 ? (x[2] & 3) << 4 : 0);
-        return resolve_fp64<D>(a, Q.gid, Q.face, b, local, &wc.fb, &wc.band);
-      };
       const uint32_t nc = own ? (uint32_t)my_total : 0u;
       const uint32_t cincl = warp_inclusive_scan<uint32_t>(nc);
       const uint32_t cfirst = cincl - nc, ncell = __shfl_sync(0xffffffffu, cincl, 31);
-      // cell (i + dd) of face j's range: its coordinates and its centre in the face's frame, whose corner
-      // is the range's first cell (one further in where the range was widened)
+      // cell (i + dd) of face j's range: its coordinates and its centre in the face's frame
       auto centre = [&](const MarkFace<D>& Q, const int* i, int d0, int d1, int d2, int* x, float* o) {
         const int dd[3] = {d0, d1, d2};
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
           x[q] = Q.lo[q] + i[q] + dd[q];
-          const float l = (float)(i[q] + dd[q] - (slots ? 0 : 1)) + 0.5f;
+          const float l = (float)(Q.off[q] + i[q] + dd[q]) + 0.5f;
           o[q] = q < D ? fmaf(l, Q.h_hi, fmaf(l, Q.h_lo, Q.shift[q])) : 0.f;
         }
       };
@@ -2385,108 +2508,177 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
         return Q.slot + (uint32_t)(((x[0] >> 2) - Q.blo[0]) +
                                    Q.nb0 * (((x[1] >> 2) - Q.blo[1]) + Q.nb1 * ((x[2] >> 2) - Q.blo[2])));
       };
-      for (uint32_t k0 = 0; k0 < ncell; k0 += 32) {
-        const int j = range_owner(cfirst, own, g0, k0, lane);
-        const int idx = (int)(k0 + lane - __shfl_sync(0xffffffffu, cfirst, j));
-        bool unsure = false;
-        if (k0 + lane < ncell) {
-          const MarkFace<D>& Q = sm.f[j];
-          int i[3], x[3];
-          float o[3];
-          cell_of(Q, idx, i);
-          centre(Q, i, 0, 0, 0, x, o);
-          ++n_tests;
-          if (slots) {
-            const int t = cell_test1<D>(sm.surv[j], o);
-            if (t == 1) atomicOr(&sm.met[slot_of(Q, x)][local_of(x) >> 5], 1u << (local_of(x) & 31));
-            unsure = t == 2;
-          } else {
-            const int b[3] = {x[0] >> 2, x[1] >> 2, x[2] >> 2};
-            const int32_t bi = find(Q.gid, b);
-            if (bi >= 0 && !((a.mask[bi] >> local_of(x)) & 1ull) && inflated(Q, j, x, o)) {
-              atomicOr(reinterpret_cast<unsigned long long*>(a.mask + bi), 1ull << local_of(x));
-              a.flag[bi] = 1;
-            }
+      // the cells' tests, 32 at a time: of whole ranges, or (ranges with long x-rows) of the part of each
+      // row that no axis separates, a lane per row finding it first
+      const uint32_t nr = own && nc ? (uint32_t)(nc / sm.f[lane].n0) : 0u;
+      const uint32_t rincl = warp_inclusive_scan<uint32_t>(nr);
+      const uint32_t rfirst = rincl - nr, nrow = __shfl_sync(0xffffffffu, rincl, 31);
+      const bool by_row = D == 3 && ncell > kCellRow * nrow;
+      for (uint32_t r0 = 0; r0 < (by_row ? nrow : 1u); r0 += 32) {
+        int jr = 0, iy = 0, iz = 0, ix = 0;
+        uint32_t rc = 0;  // cells of the lane's row, from ix on
+        if (by_row) {
+          jr = range_owner(rfirst, own && nc, g0, r0, lane);
+          const int k = (int)(r0 + lane - __shfl_sync(0xffffffffu, rfirst, jr));
+          if (r0 + lane < nrow) {
+            const MarkFace<D>& Q = sm.f[jr];
+            iz = divn(k, Q.inv_n1);
+            iy = k - iz * Q.n1;
+            row_part(sm.surv[jr], Q, iy, iz, ix, rc);
           }
         }
-        // a cell whose test is not certified: its neighbours by their own inflated boxes, a lane each
-        // (FP64 takes thousands of cycles: in parallel, and not for cells that are marked already)
-        for (unsigned ub = __ballot_sync(0xffffffffu, unsure); ub; ub &= ub - 1) {
-          const int src = __ffs(ub) - 1;
-          const int ju = __shfl_sync(0xffffffffu, j, src), iu = __shfl_sync(0xffffffffu, idx, src);
-          int t = 0, x[3] = {0, 0, 0};
-          if (lane < (D == 3 ? 27 : 9)) {
-            const MarkFace<D>& Q = sm.f[ju];
-            int i[3];
-            float o[3];
-            cell_of(Q, iu, i);
-            centre(Q, i, lane % 3 - 1, lane / 3 % 3 - 1, D == 3 ? lane / 9 - 1 : 0, x, o);
-            const uint32_t s = slot_of(Q, x);
-            const int32_t bi = sm.bi[s];
-            if (bi >= 0) {
-              const uint64_t now = __ldcg(reinterpret_cast<const unsigned long long*>(a.mask + bi));
-              if (!((now >> local_of(x)) & 1ull)) t = cell_test_grown<D>(sm.surv[ju], o, Q.h_hi);
-            }
-            if (D == 2 && t == 2) {
-              const int b[3] = {x[0] >> 2, x[1] >> 2, 0};
-              t = resolve_fp64<D>(a, Q.gid, Q.face, b, local_of(x), &wc.fb, &wc.band) ? 1 : 0;
-            }
-            if (t == 1) atomicOr(&sm.more[s][local_of(x) >> 5], 1u << (local_of(x) & 31));
-          }
-          if constexpr (D == 3) {
-            for (unsigned vb = __ballot_sync(0xffffffffu, t == 2); vb; vb &= vb - 1) {
-              const int e = __ffs(vb) - 1;
-              const MarkFace<D>& Q = sm.f[ju];
-              int y[3];
+        const uint32_t tincl = warp_inclusive_scan<uint32_t>(rc);
+        const uint32_t tfirst = tincl - rc;
+        const uint32_t items = by_row ? __shfl_sync(0xffffffffu, tincl, 31) : ncell;
+        for (uint32_t k0 = 0; k0 < items; k0 += 32) {
+          const bool valid_cell = k0 + lane < items;
+          int j, ci[3] = {0, 0, 0};
+          if (by_row) {
+            int l = 0;  // the last row that starts at or before the item
 #pragma unroll
-              for (int q = 0; q < 3; ++q) y[q] = __shfl_sync(0xffffffffu, x[q], e);
-              bool in_band;
-              const bool adj = resolve_sat_warp(a, Q.gid, Q.face, y[0] >> 2, y[1] >> 2, y[2] >> 2, local_of(y), &in_band);
-              if (lane == 0) {
-                ++wc.fb;
-                wc.band += in_band ? 1ull : 0ull;
-                if (adj) atomicOr(&sm.more[slot_of(Q, y)][local_of(y) >> 5], 1u << (local_of(y) & 31));
+            for (int st = 16; st > 0; st >>= 1) {
+              const uint32_t fs = __shfl_sync(0xffffffffu, tfirst, l + st);
+              if (fs <= k0 + lane) l += st;
+            }
+            j = __shfl_sync(0xffffffffu, jr, l);
+            ci[0] = __shfl_sync(0xffffffffu, ix, l) + (int)(k0 + lane - __shfl_sync(0xffffffffu, tfirst, l));
+            ci[1] = __shfl_sync(0xffffffffu, iy, l);
+            ci[2] = __shfl_sync(0xffffffffu, iz, l);
+          } else {
+            j = range_owner(cfirst, own && nc, g0, k0, lane);  // (a tile may have no cells)
+            const int idx = (int)(k0 + lane - __shfl_sync(0xffffffffu, cfirst, j));
+            if (valid_cell) cell_of(sm.f[j], idx, ci);
+          }
+          const MarkFace<D>& C = sm.f[j];
+          int cx[3];
+          float co[3];
+          bool sep = !valid_cell, in = true;
+          if (valid_cell) {
+            centre(C, ci, 0, 0, 0, cx, co);
+            ++n_tests;
+            cell_axes_face<D>(sm.surv[j], co, sep, in);
+          }
+          // in some rounds the face's plane passes by every cell: no edge axes then
+          if (D == 3 && __any_sync(0xffffffffu, !sep) && valid_cell) cell_axes_edges<D>(sm.surv[j], co, sep, in);
+          if (!sep && in) atomicOr(&sm.met[slot_of(C, cx)][local_of(cx) >> 5], 1u << (local_of(cx) & 31));
+          const bool unsure = !sep && !in;
+          const int idx = ci[0] + C.n0 * (ci[1] + C.n1 * ci[2]);
+          // a cell whose test is not certified: its neighbours by their own inflated boxes, a lane each;
+          // then FP64, by the whole warp in 3D
+          for (unsigned ub = __ballot_sync(0xffffffffu, unsure); ub; ub &= ub - 1) {
+            const int src = __ffs(ub) - 1;
+            const int ju = __shfl_sync(0xffffffffu, j, src), iu = __shfl_sync(0xffffffffu, idx, src);
+            const MarkFace<D>& Q = sm.f[ju];
+            int t = 0, x[3] = {0, 0, 0};
+            if (lane < (D == 3 ? 27 : 9)) {
+              int i[3];
+              float o[3];
+              cell_of(Q, iu, i);
+              centre(Q, i, lane % 3 - 1, lane / 3 % 3 - 1, D == 3 ? lane / 9 - 1 : 0, x, o);
+              const uint32_t s = slot_of(Q, x);
+              const int32_t bi = sm.bi[s];
+              if (bi >= 0) {
+                // (a record wants every cell of its face, a mask only the cells that are not marked yet)
+                const uint64_t now = REC ? 0ull : __ldcg(reinterpret_cast<const unsigned long long*>(a.mask + bi));
+                if (!((now >> local_of(x)) & 1ull)) t = cell_test_grown<D>(sm.surv[ju], o, Q.h_hi);
+              }
+              if (D == 2 && t == 2) {
+                const int b[3] = {x[0] >> 2, x[1] >> 2, 0};
+                t = resolve_fp64<D>(a, Q.gid, Q.face, b, local_of(x), &wc.fb, &wc.band) ? 1 : 0;
+              }
+              if (t == 1) atomicOr(&sm.more[s][local_of(x) >> 5], 1u << (local_of(x) & 31));
+            }
+            if constexpr (D == 3) {
+              for (unsigned vb = __ballot_sync(0xffffffffu, t == 2); vb; vb &= vb - 1) {
+                const int e = __ffs(vb) - 1;
+                int y[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) y[q] = __shfl_sync(0xffffffffu, x[q], e);
+                bool in_band;
+                const bool adj = resolve_sat_warp(a, Q.gid, Q.face, y[0] >> 2, y[1] >> 2, y[2] >> 2, local_of(y), &in_band);
+                if (lane == 0) {
+                  ++wc.fb;
+                  wc.band += in_band ? 1ull : 0ull;
+                  if (adj) atomicOr(&sm.more[slot_of(Q, y)][local_of(y) >> 5], 1u << (local_of(y) & 31));
+                }
               }
             }
+            __syncwarp();
           }
-          __syncwarp();
         }
       }
       __syncwarp();
       // widen along each axis, a lane per block (met -> tmp -> met -> tmp)
       uint64_t* met = reinterpret_cast<uint64_t*>(&sm.met[0][0]);
-      auto pass = [&](auto ax, const uint64_t* in, auto put) {
+      auto pass = [&](auto ax, const uint64_t* in, uint64_t* out, bool last) {
         constexpr int AX = decltype(ax)::value;
         for (uint32_t s = lane; s < nsl; s += 32) {
           const MarkFace<D>& Q = sm.f[sm.own[s]];
           const int k = (int)(s - Q.slot), k1 = divn(k, Q.inv_b0), k2 = divn(k1, Q.inv_b1);
-          const int at = AX == 0 ? k - k1 * Q.nb0 : (AX == 1 ? k1 - k2 * Q.nb1 : k2);
+          const int at[3] = {k - k1 * Q.nb0, k1 - k2 * Q.nb1, k2};
           const int n = AX == 0 ? Q.nb0 : (AX == 1 ? Q.nb1 : Q.nb2);
           const int step = AX == 0 ? 1 : (AX == 1 ? Q.nb0 : Q.nb0 * Q.nb1);
-          put(s, widen<AX>(in[s], at > 0 ? in[s - step] : 0ull, at + 1 < n ? in[s + step] : 0ull));
+          uint64_t w = widen<AX>(in[s], at[AX] > 0 ? in[s - step] : 0ull, at[AX] + 1 < n ? in[s + step] : 0ull);
+          if (last) {
+            w = (w | sm.more[s][0] | ((uint64_t)sm.more[s][1] << 32)) & (D == 3 ? ~0ull : 0xffffull);
+            bool send = sm.bi[s] >= 0;
+#pragma unroll
+            for (int q = 0; q < D; ++q) send = send && at[q] >= Q.c0[q] && at[q] < Q.c1[q];
+            if (!send) w = 0ull;
+          }
+          out[s] = w;
         }
         __syncwarp();
       };
-      // the last pass sends a block's new marks with one atomic
-      auto send = [&](uint32_t s, uint64_t w) {
-        const int32_t bi = sm.bi[s];
-        const uint64_t all = (w | sm.more[s][0] | ((uint64_t)sm.more[s][1] << 32)) & (D == 3 ? ~0ull : 0xffffull);
-        if (bi >= 0 && all) {
+      pass(std::integral_constant<int, 0>{}, met, sm.tmp, false);
+      pass(std::integral_constant<int, 1>{}, sm.tmp, met, D == 2);
+      if constexpr (D == 3) pass(std::integral_constant<int, 2>{}, met, sm.tmp, true);
+      const uint64_t* res = D == 3 ? sm.tmp : met;
+      // a block's new marks with one atomic; a face of a geometry that ends here leaves a record for the block
+      auto ends_here = [&](uint32_t s) {
+        return !MULTI || row<MULTI>(a, sm.f[sm.own[s]].gid).n_levels - 1 == a.level;
+      };
+      uint32_t nrec = 0;
+      for (uint32_t s0 = 0; s0 < nsl; s0 += 32) {
+        const uint32_t s = s0 + lane;
+        const uint64_t w = s < nsl ? res[s] : 0ull;
+        if (w) {
+          const int32_t bi = sm.bi[s];
           const uint64_t now = __ldcg(reinterpret_cast<const unsigned long long*>(a.mask + bi));
-          if (all & ~now) {
-            atomicOr(reinterpret_cast<unsigned long long*>(a.mask + bi), (unsigned long long)all);
+          if (w & ~now) {
+            atomicOr(reinterpret_cast<unsigned long long*>(a.mask + bi), (unsigned long long)w);
             if (now == 0) a.flag[bi] = 1;
           }
         }
-      };
-      pass(std::integral_constant<int, 0>{}, met, [&](uint32_t s, uint64_t w) { sm.tmp[s] = w; });
-      if constexpr (D == 3) {
-        pass(std::integral_constant<int, 1>{}, sm.tmp, [&](uint32_t s, uint64_t w) { met[s] = w; });
-        pass(std::integral_constant<int, 2>{}, met, send);
-      } else {
-        pass(std::integral_constant<int, 1>{}, sm.tmp, send);
+        if constexpr (REC) nrec += __popc(__ballot_sync(0xffffffffu, w && ends_here(s)));
       }
-      g0 = g1;
+      if constexpr (REC) {
+        if (nrec) {
+          uint64_t at = 0;
+          if (lane == 0) at = atomicAdd(reinterpret_cast<unsigned long long*>(a.rec_count), (unsigned long long)nrec);
+          at = __shfl_sync(0xffffffffu, at, 0);
+          for (uint32_t s0 = 0; s0 < nsl; s0 += 32) {
+            const uint32_t s = s0 + lane;
+            const uint64_t w = s < nsl ? res[s] : 0ull;
+            const bool emit = w && ends_here(s);
+            const unsigned eb = __ballot_sync(0xffffffffu, emit);
+            const uint64_t pos = at + __popc(eb & ((1u << lane) - 1u));
+            at += __popc(eb);
+            if (emit && (int64_t)pos < a.cap_recs) {
+              StagedRec r;
+              r.cells = w;
+              r.face = sm.f[sm.own[s]].face;
+              r.block = (uint32_t)sm.bi[s];
+              r.rank = (uint32_t)(atomicAdd(reinterpret_cast<unsigned long long*>(a.info + sm.bi[s]),
+                                            1ull | (unsigned long long)__popcll(w) << kInfoShift) & kInfoMask);
+              r.pad = 0u;
+              a.staged[pos] = r;
+            }
+          }
+        }
+      }
+      __syncwarp();
+      if (last_tile) g0 = g1;
     }
     __syncwarp();  // the next faces reuse the records
   }
@@ -2501,6 +2693,38 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
     if (v[1]) atomicAdd(&a.counters[CNT_BAND], v[1]);
     if (v[2]) atomicAdd(&a.counters[CNT_FACE_SETUPS], v[2]);
     if (v[3]) atomicAdd(&a.counters[CNT_FACE_TESTS], v[3]);
+  }
+}
+
+// After the faces have left their records (staged in any order, each with its rank within its block):
+// per block its pairs | adjacent cells << 32 for the row scan, and its record count for the record scan.
+__global__ void __launch_bounds__(256) k_record_counts(RefineLevel a, uint64_t* n_rec) {
+  const int64_t n = launch_count(a.n_blocks, a.n_dev, a.err);
+  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
+    const uint64_t info = a.info[b];
+    a.blockcnt[b] = info ? (info >> kInfoShift) | ((uint64_t)__popcll(a.mask[b]) << 32) : 0ull;
+    n_rec[b] = info & kInfoMask;
+  }
+}
+
+// The staged records into their blocks' runs (first[b] = scan of the counts), and each block's descriptor.
+__global__ void __launch_bounds__(256) k_place_records(RefineLevel a, const uint64_t* first) {
+  const int64_t n = (int64_t)*a.rec_count;
+  if (n > a.cap_recs) {  // some were not staged: the caller runs again with more room
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.err, ERR_OVERFLOW);
+    return;
+  }
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const StagedRec r = a.staged[i];
+    const uint64_t at = first[r.block];
+    SurvRec o;
+    o.face = r.face;
+    o.pad = 0u;
+    o.cells = r.cells;
+    a.recs[at + r.rank] = o;
+    if (r.rank == 0) {
+      a.rec_desc[r.block] = (at << kInfoShift) | (a.info[r.block] & kInfoMask);
+    }
   }
 }
 
@@ -2596,10 +2820,12 @@ int launch_mark_faces(const MarkArgs& m, int num_sms, cudaStream_t st) {
   };
   auto faces = [&](auto kernel) { go(kernel, kFaceBatch, (int64_t)num_sms * 48, (int64_t)num_sms * 8, kMarkWarps); };
   if (m.unit) {
+    const bool rec = m.lv.staged != nullptr;
     if (m.lv.dim == 3)
-      multi ? cells(k_mark_cells<3, true>) : cells(k_mark_cells<3, false>);
+      multi ? (rec ? cells(k_mark_cells<3, true, true>) : cells(k_mark_cells<3, true, false>))
+            : (rec ? cells(k_mark_cells<3, false, true>) : cells(k_mark_cells<3, false, false>));
     else
-      multi ? cells(k_mark_cells<2, true>) : cells(k_mark_cells<2, false>);
+      multi ? cells(k_mark_cells<2, true, false>) : cells(k_mark_cells<2, false, false>);
   }
   if (m.plain) {
     if (m.lv.dim == 3)
@@ -2610,6 +2836,18 @@ int launch_mark_faces(const MarkArgs& m, int num_sms, cudaStream_t st) {
             : (multi ? faces(k_mark_faces<2, 0, true>) : faces(k_mark_faces<2, 0, false>));
   }
   return k;
+}
+
+int launch_record_counts(const RefineLevel& a, uint64_t* n_rec, int num_sms, cudaStream_t st) {
+  const int64_t g = std::min<int64_t>((a.n_blocks + 255) / 256, (int64_t)num_sms * 8);
+  k_record_counts<<<(unsigned)std::max<int64_t>(1, g), 256, 0, st>>>(a, n_rec);
+  return 1;
+}
+
+int launch_place_records(const RefineLevel& a, const uint64_t* first, int num_sms, cudaStream_t st) {
+  const int64_t g = std::min<int64_t>((a.cap_recs + 255) / 256, (int64_t)num_sms * 8);
+  k_place_records<<<(unsigned)std::max<int64_t>(1, g), 256, 0, st>>>(a, first);
+  return 1;
 }
 
 size_t children_scratch_bytes(int64_t n) {

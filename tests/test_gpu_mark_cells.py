@@ -24,9 +24,9 @@ def _soup(dim, size, n, seed, snap=None):
 
 @pytest.mark.parametrize("dim", [2, 3])
 @pytest.mark.parametrize("root", [4, 5])
-@pytest.mark.parametrize("size,snap", [(0.001, None), (0.02, None), (0.3, None), (0.05, 1 / 64), (0.05, 1 / 40)])
+@pytest.mark.parametrize("size,snap", [(0.001, None), (0.02, None), (0.14, None), (0.3, None), (0.05, 1 / 64), (0.05, 1 / 40)])
 def test_cells_equal_block_walk(dim, root, size, snap):
-    n = 40 if size > 0.1 else 300
+    n = 40 if size > 0.2 else 300
     v, f = _soup(dim, size, n, seed=int(1000 * size) + root, snap=snap)
     w = Workload("soup", dim, v, f, root=root, n_levels=3, bins=6, lattice=9 if dim == 2 else 19)
     on = U.run_gpu(w, face_pass=ON)
