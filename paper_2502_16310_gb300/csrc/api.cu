@@ -62,6 +62,9 @@ constexpr int SC_NL = 32;    // [16] links per level
 constexpr int SC_RUN = 48;   // [3] running cells, pairs, links
 constexpr int SC_REC = 52;   // [16] survivor records handed out per level
 constexpr int SC_RTOT = 68;    // records placed (the record scan's total)
+constexpr int SC_HITS = 69;    // links from the faces: hits, runs, groups
+constexpr int SC_RUNS = 70;
+constexpr int SC_NGRP = 71;
 constexpr int SC_WORDS = 72;
 
 // A captured graph stays valid while no buffer it uses was reallocated
@@ -109,6 +112,9 @@ struct amr_ctx {
   DevBuf X, nrm, frec, recs, staged, hkeys, hvals, mkeys, mvals, cls, flbase, tl_cell, tl_dir, tl_q, tl_face, stage_a, stage_b, frange, count, offsets, ids, payload, scratch, misc, scal;
   LevelBufs lv[AMR_MAX_LEVELS];
   DevBuf adj_cell, adj_off, adj_ids, link_cell, link_dir, link_q, link_face, link_stage;
+  DevBuf hit_q, hit_code, run_staged, runs, grp_runs, grp_first, grp_links, grp_base;  // links from the faces
+  int64_t cap_hits = 0, cap_runs = 0;
+  bool face_links[AMR_MAX_LEVELS] = {};  // the last eager pass found the level's links from the faces
   int64_t cap_cells = 0, cap_pairs = 0, cap_links = 0;
   int64_t cap_recs = 0, want_recs = 0;  // survivor record staging (entries)
   bool sampled_bins = false;             // the last binning used the paper's sampled membership
@@ -350,17 +356,12 @@ amr_status read_scalar(amr_ctx* ctx, cudaStream_t st, int slot, uint64_t* v, uns
   return AMR_OK;
 }
 
-// Two of them.
-amr_status read_scalars(amr_ctx* ctx, cudaStream_t st, int slot0, uint64_t* v0, int slot1, uint64_t* v1,
-                        unsigned* err_out) {
-  char* h = static_cast<char*>(ctx->h_pinned);
-  TRY(small_copy(ctx, st, {{ctx->h_dev + 128, ctx->d_scal + slot0, sizeof(uint64_t)},
-                      {ctx->h_dev + 136, ctx->d_scal + slot1, sizeof(uint64_t)},
+// All of them (at 512 of the pinned block) and the error word.
+amr_status read_block(amr_ctx* ctx, cudaStream_t st, unsigned* err_out) {
+  TRY(small_copy(ctx, st, {{ctx->h_dev + 512, ctx->d_scal, sizeof(uint64_t) * SC_WORDS},
                       {ctx->h_dev + 64, ctx->d_err, sizeof(unsigned)}}));
   TRY(sync_check(ctx, st));
-  *v0 = *reinterpret_cast<uint64_t*>(h + 128);
-  *v1 = *reinterpret_cast<uint64_t*>(h + 136);
-  *err_out = *reinterpret_cast<unsigned*>(h + 64);
+  *err_out = *reinterpret_cast<unsigned*>(static_cast<char*>(ctx->h_pinned) + 64);
   return AMR_OK;
 }
 
@@ -495,6 +496,8 @@ void amr_ctx_free(amr_ctx* ctx) {
                    &ctx->link_cell, &ctx->link_dir,     &ctx->link_q,     &ctx->link_face,  &ctx->link_stage, &ctx->idx,
                    &ctx->vert_off,  &ctx->vert_corners, &ctx->face_key,   &ctx->face_acc,   &ctx->face_lines,
                    &ctx->grad_face, &ctx->sort_scratch, &ctx->group_cnt,  &ctx->lvl_ptrs,   &ctx->table,
+                   &ctx->hit_q,     &ctx->hit_code,     &ctx->run_staged, &ctx->runs,       &ctx->grp_runs,   &ctx->grp_first,
+                   &ctx->grp_links, &ctx->grp_base,
                    &ctx->face_gid,  &ctx->fstat,        &ctx->spill,      &ctx->calg,       &ctx->defer};
   for (DevBuf* b : all) release(ctx, *b);
   for (int L = 0; L < AMR_MAX_LEVELS; ++L) {
@@ -654,6 +657,11 @@ constexpr double kAutoFaceCells = 1024.0;
 // 13.8 cells 0.41 / 0.51, 19.6 cells 0.54 / 0.52).  In 2D the walk of the last level is never dearer than
 // the records' launches (0.33 / 0.35 ms for 20,000 edges).
 constexpr double kAutoUnitCells = 8192.0;
+
+// Links from the faces (k_flinks.cu) from this many (cell, face) pairs on: its seven launches cost about 30 us
+// more than the pair kernel's four (0.5 M links of 20 K faces 0.113 / 0.088 ms), from about 8 M links on it is
+// the faster (8 K faces 0.39 / 0.38 ms, 32 K faces 0.41 / 0.46, 97 M links of 72 K faces 3.13 / 4.37).
+constexpr int64_t kFaceLinkPairs = 4 << 20;
 
 // Cells of level L in the range of a face of geometry g whose largest AABB side
 // is ext root cells: (ext 2^L + 2 d_L / h_L + pad) per axis (pad 4 bounds the
@@ -928,7 +936,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
     }
     if (P.fin_at[L] && P.adjacency) {
       if (eager) TRY(ensure(ctx, ctx->scratch, scan_u64_scratch_bytes(lb.cap)));
-      int64_t cells = 0, pairs = 0;
+      int64_t cells = 0, pairs = 0, n_rec = 0;
       uint64_t tot = 0;
       for (int attempt = 0; attempt < 2; ++attempt) {
         timed(ctx, st, "adj_scan", [&] {
@@ -945,13 +953,15 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         });
         if (!eager) break;
         CK(cudaGetLastError());
-        uint64_t n_rec = 0;
         unsigned e = 0;
-        TRY(read_scalars(ctx, st, SC_TOT + L, &tot, SC_REC + L, &n_rec, &e));
+        TRY(read_block(ctx, st, &e));
+        const uint64_t* sc = reinterpret_cast<const uint64_t*>(static_cast<char*>(ctx->h_pinned) + 512);
+        tot = sc[SC_TOT + L];
+        n_rec = (int64_t)sc[SC_REC + L];
         TRY(device_error(ctx, e));
-        if (!P.rec_at[L] || (int64_t)n_rec <= ctx->cap_recs) break;
+        if (!P.rec_at[L] || n_rec <= ctx->cap_recs) break;
         // the faces left more records than there was room for: again, with room for all
-        ctx->cap_recs = (int64_t)(n_rec + n_rec / 4 + 1024);
+        ctx->cap_recs = n_rec + n_rec / 4 + 1024;
         TRY(ensure(ctx, ctx->recs, sizeof(SurvRec) * (size_t)ctx->cap_recs));
         TRY(ensure(ctx, ctx->staged, sizeof(StagedRec) * (size_t)ctx->cap_recs));
         a = level_args(ctx, P, L);
@@ -1001,7 +1011,92 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         return launch_advance(ctx->d_scal + SC_TOT + L, nullptr, ctx->d_scal + SC_RUN,
                               static_cast<uint32_t*>(ctx->adj_off.p), ctx->cap_cells, ctx->d_err, true, st);
       });
-      if (P.links) {
+      if (eager) ctx->face_links[L] = P.links && P.rec_at[L] && L > 0 && pairs >= kFaceLinkPairs;
+      if (P.links && ctx->face_links[L]) {  // (a capture follows the eager pass before it)
+        // the faces that left the records find the links too
+        FaceLinkArgs fl{};
+        fl.level = L;
+        fl.g0 = ctx->geoms[0];
+        fl.table = a.table;
+        fl.face_gid = marks.face_gid;
+        fl.rec = marks.rec;
+        fl.nf = ctx->nf;
+        for (int l = 0; l < L; ++l) fl.first_child[l] = marks.first_child[l];
+        fl.n_blocks = lb.cap;
+        fl.n_dev = a.n_dev;
+        fl.mask = a.mask;
+        fl.block_base = ea.block_base;
+        fl.run = ctx->d_scal + SC_RUN;
+        fl.hit_count = reinterpret_cast<unsigned long long*>(ctx->d_scal + SC_HITS);
+        fl.run_count = reinterpret_cast<unsigned long long*>(ctx->d_scal + SC_RUNS);
+        fl.n_groups = ctx->d_scal + SC_NGRP;
+        fl.scan_total = ctx->d_scal + SC_RTOT;
+        fl.n_links = ctx->d_scal + SC_NL + L;
+        fl.counters = ctx->counters;
+        fl.work = ctx->d_work;
+        fl.err = ctx->d_err;
+        for (int attempt = 0; attempt < 2; ++attempt) {
+          if (eager) {
+            // first guesses: a quarter more hits than (cell, face) pairs, two runs per record; a level
+            // with more of anything runs once more with room for its exact counts
+            if (attempt == 0) {
+              ctx->cap_hits = std::max(ctx->cap_hits, pairs + pairs / 4 + 1024);
+              ctx->cap_runs = std::max(ctx->cap_runs, 2 * n_rec + 4096);
+            }
+            const int64_t want = run_links + ctx->cap_hits;
+            if (want > ctx->cap_links) {
+              const size_t keep = (size_t)run_links;
+              TRY(ensure_keep(ctx, ctx->link_cell, sizeof(uint32_t) * (size_t)(want + 1), sizeof(uint32_t) * keep));
+              TRY(ensure_keep(ctx, ctx->link_dir, (size_t)(want + 1), keep));
+              TRY(ensure_keep(ctx, ctx->link_q, sizeof(float) * (size_t)(want + 1), sizeof(float) * keep));
+              TRY(ensure_keep(ctx, ctx->link_face, sizeof(uint32_t) * (size_t)(want + 1), sizeof(uint32_t) * keep));
+              ctx->cap_links = want;
+            }
+            const size_t ng = (size_t)(lb.cap / 8 + 1);
+            TRY(ensure(ctx, ctx->hit_q, sizeof(float) * (size_t)ctx->cap_hits));
+            TRY(ensure(ctx, ctx->hit_code, sizeof(uint16_t) * (size_t)ctx->cap_hits));
+            TRY(ensure(ctx, ctx->run_staged, sizeof(StagedRun) * (size_t)ctx->cap_runs));
+            TRY(ensure(ctx, ctx->runs, sizeof(HitRun) * (size_t)ctx->cap_runs));
+            TRY(ensure(ctx, ctx->grp_runs, sizeof(uint64_t) * ng));
+            TRY(ensure(ctx, ctx->grp_first, sizeof(uint64_t) * ng));
+            TRY(ensure(ctx, ctx->grp_links, sizeof(uint64_t) * ng));
+            TRY(ensure(ctx, ctx->grp_base, sizeof(uint64_t) * ng));
+            TRY(ensure(ctx, ctx->scratch, scan_u64_scratch_bytes((int64_t)ng)));
+          }
+          fl.hit_q = static_cast<float*>(ctx->hit_q.p);
+          fl.hit_code = static_cast<uint16_t*>(ctx->hit_code.p);
+          fl.cap_hits = ctx->cap_hits;
+          fl.staged = static_cast<StagedRun*>(ctx->run_staged.p);
+          fl.runs = static_cast<HitRun*>(ctx->runs.p);
+          fl.cap_runs = ctx->cap_runs;
+          fl.group_runs = static_cast<unsigned long long*>(ctx->grp_runs.p);
+          fl.first = static_cast<uint64_t*>(ctx->grp_first.p);
+          fl.group_links = static_cast<uint64_t*>(ctx->grp_links.p);
+          fl.link_base = static_cast<uint64_t*>(ctx->grp_base.p);
+          fl.link_cell = static_cast<uint32_t*>(ctx->link_cell.p);
+          fl.link_dir = static_cast<uint8_t*>(ctx->link_dir.p);
+          fl.link_q = static_cast<float*>(ctx->link_q.p);
+          fl.link_face = static_cast<uint32_t*>(ctx->link_face.p);
+          fl.link_cap = ctx->cap_links;
+          timed(ctx, st, "links", [&] { return launch_face_links(fl, ctx->scratch.p, ctx->num_sms, st); });
+          if (!eager) break;
+          CK(cudaGetLastError());
+          unsigned e = 0;
+          TRY(read_block(ctx, st, &e));
+          const uint64_t* sc = reinterpret_cast<const uint64_t*>(static_cast<char*>(ctx->h_pinned) + 512);
+          const int64_t hits = (int64_t)sc[SC_HITS], runs = (int64_t)sc[SC_RUNS];
+          if (e & ~ERR_OVERFLOW) TRY(device_error(ctx, e));
+          if (hits <= ctx->cap_hits && runs <= ctx->cap_runs) {
+            if (e) TRY(device_error(ctx, e));
+            run_links += (int64_t)sc[SC_NL + L];
+            break;
+          }
+          if (attempt) return fail(ctx, AMR_EOVERFLOW, "links: counts changed between two runs");
+          CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(unsigned), st));
+          ctx->cap_hits = std::max(ctx->cap_hits, hits);
+          ctx->cap_runs = std::max(ctx->cap_runs, runs);
+        }
+      } else if (P.links) {
         LinkArgs la{};
         la.dim = D;
         la.lattice = P.lattice;

@@ -356,6 +356,26 @@ __device__ __forceinline__ T warp_inclusive_scan(T v) {
   return v;
 }
 
+// Block count of a launch: from device memory when given (bounded by the
+// capacity; an overflow is reported), else the host count.
+__device__ __forceinline__ int64_t launch_count(int64_t n, const uint64_t* n_dev, unsigned* err) {
+  if (!n_dev) return n;
+  const uint64_t nd = *n_dev;
+  if ((int64_t)nd > n) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, ERR_OVERFLOW);
+    return n;
+  }
+  return (int64_t)nd;
+}
+
+// Owner of item k0 + lane among items numbered through consecutive ranges: lanes [g0, g1) (own) hold
+// their ranges' first items; returns the owner's lane.
+__device__ __forceinline__ int range_owner(uint32_t first, bool own, int g0, uint32_t k0, int lane) {
+  const unsigned before = __popc(__ballot_sync(0xffffffffu, own && first < k0));
+  const unsigned heads = __reduce_or_sync(0xffffffffu, own && first - k0 < 32u ? 1u << (first - k0) : 0u);
+  return g0 + (int)(before + __popc(heads & (0xffffffffu >> (31 - lane)))) - 1;
+}
+
 // --- lattice directions ------------------------------------------------------
 // D3Q19 direction i (1..18), component a: 1..6 = +x,-x,+y,-y,+z,-z; 7..18 =
 // the xy, xz and yz plane diagonals, each as (+,+), (-,-), (+,-), (-,+).
@@ -398,6 +418,14 @@ constexpr uint64_t kDir2X = pack_dir2_axis(0), kDir2Y = pack_dir2_axis(1);
 // Streaming multiprocessors of the current device (queried once per device);
 // grids of the grid-stride kernels are capped at a multiple of it.
 int current_sm_count();
+// Items a warp takes per fetch, at most `most`: the n items go in as few equal rounds over the resident warps
+// as that allows (a last round that is nearly empty would take as long as a full one: 20 K faces in fetches of
+// 6 over 3,040 warps left 373 of them a second one).
+inline int fetch_size(int64_t n, int64_t warps, int most) {
+  const int64_t rounds = (n + warps * most - 1) / (warps * most);
+  const int64_t k = rounds > 0 ? (n + warps * rounds - 1) / (warps * rounds) : 1;
+  return k < 1 ? 1 : (int)k;
+}
 // Gather nf faces into the SoA array X (row stride ld, default nf) starting at face f0.
 int launch_load_indexed(int dim, const float* verts, int64_t nv, const int32_t* idx, int64_t nf, float* X,
                         unsigned* err, cudaStream_t st, int64_t ld = -1, int64_t f0 = 0);
@@ -559,6 +587,13 @@ struct CountArgs {
 };
 int launch_count_candidates(const CountArgs& a, int num_sms, cudaStream_t st);
 
+// Table row of a geometry; a single geometry's row is a kernel argument (read in place, not copied).
+template <bool MULTI>
+__device__ __forceinline__ const GeomParams& row(const RefineLevel& a, uint32_t gid) {
+  if constexpr (MULTI) return a.table[gid];
+  return a.g0;
+}
+
 struct EmitArgs {
   RefineLevel lv;
   const uint64_t* block_base;  // exclusive scan of blockcnt over this level
@@ -674,6 +709,59 @@ struct LinkArgs {
   unsigned long long* counters;
   unsigned* err;
 };
+
+// Links found from the faces (k_flinks.cu): 3D, a level below the roots whose survivor records the
+// faces left.  Hits leave as runs, one per (face, group), a group being the 8 blocks of one parent.
+struct StagedRun {
+  unsigned long long start;    // first hit
+  uint32_t n, face;
+  uint32_t group, rank;        // rank among the group's runs
+};
+struct __align__(16) HitRun {
+  unsigned long long start;
+  uint32_t n, face;
+};
+struct FaceLinkArgs {
+  int level;
+  GeomParams g0;
+  const GeomParams* table;
+  const uint32_t* face_gid;
+  const FaceRec3* rec;
+  int64_t nf;
+  const int32_t* first_child[kMaxLevels];
+  int64_t n_blocks;            // capacity of the level (n_dev: its count)
+  const uint64_t* n_dev;
+  const uint64_t* mask;
+  const uint64_t* block_base;  // exclusive scan of blockcnt
+  const uint64_t* run;         // device running totals before this level: [0] rows, [2] links
+  float* hit_q;                // hits: q, direction << 9 | cell of the group; capacity cap_hits
+  uint16_t* hit_code;
+  int64_t cap_hits;
+  StagedRun* staged;           // runs as they leave, and by group; capacity cap_runs
+  HitRun* runs;
+  int64_t cap_runs;
+  unsigned long long* hit_count;   // device counters (run_count = hit_count + 1)
+  unsigned long long* run_count;
+  uint64_t* n_groups;
+  uint64_t* scan_total;
+  unsigned long long* group_runs;  // per group: runs, their scan, links, their scan
+  uint64_t* first;
+  uint64_t* group_links;
+  uint64_t* link_base;
+  uint32_t* link_cell;
+  uint8_t* link_dir;
+  float* link_q;
+  uint32_t* link_face;
+  int64_t link_cap;
+  uint64_t* n_links;           // device: this level's link count
+  unsigned long long* counters;
+  unsigned* work;
+  unsigned* err;
+  int batch;                   // faces per work fetch (set by the launcher)
+};
+// ERR_OVERFLOW where hits, runs or links exceed their capacity (their counts are right then).
+int launch_face_links(const FaceLinkArgs& a, void* scan_scratch, int num_sms, cudaStream_t st);
+
 size_t links_scratch_bytes(int64_t n_adj);
 size_t links_stage_bytes(int64_t cap_links);
 // Three kernels (links, the scan of the tiles' counts, placement); returns the launch count.

@@ -23,7 +23,7 @@
 // there.  No tile waits for the tiles before it.
 #include <atomic>
 
-#include "internal.cuh"
+#include "links.cuh"
 
 namespace amr {
 
@@ -43,76 +43,6 @@ static_assert(d3q19_c(7, 0) == 1 && d3q19_c(7, 1) == 1 && d3q19_c(8, 0) == -1 &&
 static_assert(d3q19_c(9, 0) == 1 && d3q19_c(9, 1) == -1 && d3q19_c(10, 0) == -1 && d3q19_c(10, 1) == 1, "xy");
 static_assert(d3q19_c(13, 0) == 1 && d3q19_c(13, 2) == -1 && d3q19_c(13, 1) == 0, "xz");
 static_assert(d3q19_c(18, 1) == -1 && d3q19_c(18, 2) == 1 && d3q19_c(18, 0) == 0, "yz");
-
-__device__ __forceinline__ void d3q19_dir(int i, int& cx, int& cy, int& cz) {
-  cx = d3q19_c(i, 0);
-  cy = d3q19_c(i, 1);
-  cz = d3q19_c(i, 2);
-}
-
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
-
-__device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
-  p = a * b;
-  e = fmaf(a, b, -p);
-}
-
-struct LinkHit {
-  bool hit;
-  bool band;
-  double t;
-};
-
-__device__ __noinline__ LinkHit link_fp64_3(const float* V, const double* xc, const int* ci, double h);
-
-// FP64 evaluation of direction di for the cell (block coordinates blk3, cell bit),
-// with the cell centre formed in FP64 (the slow path of undecided signs).
-__device__ __noinline__ LinkHit link_fallback_3(const float* V, const int* blk3, uint32_t bit, const double* origin,
-                                                double h, int di) {
-  int ci[3];
-  d3q19_dir(di, ci[0], ci[1], ci[2]);
-  double xc[3];
-  for (int c = 0; c < 3; ++c) {
-    const int gc = 4 * blk3[c] + (int)((bit >> (2 * c)) & 3u);
-    xc[c] = __dadd_rn(origin[c], __dmul_rn((double)gc + 0.5, h));
-  }
-  return link_fp64_3(V, xc, ci, h);
-}
-
-// FP64 evaluation of one (link, face) pair, same definition as the FP32 path.
-__device__ __noinline__ LinkHit link_fp64_3(const float* V, const double* xc, const int* ci, double h) {
-  LinkHit r{false, false, 0.0};
-  double p[3][3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) p[k][c] = (double)V[3 * k + c] - xc[c];
-  const double d[3] = {ci[0] * h, ci[1] * h, ci[2] * h};
-  const double u[3] = {p[1][0] - p[0][0], p[1][1] - p[0][1], p[1][2] - p[0][2]};
-  const double w[3] = {p[2][0] - p[0][0], p[2][1] - p[0][1], p[2][2] - p[0][2]};
-  const double n[3] = {u[1] * w[2] - u[2] * w[1], u[2] * w[0] - u[0] * w[2], u[0] * w[1] - u[1] * w[0]};
-  const double ln = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-  if (ln == 0.0) return r;
-  const double den = d[0] * n[0] + d[1] * n[1] + d[2] * n[2];
-  if (den == 0.0) return r;
-  const double ld = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-  if (fabs(den) <= kBandRel * ld * ln) r.band = true;
-  auto vol = [&](const double* a, const double* b) {
-    const double c0 = a[1] * b[2] - a[2] * b[1], c1 = a[2] * b[0] - a[0] * b[2], c2 = a[0] * b[1] - a[1] * b[0];
-    return d[0] * c0 + d[1] * c1 + d[2] * c2;
-  };
-  const double l0 = vol(p[1], p[2]) / den, l1 = vol(p[2], p[0]) / den, l2 = vol(p[0], p[1]) / den;
-  const double t = (p[0][0] * n[0] + p[0][1] * n[1] + p[0][2] * n[2]) / den;
-  const double mu = fmin(fmin(fmin(l0, l1), l2), fmin(t, 1.0 - t));
-  if (fabs(mu) <= kBandRel) r.band = true;
-  r.hit = mu >= 0.0;
-  r.t = t;
-  return r;
-}
 
 __device__ __noinline__ LinkHit link_fp64_2(const float* V, const double* xc, const int* ci, double h) {
   LinkHit r{false, false, 0.0};
@@ -353,7 +283,7 @@ __global__ void __launch_bounds__(kLThreads) k_links(LinkArgs a, LinkTiles lt) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
               float sm, err;
-              two_sum(V[3 * k + c], -ohi[c], sm, err);
+              df_two_sum(V[3 * k + c], -ohi[c], sm, err);
               const float l = err - olo[c];
               if (k == 0) {
                 ph0[c] = sm;
@@ -364,12 +294,12 @@ __global__ void __launch_bounds__(kLThreads) k_links(LinkArgs a, LinkTiles lt) {
             }
           // num = n . (v0 - x) in double-float
           float ns, ne;
-          two_prod(nh[0], ph0[0], ns, ne);
+          df_two_prod(nh[0], ph0[0], ns, ne);
 #pragma unroll
           for (int c = 1; c < 3; ++c) {
             float pp, pe, sm, t;
-            two_prod(nh[c], ph0[c], pp, pe);
-            two_sum(ns, pp, sm, t);
+            df_two_prod(nh[c], ph0[c], pp, pe);
+            df_two_sum(ns, pp, sm, t);
             ns = sm;
             ne += t + pe;
           }
@@ -461,8 +391,8 @@ __global__ void __launch_bounds__(kLThreads) k_links(LinkArgs a, LinkTiles lt) {
             const float cl = fabsf(cx) + fabsf(cy) + fabsf(cz);
             // den = c . n in double-float (c has at most two non-zero unit entries)
             float s1, e1, dh, e2;
-            two_sum(cx * nh[0], cy * nh[1], s1, e1);
-            two_sum(s1, cz * nh[2], dh, e2);
+            df_two_sum(cx * nh[0], cy * nh[1], s1, e1);
+            df_two_sum(s1, cz * nh[2], dh, e2);
             const float dl = (e1 + e2) + (cx * nl[0] + cy * nl[1] + cz * nl[2]);
             const float den = dh + dl;
             bool test = !(den == 0.0f && dh == 0.0f);  // else c_i parallel to the face plane: no hit

@@ -815,18 +815,6 @@ template <int D>
 __device__ __forceinline__ void store_records(const RefineLevel& a, WarpSmem<D>& sm, uint32_t K, unsigned blk,
                                               int lane);
 
-// Block count of a launch: from device memory when given (bounded by the
-// capacity; an overflow is reported), else the host count.
-__device__ __forceinline__ int64_t launch_count(int64_t n, const uint64_t* n_dev, unsigned* err) {
-  if (!n_dev) return n;
-  const uint64_t nd = *n_dev;
-  if ((int64_t)nd > n) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(err, ERR_OVERFLOW);
-    return n;
-  }
-  return (int64_t)nd;
-}
-
 template <int D>
 __device__ __forceinline__ void store_records(const RefineLevel& a, WarpSmem<D>& sm, uint32_t K, unsigned blk,
                                               int lane) {
@@ -1826,13 +1814,6 @@ __device__ __forceinline__ int cell_test1(const Surv<D>& S, const float* o) {
   return sep ? 0 : (in ? 1 : 2);
 }
 
-// Table row of a geometry; a single geometry's row is a kernel argument (read in place, not copied).
-template <bool MULTI>
-__device__ __forceinline__ const GeomParams& row(const RefineLevel& a, uint32_t gid) {
-  if constexpr (MULTI) return a.table[gid];
-  return a.g0;
-}
-
 // setup_face without the block cull, lane-parallel: lane ai < 13 (2D: 3)
 // computes axis ai with setup_face's arithmetic; lane 0 stores the edges.
 template <int D>
@@ -2190,14 +2171,6 @@ struct CellSmem {
   uint8_t own[kCellPool];        // its face
   int whole[4][3];               // a face taken in tiles: lo, n, blo, nb of its range
 };
-
-// Owner of item k0 + lane among items numbered through consecutive ranges: lanes [g0, g1) (own) hold
-// their ranges' first items; returns the owner's lane.
-__device__ __forceinline__ int range_owner(uint32_t first, bool own, int g0, uint32_t k0, int lane) {
-  const unsigned before = __popc(__ballot_sync(0xffffffffu, own && first < k0));
-  const unsigned heads = __reduce_or_sync(0xffffffffu, own && first - k0 < 32u ? 1u << (first - k0) : 0u);
-  return g0 + (int)(before + __popc(heads & (0xffffffffu >> (31 - lane)))) - 1;
-}
 
 // cell_test1 for the cell's box widened by grow: the thresholds move by grow |a|_1, and the
 // certificates by the rounding of that.
@@ -2806,19 +2779,21 @@ int launch_mark_faces(const MarkArgs& m, int num_sms, cudaStream_t st) {
   if (m.lv.nf <= 0) return 0;
   const bool point = m.lv.pred == 1, multi = m.lv.table != nullptr;
   int k = 0;
-  // `per` faces at most per fetch, fewer where that would leave warps without work
-  auto go = [&](auto kernel, int per, int64_t fetches, int64_t resident, int warps) {
+  auto go = [&](auto kernel, int batch, int64_t resident, int warps) {
     MarkArgs x = m;
-    x.batch = (int)std::max<int64_t>(1, std::min<int64_t>(per, m.lv.nf / fetches));
+    x.batch = batch;
     const int64_t need = (m.lv.nf + (int64_t)x.batch * warps - 1) / ((int64_t)x.batch * warps);
     if (k++) cudaMemsetAsync(m.lv.work, 0, sizeof(unsigned), st);
     kernel<<<(unsigned)std::min<int64_t>(need, resident), warps * 32, 0, st>>>(x);
   };
   auto cells = [&](auto kernel) {
     const int64_t grid = (int64_t)num_sms * kCellBlocks;
-    go(kernel, kCellFaces, grid * kCellWarps, grid, kCellWarps);
+    go(kernel, fetch_size(m.lv.nf, grid * kCellWarps, kCellFaces), grid, kCellWarps);
   };
-  auto faces = [&](auto kernel) { go(kernel, kFaceBatch, (int64_t)num_sms * 48, (int64_t)num_sms * 8, kMarkWarps); };
+  auto faces = [&](auto kernel) {
+    const int64_t few = m.lv.nf / ((int64_t)num_sms * 48);  // two fetches for each of 24 warps per SM
+    go(kernel, (int)std::max<int64_t>(1, std::min<int64_t>(kFaceBatch, few)), (int64_t)num_sms * 8, kMarkWarps);
+  };
   if (m.unit) {
     const bool rec = m.lv.staged != nullptr;
     if (m.lv.dim == 3)
