@@ -1647,6 +1647,9 @@ amr_status amr_classify_nodes(amr_ctx* ctx, const uint8_t** cell_solid, int64_t*
   a.level = r.n_levels - 1;
   a.g0 = ctx->geoms[0];
   a.blocks = r.block_coords[r.n_levels - 1];
+  a.n_blocks = r.n_blocks[r.n_levels - 1];
+  a.mask = r.cell_mask[r.n_levels - 1];
+  a.block_base = static_cast<const uint64_t*>(ctx->lv[r.n_levels - 1].base.p);
   a.adj_cell = r.adj_cell;
   a.row0 = 0;
   a.n_rows = n;

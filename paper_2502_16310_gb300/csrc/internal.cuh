@@ -640,6 +640,9 @@ struct ClassifyArgs {
   const int32_t* blocks;       // the finest level's blocks
   const uint32_t* adj_cell;
   int64_t row0, n_rows;
+  int64_t n_blocks;            // 3D: blocks of the level, their masks and row bases (scan of pairs | cells << 32)
+  const uint64_t* mask;
+  const uint64_t* block_base;
   const uint32_t* offsets;     // exact bins
   const void* payload;
   const float* X;              // faces (SoA), for the winding-number fallback

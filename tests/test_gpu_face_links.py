@@ -23,6 +23,7 @@ def _box(lo, hi, m):
     for axis in range(3):
         for side in (0.0, 1.0):
             q = np.insert(quad, axis, side, axis=2)
+            q = q[:, ::-1] if (axis == 1) == (side == 1.0) else q  # outward
             out += [q[:, [0, 1, 2]], q[:, [0, 2, 3]]]
     return (lo + (hi - lo) * np.concatenate(out)).astype(np.float32)
 
