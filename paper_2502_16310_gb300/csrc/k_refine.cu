@@ -437,6 +437,76 @@ __device__ __forceinline__ int point_test(const Surv<D>& S, const float* o, floa
   }
 }
 
+// Point predicate, quick test: the face's centroid c (in the frame) and the squares of the radii within which
+// a cell centre is certainly within d of the face (c is a point of it) and beyond which it certainly is not
+// (every point of the face lies within rho of c).  Stored behind setup_point's data.  False when no cell centre
+// of the block can be within d.  The radii leave 16 u (P + O) + 8 u d for the rounding of the offsets and of d.
+// A face that is small against d settles nearly every cell this way: 8 operations instead of about 100.
+// Bound by: issue slots.  3D, 112,500 faces, d = 0.05 of the domain (3 to 12 cells), masks of three levels: 10.98 ->
+// 5.50 ms per pass (88.5 million candidates, 7.3 million survivors); sampled bins and own-bin candidates 3.71 ->
+// 2.91 ms.  The separating axes (about 100 operations per face and block) are left to faces whose radius passes a
+// quarter of the block's: a smaller one leaves the sphere little that the axes could take out.
+template <int D>
+__device__ __forceinline__ bool setup_centre(const float* V, const BlockFrame<D>& F, float d, float& rho, Surv<D>& S) {
+  float p[3][3], c[3] = {0.f, 0.f, 0.f}, P = 0.f;
+#pragma unroll
+  for (int k = 0; k < D; ++k)
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+      p[k][q] = V[D * k + q] - F.Xb[q];
+      P = fmaxf(P, fabsf(p[k][q]));
+      c[q] += p[k][q];
+    }
+  float r2 = 0.f, b2 = 0.f;
+  const float box = 1.5f * F.h;  // the cell centres' box
+#pragma unroll
+  for (int q = 0; q < D; ++q) {
+    c[q] *= D == 3 ? 1.0f / 3.0f : 0.5f;
+    const float x = fmaxf(fabsf(c[q] - F.cB[q]) - box, 0.f);
+    b2 = fmaf(x, x, b2);
+  }
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < D; ++q) s = fmaf(p[k][q] - c[q], p[k][q] - c[q], s);
+    r2 = fmaxf(r2, s);
+  }
+  const float e = 16.0f * kU32 * (P + F.O) + 8.0f * kU32 * d;
+  rho = sqrtf(r2) + e;
+  const float in = fmaxf(d - e, 0.f), out = d + rho + e;
+  // squares that would leave FP32's range: within is left to point_test, beyond starts at a safe one
+  const float in2 = in > 1e-15f && in < 1e18f ? in * in * (1.0f - 8.0f * kU32) : -1.0f;
+  const float out2 = fmaxf(out * out * (1.0f + 8.0f * kU32), 1e-30f);
+  if constexpr (D == 3) {
+    S.t[10] = make_float4(c[0], c[1], c[2], out2);
+    S.t[11].x = in2;
+  } else {
+    S.t[2] = make_float4(c[0], c[1], out2, in2);
+  }
+  return b2 <= out2;
+}
+
+// 0 farther than d, 1 within d, 3 left to point_test.
+template <int D>
+__device__ __forceinline__ int quick_test(const Surv<D>& S, const float* o) {
+  float q, out2, in2;
+  if constexpr (D == 3) {
+    const float4 t = S.t[10];
+    const float x = o[0] - t.x, y = o[1] - t.y, z = o[2] - t.z;
+    q = fmaf(z, z, fmaf(y, y, x * x));
+    out2 = t.w;
+    in2 = S.t[11].x;
+  } else {
+    const float4 t = S.t[2];
+    const float x = o[0] - t.x, y = o[1] - t.y;
+    q = fmaf(y, y, x * x);
+    out2 = t.z;
+    in2 = t.w;
+  }
+  return q > out2 ? 0 : (q <= in2 ? 1 : 3);
+}
+
 struct WarpCounters {
   unsigned long long fb = 0, band = 0, cand = 0, surv = 0, big = 0;
 };
@@ -718,9 +788,17 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
           float V[D * D];
 #pragma unroll
           for (int j = 0; j < D * D; ++j) V[j] = ent.v[j];
-          surv = setup_face<D>(V, nh, F, sm.surv[lane]);
           if constexpr (kPoint) {
+            // the separating axes only for a face that is large against the block's reach
+            float rho;
+            surv = setup_centre<D>(V, F, g.d, rho, sm.surv[lane]);
+            if (surv && rho > 0.25f * F.rb) {
+              surv = setup_face<D>(V, nh, F, sm.surv[lane]);
+              if (surv) setup_centre<D>(V, F, g.d, rho, sm.surv[lane]);
+            }
             if (surv) setup_point<D>(V, nh, F, sm.surv[lane]);
+          } else {
+            surv = setup_face<D>(V, nh, F, sm.surv[lane]);
           }
           if constexpr (kOwnBin) {
             sm.surv[lane].pad[0] = ent.bin[0] | (ent.bin[1] << 16);
@@ -737,17 +815,22 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
         m &= m - 1;
         const Surv<D>& S = sm.surv[s];
         int t0 = 0, t1 = 0;
-        if (!(kMarkOnly && h0 && h1)) {
+        if constexpr (kPoint) {
+          // cells that the face can count for: the lane's own, unmarked, in the entry's bin
+          bool w0 = lane_cell && !(kMarkOnly && h0), w1 = D == 3 && !(kMarkOnly && h1);
           if constexpr (kOwnBin) {
             const uint32_t sz = D == 3 ? S.pad[1] : 0u;
-            t0 = (own0 == S.pad[0] && oz0 == sz) ? point_test<D>(S, o0, R2) : 0;
-            t1 = D == 3 && own1 == S.pad[0] && oz1 == sz ? point_test<D>(S, o1, R2) : 0;
-          } else if constexpr (kPoint) {
-            t0 = point_test<D>(S, o0, R2);
-            t1 = D == 3 ? point_test<D>(S, o1, R2) : 0;
-          } else {
-            cell_test2<D>(S, o0, o1, t0, t1);
+            w0 = w0 && own0 == S.pad[0] && oz0 == sz;
+            w1 = w1 && own1 == S.pad[0] && oz1 == sz;
           }
+          t0 = w0 ? quick_test<D>(S, o0) : 0;
+          t1 = w1 ? quick_test<D>(S, o1) : 0;
+          if (__any_sync(0xffffffffu, t0 == 3 || t1 == 3)) {
+            if (t0 == 3) t0 = point_test<D>(S, o0, R2);
+            if (t1 == 3) t1 = point_test<D>(S, o1, R2);
+          }
+        } else if (!(kMarkOnly && h0 && h1)) {
+          cell_test2<D>(S, o0, o1, t0, t1);
         }
         if constexpr (D == 3 && !kPoint) {
           for (uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h0) && t0 == 2) |
