@@ -1425,27 +1425,20 @@ __global__ void __launch_bounds__(kGroupWarps * 32, 4) k_refine_groups(RefineLev
   }
 }
 
-// Ascending sort of P keys in shared memory (P a power of two; pad the tail
-// with ~0), with a 64-bit payload per key when pay is given, by the whole warp:
-// the bitonic network, one compare-exchange per lane and pair of each stage.
-__device__ __noinline__ void warp_bitonic(uint32_t* k, uint64_t* pay, uint32_t P, int lane) {
+// Ascending sort of P keys in shared memory (P a power of two from 64 up; pad the
+// tail with ~0) by the whole warp: the bitonic network, each lane taking every
+// 32nd compare-exchange of a stage, four of them in flight.
+template <typename T>
+__device__ __noinline__ void warp_bitonic(T* k, uint32_t P, int lane) {
   for (uint32_t s = 2; s <= P; s <<= 1)
     for (uint32_t j = s >> 1; j > 0; j >>= 1) {
-      for (uint32_t i = (uint32_t)lane; i < P; i += 32) {
-        const uint32_t l = i ^ j;
-        if (l > i) {
-          const bool up = (i & s) == 0;
-          const uint32_t x = k[i], y = k[l];
-          if (up ? x > y : x < y) {
-            k[i] = y;
-            k[l] = x;
-            if (pay) {
-              const uint64_t t = pay[i];
-              pay[i] = pay[l];
-              pay[l] = t;
-            }
-          }
-        }
+#pragma unroll 4
+      for (uint32_t t = (uint32_t)lane; t < P / 2; t += 32) {
+        const uint32_t low = t & (j - 1), i = ((t - low) << 1) | low;
+        const T x = k[i], y = k[i + j];
+        const bool swap = ((i & s) == 0) == (x > y);
+        k[i] = swap ? y : x;
+        k[i + j] = swap ? x : y;
       }
       __syncwarp();
     }
@@ -1463,11 +1456,11 @@ __device__ __noinline__ void sort_cell_lists(uint32_t* adj_ids, int NC, uint32_t
     if (cnt <= 1) continue;
     uint32_t* L = adj_ids + off;
     if (cnt <= cap) {
-      uint32_t P = 32;
+      uint32_t P = 64;
       while (P < cnt) P <<= 1;
       for (uint32_t i = lane; i < P; i += 32) sf[i] = i < cnt ? L[i] : 0xffffffffu;
       __syncwarp();
-      warp_bitonic(sf, nullptr, P, lane);
+      warp_bitonic(sf, P, lane);
       for (uint32_t i = lane; i < cnt; i += 32) L[i] = sf[i];
       __syncwarp();
     } else if (lane == 0) {
@@ -1485,32 +1478,37 @@ __device__ __noinline__ void sort_cell_lists(uint32_t* adj_ids, int NC, uint32_t
   }
 }
 
-// A block's K survivor records sorted by face id into shared memory at sf (the
-// face ids; the cell masks follow them, returned), by the whole warp.
-__device__ __noinline__ const uint64_t* sort_records(const SurvRec* recs, uint32_t K, uint32_t* sf, int lane) {
+// A block's K survivor records in ascending order of face id, by the whole warp: face id and place of each in sk.
+__device__ __noinline__ void sort_records(const SurvRec* recs, uint32_t K, uint64_t* sk, int lane) {
   uint32_t P = 64;
   while (P < K) P <<= 1;
-  uint64_t* sk = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(sf) + 4 * P);
-  for (uint32_t i = lane; i < P; i += 32) {
-    if (i < K) {
-      const SurvRec r = recs[i];
-      sf[i] = r.face;
-      sk[i] = r.cells;
-    } else {
-      sf[i] = 0xffffffffu;
-      sk[i] = 0ull;
-    }
-  }
+  for (uint32_t i = lane; i < P; i += 32) sk[i] = i < K ? (uint64_t)recs[i].face << 32 | i : ~0ull;
   __syncwarp();
-  warp_bitonic(sf, sk, P, lane);
-  return sk;
+  warp_bitonic(sk, P, lane);
 }
 
-// Shared memory of a warp that a sort may use: the survivor data and the entry
-// buffers (not the mbarriers that follow them).
+// Shared memory of a warp of the adjacency's second pass: room to sort kSortRecs records (8 bytes each), over
+// which the walk's memory is laid so that only the part before its mbarriers is shared.  Bound by: the sort's chain
+// of shared memory exchanges.  2D, 4,832 blocks of about 260 records, 16.9 million pairs: 2.35 ms with room for 256
+// records (the walk's memory; blocks with more were walked again and their lists sorted one by one) -> 0.28 with
+// room for all and whole cells written side by side -> 0.14 with four exchanges in flight, the masks left in place
+// and blocks handed out singly.
+constexpr uint32_t kSortRecs = 1024;  // what the refine pass keeps of a block at most
+static_assert(kRecCap + kSpillCap <= (int)kSortRecs, "every block that kept its records is sorted");
+constexpr uint32_t kSortRegion = 8 * kSortRecs;
 template <int D>
-__host__ __device__ constexpr uint32_t sort_region_bytes() {
-  return (uint32_t)(sizeof(Surv<D>) * 32 + sizeof(typename EntryT<D>::type) * 64);
+__host__ __device__ constexpr uint32_t walk_offset() {
+  constexpr uint32_t walk = (uint32_t)(sizeof(Surv<D>) * 32 + sizeof(typename EntryT<D>::type) * 64);
+  return walk < kSortRegion ? kSortRegion - walk : 0u;
+}
+template <int D>
+__host__ __device__ constexpr uint32_t second_pass_bytes() {  // (a multiple of 16 for each warp's copies)
+  static_assert(walk_offset<D>() % 16 == 0 && sizeof(WarpSmem<D>) % 16 == 0, "16-byte aligned walk memory");
+  return walk_offset<D>() + (uint32_t)sizeof(WarpSmem<D>);
+}
+template <int D>
+__device__ __forceinline__ uint32_t* sort_area(WarpSmem<D>& sm) {
+  return reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(&sm) - walk_offset<D>());
 }
 // Largest power of two P with P keys (and P payloads of 8 bytes) in the region.
 __host__ __device__ constexpr uint32_t pow2_floor(uint32_t x) {
@@ -1625,8 +1623,7 @@ __device__ __forceinline__ void emit_block(const EmitArgs& a, unsigned blk, uint
         }
       }
     };
-    constexpr uint32_t kSortRecs = pow2_floor(sort_region_bytes<D>() / 12);  // key + payload per record
-    constexpr uint32_t kSortKeys = pow2_floor(sort_region_bytes<D>() / 4);
+    constexpr uint32_t kSortKeys = pow2_floor(kSortRegion / 4);
     if constexpr (MODE == 0) {
     if (held) {
       // the refine pass left this block's surviving faces with their cell masks:
@@ -1669,11 +1666,41 @@ __device__ __forceinline__ void emit_block(const EmitArgs& a, unsigned blk, uint
     } else {
     if (desc != ~0ull && K > (uint32_t)kRecCap && K <= kSortRecs) {
       // many records: sort them by face id in shared memory, then list the cells' faces in that order
-      uint32_t* sf = reinterpret_cast<uint32_t*>(&sm);
-      const uint64_t* sk = sort_records(a.lv.recs + rec0, K, sf, lane);
-      for (uint32_t j = 0; j < K; ++j) {
-        const uint64_t mj = sk[j];
-        put(lane < NC && ((mj >> lane) & 1ull), D == 3 && ((mj >> (lane + 32)) & 1ull), sf[j]);
+      uint64_t* sk = reinterpret_cast<uint64_t*>(sort_area<D>(sm));
+      const SurvRec* recs = a.lv.recs + rec0;
+      sort_records(recs, K, sk, lane);
+      if constexpr (D == 3) {
+        for (uint32_t j0 = 0; j0 < K; j0 += 32) {
+          const uint64_t key = j0 + lane < K ? sk[j0 + lane] : 0ull;
+          const uint64_t my = j0 + lane < K ? recs[(uint32_t)key].cells : 0ull;
+          const uint32_t n = K - j0 < 32u ? K - j0 : 32u;
+          for (uint32_t j = 0; j < n; ++j) {
+            const uint64_t mj = __shfl_sync(0xffffffffu, my, (int)j);
+            put((mj >> lane) & 1ull, (mj >> (lane + 32)) & 1ull,
+                __shfl_sync(0xffffffffu, (uint32_t)(key >> 32), (int)j));
+          }
+        }
+      } else if (__all_sync(0xffffffffu, can0)) {
+        // 32 records and one cell at a time: the cell's faces leave side by side
+        uint32_t at = (uint32_t)off0;  // (offsets are 32 bits, as adj_off holds them)
+        for (uint32_t j0 = 0; j0 < K; j0 += 32) {
+          const uint64_t key = j0 + lane < K ? sk[j0 + lane] : 0ull;
+          const uint32_t mj = j0 + lane < K ? (uint32_t)recs[(uint32_t)key].cells : 0u, fj = (uint32_t)(key >> 32);
+          uint32_t any = __reduce_or_sync(0xffffffffu, mj);
+          while (any) {
+            const int c = __ffs(any) - 1;
+            any &= any - 1;
+            const bool r = (mj >> c) & 1u;
+            const uint32_t who = __ballot_sync(0xffffffffu, r);
+            const uint32_t to = __shfl_sync(0xffffffffu, at, c);
+            const uint32_t i = to + __popc(who & ((1u << lane) - 1u));
+            if (r && (int64_t)i < a.cap_pairs) a.adj_ids[i] = fj;
+            if (lane == c) at += __popc(who);
+          }
+        }
+        c0 = at - (uint32_t)off0;
+      } else {
+        bad = true;
       }
       __syncwarp();
       if (bad || c0 != n0 || c1 != n1) atomicOr(a.lv.err, ERR_OVERFLOW);
@@ -1685,7 +1712,7 @@ __device__ __forceinline__ void emit_block(const EmitArgs& a, unsigned blk, uint
     if (bad || c0 != n0 || c1 != n1) atomicOr(a.lv.err, ERR_OVERFLOW);
     if (!__all_sync(0xffffffffu, can0 && can1)) return;  // lists beyond the capacity (reported)
     // ascending face ids per cell
-    sort_cell_lists(a.adj_ids, NC, n0, n1, off0, off1, reinterpret_cast<uint32_t*>(&sm), kSortKeys, lane);
+    sort_cell_lists(a.adj_ids, NC, n0, n1, off0, off1, sort_area<D>(sm), kSortKeys, lane);
     }
 }
 
@@ -1696,7 +1723,8 @@ __global__ void __launch_bounds__(256) k_adjacency(EmitArgs a) {
   __shared__ uint32_t s_rf[MODE == 0 ? kW : 1][kRecCap];
   extern __shared__ __align__(16) unsigned char s_raw[];  // MODE 1: the walk's per-warp memory
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  WarpSmem<D>& sm = reinterpret_cast<WarpSmem<D>*>(s_raw)[MODE == 0 ? 0 : wid];
+  WarpSmem<D>& sm = *reinterpret_cast<WarpSmem<D>*>(
+      s_raw + (MODE == 0 ? 0u : (uint32_t)wid * second_pass_bytes<D>() + walk_offset<D>()));
   uint32_t phase = 0;
   if constexpr (MODE == 1) warp_smem_init<D>(sm, lane);
   uint64_t* rm = s_rm[MODE == 0 ? wid : 0];
@@ -1705,14 +1733,17 @@ __global__ void __launch_bounds__(256) k_adjacency(EmitArgs a) {
   WarpCounters wc;
   if constexpr (MODE == 0) {
     const int64_t n = launch_count(a.lv.n_blocks, a.lv.n_dev, a.lv.err);
-    // 32 blocks per atomic: each lane reads one block's mask, the warp then takes
-    // the marked blocks of the group one after another
+    // Up to 32 blocks per atomic: each lane reads one block's mask, the warp then takes the marked blocks of the
+    // group one after another.  Fewer where every warp of the launch would not get 32 (a block costs about 1.5 us of
+    // one warp's time: 396 blocks took 0.057 ms as 13 groups of 32, 0.030 as 396 of one).
+    const int64_t share = n / ((int64_t)gridDim.x * (blockDim.x >> 5));
+    const unsigned batch = share < 1 ? 1u : (share < 32 ? (unsigned)share : 32u);
     for (;;) {
       unsigned base = 0;
-      if (lane == 0) base = atomicAdd(a.lv.work, 32u);
+      if (lane == 0) base = atomicAdd(a.lv.work, batch);
       base = __shfl_sync(0xffffffffu, base, 0);
       if (base >= n) break;
-      const bool in_range = (int64_t)base + lane < n;
+      const bool in_range = (unsigned)lane < batch && (int64_t)base + lane < n;
       const uint64_t my_mask = in_range ? a.lv.mask[base + lane] : 0ull;
       const uint32_t my_gid = in_range && a.lv.gid ? a.lv.gid[base + lane] : 0u;
       // the marked blocks' row bases and record descriptors, one coalesced load for the batch
@@ -2832,7 +2863,7 @@ int launch_adjacency(const EmitArgs& a, int num_sms, cudaStream_t st) {
   // first pass: little shared memory, so up to 64 warps per SM
   {
     const int64_t cap = (int64_t)num_sms * (64 / warps > 0 ? 64 / warps : 1);
-    int64_t g = a.lv.n_dev ? cap : (a.lv.n_blocks / 32 + warps) / warps;
+    int64_t g = a.lv.n_dev ? cap : (a.lv.n_blocks + warps - 1) / warps;
     if (g > cap) g = cap;
     if (g < 1) g = 1;
     auto go = [&](auto kernel) { kernel<<<(unsigned)g, warps * 32, 0, st>>>(a); };
@@ -2845,7 +2876,7 @@ int launch_adjacency(const EmitArgs& a, int num_sms, cudaStream_t st) {
   cudaMemsetAsync(a.lv.work, 0, sizeof(unsigned), st);
   {
     const int g = grid_warps(num_sms, 0, warps, true);
-    const size_t smem = (size_t)warps * (a.lv.dim == 3 ? sizeof(WarpSmem<3>) : sizeof(WarpSmem<2>));
+    const size_t smem = (size_t)warps * (a.lv.dim == 3 ? second_pass_bytes<3>() : second_pass_bytes<2>());
     auto go = [&](auto kernel) {
       allow_smem(kernel, smem);
       kernel<<<g, warps * 32, smem, st>>>(a);
