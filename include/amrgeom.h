@@ -353,6 +353,23 @@ AMR_API amr_status amr_batch_set_bins(amr_batch* b, int index, int bin_density);
  * want_links, use_graph, warps_per_cta (n_levels and distances are per geometry). */
 AMR_API amr_status amr_batch_run(amr_batch* b, const amr_refine_params* params, amr_refine_result* out);
 AMR_API amr_status amr_batch_get_view(amr_batch* b, int index, amr_batch_view* out);
+
+/* Copies n arrays into the caller's own in one launch per 32 of them on `stream` (a cudaStream_t, NULL = the
+ * default stream), turning batch-global indices into local ones on the way: dst[i] = src[i] - minus.  Arrays are
+ * device pointers, n elements each; `kind` names the elements.  EINVAL for an unknown kind or a negative n. */
+typedef enum {
+  AMR_COPY_8 = 1,       /* 1-byte elements, as they are (minus ignored) */
+  AMR_COPY_32 = 4,      /* 4-byte elements, as they are (minus ignored) */
+  AMR_COPY_64 = 8,      /* 8-byte elements, as they are (minus ignored) */
+  AMR_COPY_I32 = 32,    /* int32 to int32, minus subtracted */
+  AMR_COPY_I32_I64 = 64 /* int32 widened to int64, minus subtracted */
+} amr_copy_kind;
+typedef struct {
+  const void* src;
+  void* dst;
+  int64_t n, minus, kind;
+} amr_copy;
+AMR_API amr_status amr_batch_copy(amr_batch* b, const amr_copy* c, int n, void* stream);
 /* Adjoint of all links of the last run: grad_out [sum n_verts][dim] (indexed) or
  * [sum n_faces][dim][dim]; device pointers. */
 AMR_API amr_status amr_batch_q_backward(amr_batch* b, const float* grad_q, float* grad_out);

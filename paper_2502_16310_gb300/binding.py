@@ -12,6 +12,7 @@ the calls raise.
 from __future__ import annotations
 
 import ctypes as C
+import math
 import os
 import threading
 
@@ -33,7 +34,11 @@ EXPORTED = ["amr_create", "amr_destroy", "amr_status_str", "amr_last_error", "am
             "amr_timing_reset", "amr_timing_get", "amr_launch_count", "amr_bin_faces_static", "amr_q_backward",
             "amr_classify_nodes", "amr_fluid_links", "amr_adapt_diff_get", "amr_candidate_count", "amr_autotune",
             "amr_batch_create", "amr_batch_destroy", "amr_batch_add", "amr_batch_set_bins", "amr_batch_run",
-            "amr_batch_get_view", "amr_batch_q_backward", "amr_batch_last_error", "amr_batch_launch_count"]
+            "amr_batch_get_view", "amr_batch_copy", "amr_batch_q_backward", "amr_batch_last_error",
+            "amr_batch_launch_count"]
+
+# element kinds of amr_batch_copy
+AMR_COPY_8, AMR_COPY_32, AMR_COPY_64, AMR_COPY_I32, AMR_COPY_I32_I64 = 1, 4, 8, 32, 64
 
 
 class AmrError(RuntimeError):
@@ -164,6 +169,8 @@ def lib(build_if_missing: bool = True):
         L.amr_batch_run.argtypes = [P, C.POINTER(amr_refine_params), C.POINTER(amr_refine_result)]
         L.amr_batch_get_view.restype = C.c_int
         L.amr_batch_get_view.argtypes = [P, C.c_int, C.POINTER(amr_batch_view)]
+        L.amr_batch_copy.restype = C.c_int
+        L.amr_batch_copy.argtypes = [P, P, C.c_int, P]
         L.amr_batch_q_backward.restype = C.c_int
         L.amr_batch_q_backward.argtypes = [P, P, P]
         L.amr_batch_last_error.restype = C.c_char_p
@@ -382,7 +389,7 @@ class _LazyDict(dict):
 def _view(ptr, shape, dtype):
     import torch
 
-    n = int(np.prod(shape)) if len(shape) else 1
+    n = math.prod(shape)
     if n == 0 or not ptr:
         return torch.empty(tuple(shape), dtype=dtype, device="cuda")
     typestr = {torch.float32: "<f4", torch.int32: "<i4", torch.int64: "<i8", torch.uint8: "|u1"}[dtype]
@@ -719,30 +726,46 @@ class AmrBatch:
         _bcheck(self.b, lib().amr_batch_get_view(self.b, int(i), C.byref(v)))
         r, D = v.r, self.dim
         nc = 64 if D == 3 else 16
+        copies = []
+
+        def take(ptr, shape, dtype, kind, minus=0):
+            t = torch.empty(shape, dtype=dtype, device="cuda")
+            n = math.prod(shape)
+            if n and ptr:
+                copies.append((ptr, t.data_ptr(), n, minus, kind))
+            return t
+
+        def index(ptr, n, base):
+            return take(ptr, (n,), torch.int64, AMR_COPY_I32_I64, base)
+
         levels = []
         for L in range(r.n_levels):
             n = int(r.n_blocks[L])
             par = None
             if L > 0:
-                par = _view(r.block_parent[L], (n,), torch.int32).clone() - int(v.level_base[L - 1])
-            levels.append({"blocks": _view(r.block_coords[L], (n, D), torch.int32).clone(), "parent": par,
-                           "mask": _view(r.cell_mask[L], (n,), torch.int64).clone(),
-                           "flag": _view(r.block_flag[L], (n,), torch.uint8).clone()})
+                par = take(r.block_parent[L], (n,), torch.int32, AMR_COPY_I32, int(v.level_base[L - 1]))
+            levels.append({"blocks": take(r.block_coords[L], (n, D), torch.int32, AMR_COPY_32), "parent": par,
+                           "mask": take(r.cell_mask[L], (n,), torch.int64, AMR_COPY_64),
+                           "flag": take(r.block_flag[L], (n,), torch.uint8, AMR_COPY_8)})
         out = {"levels": levels}
         adj, links = self.want
         Lf = r.n_levels - 1
         if adj:
             na, npairs = int(r.n_adj_cells), int(r.n_adj_pairs)
-            out["adj_cell"] = _u32(r.adj_cell, na).long() - int(v.level_base[Lf]) * nc
-            out["adj_off"] = _u32(r.adj_off, na + 1).long() - int(v.pair_base)
-            out["adj_ids"] = _u32(r.adj_ids, npairs).long() - int(v.face_base)
+            out["adj_cell"] = index(r.adj_cell, na, int(v.level_base[Lf]) * nc)
+            out["adj_off"] = index(r.adj_off, na + 1, int(v.pair_base))
+            out["adj_ids"] = index(r.adj_ids, npairs, int(v.face_base))
         if links:
             nl = int(r.n_links)
-            out["link_cell"] = _u32(r.link_cell, nl).long() - int(v.adj_base)
-            out["link_dir"] = _view(r.link_dir, (nl,), torch.uint8).clone()
-            out["link_q"] = _view(r.link_q, (nl,), torch.float32).clone()
-            out["link_face"] = _u32(r.link_face, nl).long() - int(v.face_base)
+            out["link_cell"] = index(r.link_cell, nl, int(v.adj_base))
+            out["link_dir"] = take(r.link_dir, (nl,), torch.uint8, AMR_COPY_8)
+            out["link_q"] = take(r.link_q, (nl,), torch.float32, AMR_COPY_32)
+            out["link_face"] = index(r.link_face, nl, int(v.face_base))
         out["bases"] = {"face": int(v.face_base), "vert": int(v.vert_base), "link": int(v.link_base)}
+        if copies:
+            rows = np.array(copies, dtype=np.int64)  # the fields of amr_copy, 8 bytes each
+            _bcheck(self.b, lib().amr_batch_copy(self.b, rows.ctypes.data, len(copies),
+                                                 torch.cuda.current_stream().cuda_stream))
         return out
 
     def q_backward(self, grad_q):
