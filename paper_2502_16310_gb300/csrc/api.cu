@@ -1950,10 +1950,10 @@ __global__ void k_batch_segments(SegArgs a) {
     }
     o[L] = s;
     o[16 + L] = e - s;
-    const uint64_t tot = a.scal[SC_TOT + L];
+    const uint64_t tot = a.base[L] ? a.scal[SC_TOT + L] : 0ull;
     if (L == P.n_levels - 1) {
-      const uint64_t bs = s < n ? a.base[L][s] : tot;
-      const uint64_t be = e < n ? a.base[L][e] : tot;
+      const uint64_t bs = a.base[L] && s < n ? a.base[L][s] : tot;
+      const uint64_t be = a.base[L] && e < n ? a.base[L][e] : tot;
       o[32] = run_cells + (int64_t)(bs >> 32);
       o[33] = run_cells + (int64_t)(be >> 32);
       o[34] = run_pairs + (int64_t)(bs & 0xffffffffull);
@@ -2048,7 +2048,7 @@ amr_status batch_gather(amr_batch* b) {
   return AMR_OK;
 }
 
-amr_status batch_segments(amr_batch* b, int NL) {
+amr_status batch_segments(amr_batch* b, int NL, bool adjacency, bool links) {
   amr_ctx* ctx = &b->ctx;
   const int G = (int)ctx->geoms.size();
   DevBuf d_out;
@@ -2059,10 +2059,10 @@ amr_status batch_segments(amr_batch* b, int NL) {
   sa.scal = ctx->d_scal;
   for (int L = 0; L < NL; ++L) {
     sa.gid[L] = static_cast<const uint32_t*>(ctx->lv[L].gid.p);
-    sa.base[L] = static_cast<const uint64_t*>(ctx->lv[L].base.p);
+    sa.base[L] = adjacency ? static_cast<const uint64_t*>(ctx->lv[L].base.p) : nullptr;  // (masks only: none was made)
   }
   sa.table = static_cast<const GeomParams*>(ctx->table.p);
-  sa.link_cell = static_cast<const uint32_t*>(ctx->link_cell.p);
+  sa.link_cell = links ? static_cast<const uint32_t*>(ctx->link_cell.p) : nullptr;
   sa.out = static_cast<int64_t*>(d_out.p);
   k_batch_segments<<<(G + 63) / 64, 64, 0, ctx->stream>>>(sa);
   ctx->launches += 1;
@@ -2193,7 +2193,7 @@ amr_status amr_batch_run(amr_batch* b, const amr_refine_params* prm, amr_refine_
   TRY(amr_bin_all(ctx));
   amr_refine_result r{};
   TRY(amr_run_refine(ctx, prm, &r));
-  TRY(batch_segments(b, r.n_levels));
+  TRY(batch_segments(b, r.n_levels, prm->want_adjacency || prm->want_links, prm->want_links != 0));
   ctx->refined = true;
   ctx->last = r;
   ctx->n_links = prm->want_links ? r.n_links : -1;
