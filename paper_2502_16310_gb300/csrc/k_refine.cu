@@ -446,45 +446,107 @@ __device__ __forceinline__ int point_test(const Surv<D>& S, const float* o, floa
 // 5.50 ms per pass (88.5 million candidates, 7.3 million survivors); sampled bins and own-bin candidates 3.71 ->
 // 2.91 ms.  The separating axes (about 100 operations per face and block) are left to faces whose radius passes a
 // quarter of the block's: a smaller one leaves the sphere little that the axes could take out.
+struct FaceCentre {
+  float c[3], in2, out2, rho, P;
+};
 template <int D>
-__device__ __forceinline__ bool setup_centre(const float* V, const BlockFrame<D>& F, float d, float& rho, Surv<D>& S) {
-  float p[3][3], c[3] = {0.f, 0.f, 0.f}, P = 0.f;
+__device__ __forceinline__ FaceCentre face_centre(const float* V, const BlockFrame<D>& F, float d) {
+  FaceCentre C;
+  float p[3][3];
+  C.P = 0.f;
+  C.c[0] = C.c[1] = C.c[2] = 0.f;
 #pragma unroll
   for (int k = 0; k < D; ++k)
 #pragma unroll
     for (int q = 0; q < D; ++q) {
       p[k][q] = V[D * k + q] - F.Xb[q];
-      P = fmaxf(P, fabsf(p[k][q]));
-      c[q] += p[k][q];
+      C.P = fmaxf(C.P, fabsf(p[k][q]));
+      C.c[q] += p[k][q];
     }
-  float r2 = 0.f, b2 = 0.f;
-  const float box = 1.5f * F.h;  // the cell centres' box
+  float r2 = 0.f;
 #pragma unroll
-  for (int q = 0; q < D; ++q) {
-    c[q] *= D == 3 ? 1.0f / 3.0f : 0.5f;
-    const float x = fmaxf(fabsf(c[q] - F.cB[q]) - box, 0.f);
-    b2 = fmaf(x, x, b2);
-  }
+  for (int q = 0; q < D; ++q) C.c[q] *= D == 3 ? 1.0f / 3.0f : 0.5f;
 #pragma unroll
   for (int k = 0; k < D; ++k) {
     float s = 0.f;
 #pragma unroll
-    for (int q = 0; q < D; ++q) s = fmaf(p[k][q] - c[q], p[k][q] - c[q], s);
+    for (int q = 0; q < D; ++q) s = fmaf(p[k][q] - C.c[q], p[k][q] - C.c[q], s);
     r2 = fmaxf(r2, s);
   }
-  const float e = 16.0f * kU32 * (P + F.O) + 8.0f * kU32 * d;
-  rho = sqrtf(r2) + e;
-  const float in = fmaxf(d - e, 0.f), out = d + rho + e;
+  const float e = 16.0f * kU32 * (C.P + F.O) + 8.0f * kU32 * d;
+  C.rho = sqrtf(r2) + e;
+  const float in = fmaxf(d - e, 0.f), out = d + C.rho + e;
   // squares that would leave FP32's range: within is left to point_test, beyond starts at a safe one
-  const float in2 = in > 1e-15f && in < 1e18f ? in * in * (1.0f - 8.0f * kU32) : -1.0f;
-  const float out2 = fmaxf(out * out * (1.0f + 8.0f * kU32), 1e-30f);
-  if constexpr (D == 3) {
-    S.t[10] = make_float4(c[0], c[1], c[2], out2);
-    S.t[11].x = in2;
-  } else {
-    S.t[2] = make_float4(c[0], c[1], out2, in2);
+  C.in2 = in > 1e-15f && in < 1e18f ? in * in * (1.0f - 8.0f * kU32) : -1.0f;
+  C.out2 = fmaxf(out * out * (1.0f + 8.0f * kU32), 1e-30f);
+  return C;
+}
+
+// Squared distance from the centroid to the box ctr +- half (in the frame): beyond out2, no point of the box is
+// within d of the face.
+template <int D>
+__device__ __forceinline__ float centre_to_box2(const FaceCentre& C, const float* ctr, const float* half) {
+  float b2 = 0.f;
+#pragma unroll
+  for (int q = 0; q < D; ++q) {
+    const float x = fmaxf(fabsf(C.c[q] - ctr[q]) - half[q], 0.f);
+    b2 = fmaf(x, x, b2);
   }
-  return b2 <= out2;
+  return b2;
+}
+
+template <int D>
+__device__ __forceinline__ bool setup_centre(const float* V, const BlockFrame<D>& F, float d, float& rho, Surv<D>& S) {
+  const FaceCentre C = face_centre<D>(V, F, d);
+  rho = C.rho;
+  if constexpr (D == 3) {
+    S.t[10] = make_float4(C.c[0], C.c[1], C.c[2], C.out2);
+    S.t[11].x = C.in2;
+  } else {
+    S.t[2] = make_float4(C.c[0], C.c[1], C.out2, C.in2);
+  }
+  const float half[3] = {1.5f * F.h, 1.5f * F.h, 1.5f * F.h};  // the cell centres' box
+  return centre_to_box2<D>(C, F.cB, half) <= C.out2;
+}
+
+// A face whose bounding box or plane (line) lies certainly farther than d from the box ctr +- half: differences of
+// frame coordinates are within 4 u (P + O), their products with the normal within 32 u |n|_1 (P + O).
+template <int D>
+__device__ __forceinline__ bool face_beyond(const float* V, const float* nh, const BlockFrame<D>& F, float d, float P,
+                                            const float* ctr, const float* half) {
+  const float w = P + F.O, e = 8.0f * kU32 * (w + d);
+  bool far = false;
+  float p0[3], p1[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+  for (int q = 0; q < D; ++q) {
+    p0[q] = V[q] - F.Xb[q];
+    p1[q] = V[D + q] - F.Xb[q];
+    float lo = fminf(p0[q], p1[q]), hi = fmaxf(p0[q], p1[q]);
+    if (D == 3) {
+      const float p2 = V[2 * D + q] - F.Xb[q];
+      lo = fminf(lo, p2);
+      hi = fmaxf(hi, p2);
+    }
+    far |= lo - (ctr[q] + half[q]) > d + e || (ctr[q] - half[q]) - hi > d + e;
+  }
+  float n[3] = {nh[0], nh[1], nh[2]};
+  if (D == 2) {
+    n[0] = p0[1] - p1[1];
+    n[1] = p1[0] - p0[0];
+    n[2] = 0.f;
+  }
+  float s = 0.f, reach = 0.f, n1 = 0.f, n2 = 0.f;
+#pragma unroll
+  for (int q = 0; q < D; ++q) {
+    s = fmaf(n[q], ctr[q] - p0[q], s);
+    reach = fmaf(fabsf(n[q]), half[q], reach);
+    n1 += fabsf(n[q]);
+    n2 = fmaf(n[q], n[q], n2);
+  }
+  // (2D: the normal is a rounded difference, within 4 u w per component)
+  const float en = 32.0f * kU32 * w * (D == 3 ? n1 : n1 + w);
+  const float slab = (sqrtf(n2) * d + reach) * (1.0f + 8.0f * kU32) + en;
+  return far || (slab < 1e30f && fabsf(s) > slab);
 }
 
 // 0 farther than d, 1 within d, 3 left to point_test.
@@ -595,19 +657,6 @@ __device__ __noinline__ bool resolve_sat_warp(const RefineLevel& a, uint32_t gid
   return sep == 0u;
 }
 
-// Shared walk of one block: bins of the query box, canonical-bin dedup,
-// block-level cull, cell tests.  For every surviving face the whole warp calls
-// `on_surv(face, r0, r1)`, r0 / r1 = whether the face meets the lane's cell
-// `lane` / `lane + 32`; h0 / h1 accumulate them.  kMarkOnly: only the mask is
-// wanted, so marked cells skip further tests and the walk ends as soon as every
-// cell of the block is marked.
-//
-// The block frame is built in FP32 from the geometry row's double-float h0 and
-// origin: the block corner origin + 4 b h is formed as hi + lo (hi = the frame
-// origin, lo = its rounding error, carried into the cell and block centres),
-// so no FP64 instruction runs per block.  The bin query range is widened by
-// a margin that covers the FP32 error of the bin coordinate (a superset of
-// bins only adds candidates the block test rejects).
 // Per-warp shared memory of the walk: survivor data, a double buffer of bin
 // entries filled by TMA bulk copies with one mbarrier per buffer, and the
 // block's survivor records.
@@ -649,6 +698,116 @@ __device__ __forceinline__ void issue_chunk(const E* payload, uint32_t s, uint32
   }
 }
 
+// Mark-only walk, point predicate: the cells of a block not yet marked (bits of um) that one of the ns faces in
+// sm.surv (vertices and normal at the front of each slot) reaches; returns what is left of um.  A lane per face, one
+// cell at a time: where some face's quick test is sure the cell is done; what the quick tests leave open is queued as
+// (face, cell) pairs in the record stage, which only runs the closest-point test, 32 pairs at a time, for cells that
+// nothing else has marked by then.  Bound by: issue slots.  3D, 112,500 faces, d = 0.05 (3 to 12 cells), the two
+// walked levels: 4.92 ms one face at a time over the lanes' cells (any open cell cost the whole warp a closest-point
+// test) -> 2.68 with 32 faces at a time -> 2.20 with the bins beyond d left out and the nearest rows first (90 -> 49
+// million candidates) -> 1.79 in rows of four cells; own-bin candidates 2.46 -> 0.87 ms.
+template <int D, int PRED>
+__device__ __forceinline__ uint64_t mark_batch(const RefineLevel& a, uint32_t gid, const int* b, WarpSmem<D>& sm,
+                                               uint32_t ns, uint64_t um, const BlockFrame<D>& F, const FastGeom& g,
+                                               const float* shift, uint32_t own0, uint32_t own1, uint32_t oz0,
+                                               uint32_t oz1, int lane, WarpCounters& wc) {
+  constexpr bool kOwnBin = PRED == 2;
+  constexpr uint32_t kQueue = (sizeof(sm.rm) + sizeof(sm.rf)) / 2;
+  uint16_t* pairs = reinterpret_cast<uint16_t*>(sm.rm);
+  const float R2 = g.d * g.d;
+  FaceCentre C{};
+  uint32_t bin = 0, binz = 0;
+  const bool have = (uint32_t)lane < ns;
+  if (have) {
+    Surv<D>& S = sm.surv[lane];
+    float V[D * D], nh[3] = {0.f, 0.f, 0.f};
+    if constexpr (D == 3) {
+      const float4 v0 = S.t[0], v1 = S.t[1], v2 = S.t[2];
+      V[0] = v0.x, V[1] = v0.y, V[2] = v0.z, V[3] = v0.w, V[4] = v1.x, V[5] = v1.y, V[6] = v1.z, V[7] = v1.w, V[8] = v2.x;
+      nh[0] = v2.y, nh[1] = v2.z, nh[2] = v2.w;
+    } else {
+      const float4 v0 = S.t[0];
+      V[0] = v0.x, V[1] = v0.y, V[2] = v0.z, V[3] = v0.w;
+    }
+    C = face_centre<D>(V, F, g.d);
+    setup_point<D>(V, nh, F, S);
+    if constexpr (kOwnBin) {
+      bin = S.pad[0];
+      if constexpr (D == 3) binz = S.pad[1];
+    }
+  }
+  __syncwarp();
+  auto place = [&](int l, int c) {  // of cell l along axis c
+    const float k = (float)l + 0.5f;
+    return fmaf(k, g.h_hi, fmaf(k, g.h_lo, shift[c]));
+  };
+  float dx2[4];
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    const float dx = place(l, 0) - C.c[0];
+    dx2[l] = dx * dx;
+  }
+  uint32_t nq = 0;
+  for (uint64_t u = um; u;) {
+    // a row of four cells
+    const int row = (__ffsll((long long)u) - 1) >> 2;
+    const uint32_t cells = (uint32_t)(u >> (4 * row)) & 15u;
+    u &= ~(15ull << (4 * row));
+    const float dy = place(row & 3, 1) - C.c[1];
+    float yz = dy * dy;
+    if constexpr (D == 3) {
+      const float dz = place(row >> 2, 2) - C.c[2];
+      yz = fmaf(dz, dz, yz);
+    }
+    uint32_t done = 0;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      if (!((cells >> l) & 1u)) continue;
+      const int cell = 4 * row + l;
+      bool want = have;
+      if constexpr (kOwnBin) {
+        // (every lane takes part in the exchange)
+        const uint32_t cb = __shfl_sync(0xffffffffu, cell < 32 ? own0 : own1, cell & 31);
+        const uint32_t cz = D == 3 ? __shfl_sync(0xffffffffu, cell < 32 ? oz0 : oz1, cell & 31) : 0u;
+        want = want && bin == cb && binz == cz;
+      }
+      const float q = yz + dx2[l];
+      if (__any_sync(0xffffffffu, want && q <= C.in2)) {
+        done |= 1u << l;
+      } else {
+        const bool open = want && !(q > C.out2);
+        const unsigned ob = __ballot_sync(0xffffffffu, open);
+        if (open) pairs[nq + __popc(ob & ((1u << lane) - 1u))] = (uint16_t)(lane | cell << 5);
+        nq += __popc(ob);
+      }
+    }
+    um &= ~((uint64_t)done << (4 * row));
+    if (nq > kQueue - 128u || !u) {
+      __syncwarp();
+      for (uint32_t q0 = 0; q0 < nq; q0 += 32) {
+        const uint32_t e = q0 + lane < nq ? pairs[q0 + lane] : 0u;
+        const int c = (int)(e >> 5);
+        int t = 0;
+        if (q0 + lane < nq && ((um >> c) & 1ull)) {
+          const Surv<D>& S = sm.surv[e & 31u];
+          float x[3];
+#pragma unroll
+          for (int k = 0; k < D; ++k) x[k] = place((c >> (2 * k)) & 3, k);
+          t = point_test<D>(S, x, R2);
+          if (t == 2) t = resolve_fp64<D>(a, gid, S.face, b, c, &wc.fb, &wc.band) ? 1 : 0;
+        }
+        const uint32_t lo = __reduce_or_sync(0xffffffffu, t && c < 32 ? 1u << c : 0u);
+        const uint32_t hi = D == 3 ? __reduce_or_sync(0xffffffffu, t && c >= 32 ? 1u << (c - 32) : 0u) : 0u;
+        um &= ~((uint64_t)hi << 32 | lo);
+      }
+      nq = 0;
+      u &= um;
+      __syncwarp();
+    }
+  }
+  return um;
+}
+
 // Shared walk of one block: bins of the query box, canonical-bin dedup,
 // block-level cull, cell tests.  For every surviving face the whole warp calls
 // `on_surv(face, r0, r1)`, r0 / r1 = whether the face meets the lane's cell
@@ -667,6 +826,7 @@ __device__ __forceinline__ void issue_chunk(const E* payload, uint32_t s, uint32
 // row); entries then arrive in shared memory by TMA bulk copies in chunks of
 // 32, double-buffered: the next chunk is requested before the warp tests the
 // current one.
+constexpr uint32_t kFirstBatch = 8;  // faces of a block's first mark_batch
 template <int D, int PRED, bool kMarkOnly, typename OnSurv>
 __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParams& P, uint32_t gid, const int* b,
                                            WarpSmem<D>& sm, uint32_t& phase, int lane, WarpCounters& wc, bool& h0,
@@ -740,19 +900,74 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
       o1[c] = fmaf(l1, g.h_hi, fmaf(l1, g.h_lo, shift[c]));
     }
   }
+  // marks of the point predicate: the unmarked cells, their centres' box, the faces gathered for mark_batch
+  constexpr bool kMarkPoint = kPoint && kMarkOnly;
+  uint64_t um = D == 3 ? ~0ull : 0xffffull;
+  float ctr[3] = {F.cB[0], F.cB[1], D == 3 ? F.cB[D - 1] : 0.f}, half[3] = {1.5f * hf, 1.5f * hf, 1.5f * hf};
+  uint32_t ns = 0, most = kFirstBatch;
   const int64_t B = Bn;
   const E* payload = static_cast<const E*>(a.payload);
-  const int nx = qhi[0] - qlo[0] + 1, ny = qhi[1] - qlo[1] + 1;
+  constexpr bool kTrim = kMarkPoint && !kOwnBin;  // (marks: a face may come twice)
+  const int ny = qhi[1] - qlo[1] + 1;
+  [[maybe_unused]] float bc[3] = {0.f, 0.f, 0.f};  // block centre relative to the domain's origin
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    const float k = (float)(4 * b[c] + 2);
+    bc[c] = fmaf(k, g.h_hi, k * g.h_lo);
+  }
   const int nrows = ny * (D == 3 ? qhi[2] - qlo[2] + 1 : 1);
   for (int rg = 0; rg < nrows; rg += 32) {
     // this group's rows: one lane each
     uint32_t rs = 0, rn = 0;
     const int ri = rg + lane;
+    float far2 = 0.f;  // a row's distance from the block's centre, squared
     if (ri < nrows) {
       const int y = qlo[1] + ri % ny, z = D == 3 ? qlo[2] + ri / ny : 0;
-      const int64_t b0 = P.bin_base + qlo[0] + B * (y + B * (int64_t)z);
-      rs = a.offsets[b0];
-      rn = a.offsets[b0 + nx] - rs;
+      int x0 = qlo[0], x1 = qhi[0];
+      if constexpr (kTrim) {
+        // the bins within d of the cell centres' box: a face that reaches a centre has its nearest point in one of
+        // them (bins at the domain's sides go on outside it); margins in bins as above
+        float left2 = g.d * g.d * (1.0f + 1e-4f);
+#pragma unroll
+        for (int c = 1; c < D; ++c) {
+          const int i = c == 1 ? y : z;
+          const float inv = 1.0f / P.scale32[c];
+          const float lo = i == 0 ? -INFINITY : ((float)i - margin) * inv;
+          const float hi = i == Bn - 1 ? INFINITY : ((float)(i + 1) + margin) * inv;
+          const float gap = fmaxf(0.f, fmaxf(lo - bc[c] - 1.5f * hf, bc[c] - 1.5f * hf - hi));
+          left2 -= gap * gap;
+          const float off = ((float)i + 0.5f) * inv - bc[c];
+          far2 = fmaf(off, off, far2);
+        }
+        if (left2 < 0.f) {
+          x1 = x0 - 1;
+        } else {
+          const float reach = sqrtf(left2) * (1.0f + 1e-4f) + 1.5f * hf;
+          const float tl = floorf((bc[0] - reach) * P.scale32[0] - margin);
+          const float th = floorf((bc[0] + reach) * P.scale32[0] + margin);
+          x0 = max(x0, tl > (float)(Bn - 1) ? Bn - 1 : (int)fmaxf(tl, 0.f));
+          x1 = min(x1, th < 0.f ? 0 : (int)fminf(th, (float)(Bn - 1)));
+        }
+      }
+      if (!kTrim || x1 >= x0) {
+        const int64_t b0 = P.bin_base + x0 + B * (y + B * (int64_t)z);
+        rs = a.offsets[b0];
+        rn = a.offsets[b0 + (x1 - x0 + 1)] - rs;
+      }
+    }
+    if constexpr (kTrim) {
+      // the nearest rows first: a face close to the block marks all of it and ends the walk
+      const float key = rn ? far2 : INFINITY;
+      const int n = nrows - rg < 32 ? nrows - rg : 32;
+      int rank = 0, src = lane;
+      for (int i = 0; i < n; ++i) {
+        const float k = __shfl_sync(0xffffffffu, key, i);
+        rank += k < key || (k == key && i < lane) ? 1 : 0;
+      }
+      for (int i = 0; i < n; ++i)
+        if (__shfl_sync(0xffffffffu, rank, i) == lane) src = i;
+      rs = __shfl_sync(0xffffffffu, rs, src);
+      rn = __shfl_sync(0xffffffffu, rn, src);
     }
     const uint32_t incl = warp_inclusive_scan<uint32_t>(rn);
     const uint32_t T = __shfl_sync(0xffffffffu, incl, 31);
@@ -776,8 +991,8 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
         bool canon = kOwnBin || ((id >> 29) & 1u) || (int)ent.bin[0] == qlo[0];
         canon = canon && (kOwnBin || ((id >> 30) & 1u) || (int)ent.bin[1] == qlo[1]);
         if (D == 3) canon = canon && (kOwnBin || ((id >> 31) & 1u) || (int)ent.bin[2] == qlo[2]);
-        if (canon) {
-          wc.cand++;
+        wc.cand += canon ? 1u : 0u;
+        if (kTrim || canon) {
           const uint32_t f = id & kIdMask;
           float nh[3] = {0.f, 0.f, 0.f};
           if constexpr (D == 3) {
@@ -788,7 +1003,11 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
           float V[D * D];
 #pragma unroll
           for (int j = 0; j < D * D; ++j) V[j] = ent.v[j];
-          if constexpr (kPoint) {
+          if constexpr (kMarkPoint) {
+            const FaceCentre C = face_centre<D>(V, F, g.d);
+            surv = centre_to_box2<D>(C, ctr, half) <= C.out2;
+            if (surv && C.rho > 0.25f * F.rb) surv = !face_beyond<D>(V, nh, F, g.d, C.P, ctr, half);
+          } else if constexpr (kPoint) {
             // the separating axes only for a face that is large against the block's reach
             float rho;
             surv = setup_centre<D>(V, F, g.d, rho, sm.surv[lane]);
@@ -800,13 +1019,68 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
           } else {
             surv = setup_face<D>(V, nh, F, sm.surv[lane]);
           }
-          if constexpr (kOwnBin) {
-            sm.surv[lane].pad[0] = ent.bin[0] | (ent.bin[1] << 16);
-            if constexpr (D == 3) sm.surv[lane].pad[1] = ent.bin[2];
+          if constexpr (!kMarkPoint) {
+            if constexpr (kOwnBin) {
+              sm.surv[lane].pad[0] = ent.bin[0] | (ent.bin[1] << 16);
+              if constexpr (D == 3) sm.surv[lane].pad[1] = ent.bin[2];
+            }
+            sm.surv[lane].face = f;
           }
-          sm.surv[lane].face = f;
         }
       }
+      if constexpr (kMarkPoint) {
+        // survivors into the free slots; a full set (a small one at first: near faces settle whole blocks) is worked off
+        unsigned left = __ballot_sync(0xffffffffu, surv);
+        wc.surv += __popc(left);
+        while (left || (!more && ns)) {
+          const uint32_t at = ns + __popc(left & ((1u << lane) - 1u));
+          const bool put = ((left >> lane) & 1u) && at < 32u;
+          if (put) {
+            const E& ent = sm.buf[cb][lane];
+            Surv<D>& S = sm.surv[at];
+            S.t[0] = make_float4(ent.v[0], ent.v[1], ent.v[2], ent.v[3]);
+            if constexpr (D == 3) {
+              S.t[1] = make_float4(ent.v[4], ent.v[5], ent.v[6], ent.v[7]);
+              S.t[2] = make_float4(ent.v[8], ent.n[0], ent.n[1], ent.n[2]);
+            }
+            if constexpr (kOwnBin) {
+              S.pad[0] = ent.bin[0] | (ent.bin[1] << 16);
+              if constexpr (D == 3) S.pad[1] = ent.bin[2];
+            }
+            S.face = ent.id & kIdMask;
+          }
+          const unsigned got = __ballot_sync(0xffffffffu, put);
+          left &= ~got;
+          ns += __popc(got);
+          __syncwarp();
+          if (ns < most && more) continue;
+          um = mark_batch<D, PRED>(a, gid, b, sm, ns, um, F, g, shift, own0, own1, oz0, oz1, lane, wc);
+          ns = 0;
+          most = 32u;
+          if (!um) break;
+          // the box of the cells that are left
+          auto span = [&](uint32_t any, int c) {  // any: 4 bits, one per cell coordinate
+            const float lo = (float)(__ffs(any) - 1), hi = (float)(31 - __clz(any));
+            ctr[c] = fmaf(0.5f * (lo + hi + 1.0f), g.h_hi, shift[c]);
+            half[c] = 0.5f * (hi - lo) * g.h_hi;
+          };
+          const uint64_t pz = um | um >> 32, pl = pz | pz >> 16;      // over z
+          const uint32_t xy = (uint32_t)pl & 0xffffu, x2 = xy | xy >> 8;
+          span((x2 | x2 >> 4) & 15u, 0);
+          uint32_t any = 0;
+#pragma unroll
+          for (int l = 0; l < 4; ++l) any |= ((xy >> (4 * l)) & 15u) ? 1u << l : 0u;
+          span(any, 1);
+          if constexpr (D == 3) {
+            any = 0;
+#pragma unroll
+            for (int l = 0; l < 4; ++l) any |= ((um >> (16 * l)) & 0xffffull) ? 1u << l : 0u;
+            span(any, 2);
+          }
+        }
+        h0 = !((um >> lane) & 1ull) && lane_cell;
+        h1 = D == 3 && !((um >> (lane + 32)) & 1ull);
+      } else {
       unsigned m = __ballot_sync(0xffffffffu, surv);
       __syncwarp();
       wc.surv += __popc(m);
@@ -859,6 +1133,7 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
         h0 |= r0;
         h1 |= r1;
         on_surv(S.face, r0, r1);
+      }
       }
       __syncwarp();
       // marking only: once every cell of the block is marked, the rest of the walk cannot change the mask
@@ -926,7 +1201,9 @@ __device__ __forceinline__ void store_records(const RefineLevel& a, WarpSmem<D>&
   __syncwarp();
 }
 
-template <int D, int PRED>
+// ENDS: 0 no geometry of the launch ends at this level, 1 all do, 2 some may (the point predicate's two walks share
+// no code: one kernel with both held 112 registers, and the walk that keeps records took 0.386 instead of 0.341 ms).
+template <int D, int PRED, int ENDS>
 __global__ void __launch_bounds__(256) k_refine(RefineLevel a) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   WarpSmem<D>& sm = reinterpret_cast<WarpSmem<D>*>(s_raw)[threadIdx.x >> 5];
@@ -957,11 +1234,12 @@ __global__ void __launch_bounds__(256) k_refine(RefineLevel a) {
     const uint32_t gid = __shfl_sync(0xffffffffu, gv, q);
     const GeomParams& P = a.table ? a.table[gid] : a.g0;
     // per-cell face counts and survivor records only where the block's geometry ends here
-    const bool fin = a.blockcnt && a.level == P.n_levels - 1;
+    const bool fin = ENDS == 2 ? a.blockcnt && a.level == P.n_levels - 1 : ENDS == 1;
     if (a.skip_mark_only && ((P.face_levels >> a.level) & 1u)) continue;  // marked face by face
     uint32_t cnt0 = 0, cnt1 = 0;
     bool h0 = false, h1 = false;
-    if (fin) {
+    if (ENDS == 1 || (ENDS == 2 && fin)) {
+      if constexpr (ENDS != 0) {
       uint32_t K = 0;  // records of this block (warp-uniform); past kRecCap into the warp's spill area
       walk_block<D, PRED, false>(a, P, gid, b, sm, phase, lane, wc, h0, h1, [&](uint32_t f, bool r0, bool r1) {
         cnt0 += r0 ? 1u : 0u;
@@ -986,7 +1264,8 @@ __global__ void __launch_bounds__(256) k_refine(RefineLevel a) {
         if (K > (uint32_t)kRecCap) wc.big += 1;
         store_records<D>(a, sm, K, blk, lane);
       }
-    } else {
+      }
+    } else if constexpr (ENDS != 1) {
       walk_block<D, PRED, true>(a, P, gid, b, sm, phase, lane, wc, h0, h1, [](uint32_t, bool, bool) {});
       cnt0 = h0 ? 1u : 0u;
       cnt1 = h1 ? 1u : 0u;
@@ -2849,10 +3128,24 @@ int launch_refine(const RefineLevel& a, int num_sms, cudaStream_t st) {
     k_refine_groups<<<gg, kGroupWarps * 32, gsm, st>>>(a);
     return 1;
   }
-  if (a.dim == 3)
-    mode == 2 ? go(k_refine<3, 2>) : (mode == 1 ? go(k_refine<3, 1>) : go(k_refine<3, 0>));
-  else
-    mode == 2 ? go(k_refine<2, 2>) : (mode == 1 ? go(k_refine<2, 1>) : go(k_refine<2, 0>));
+  // one geometry: every block ends here or none does
+  const int ends = mode == 0 ? 2 : (!a.blockcnt ? 0 : (a.table ? 2 : 1));
+  auto pick = [&](auto k0, auto k1, auto k2) { ends == 0 ? go(k0) : (ends == 1 ? go(k1) : go(k2)); };
+  if (a.dim == 3) {
+    if (mode == 2)
+      pick(k_refine<3, 2, 0>, k_refine<3, 2, 1>, k_refine<3, 2, 2>);
+    else if (mode == 1)
+      pick(k_refine<3, 1, 0>, k_refine<3, 1, 1>, k_refine<3, 1, 2>);
+    else
+      go(k_refine<3, 0, 2>);
+  } else {
+    if (mode == 2)
+      pick(k_refine<2, 2, 0>, k_refine<2, 2, 1>, k_refine<2, 2, 2>);
+    else if (mode == 1)
+      pick(k_refine<2, 1, 0>, k_refine<2, 1, 1>, k_refine<2, 1, 2>);
+    else
+      go(k_refine<2, 0, 2>);
+  }
   return 1;
 }
 
