@@ -130,6 +130,7 @@ struct amr_ctx {
   unsigned* d_work = nullptr;
   uint64_t* d_tot = nullptr;
   DevBuf fstat;                           // per geometry: face-size statistics (see FaceBinArgs)
+  DevBuf spheres;                         // per bin entry (marks of the 3D point predicate)
   DevBuf spill;                           // per-warp spill of survivor records (once a call needed it)
   DevBuf calg;                            // per-level algorithmic test counts (amr_candidate_count)
   DevBuf defer;                           // the adjacency's second-pass block list
@@ -530,7 +531,7 @@ void amr_ctx_free(amr_ctx* ctx) {
                    &ctx->grad_face, &ctx->sort_scratch, &ctx->group_cnt,  &ctx->lvl_ptrs,   &ctx->table,
                    &ctx->hit_q,     &ctx->hit_code,     &ctx->run_staged, &ctx->runs,       &ctx->grp_runs,   &ctx->grp_first,
                    &ctx->grp_links, &ctx->grp_base,
-                   &ctx->face_gid,  &ctx->fstat,        &ctx->spill,      &ctx->calg,       &ctx->defer};
+                   &ctx->face_gid,  &ctx->fstat,        &ctx->spill,      &ctx->calg,       &ctx->defer,      &ctx->spheres};
   for (DevBuf* b : all) release(ctx, *b);
   for (int L = 0; L < AMR_MAX_LEVELS; ++L) {
     LevelBufs& l = ctx->lv[L];
@@ -783,6 +784,7 @@ RefineLevel level_args(amr_ctx* ctx, const Plan& P, int L) {
   a.n_dev = ctx->d_scal + SC_N + L;
   a.offsets = static_cast<const uint32_t*>(ctx->offsets.p);
   a.payload = ctx->payload.p;
+  a.spheres = static_cast<const float4*>(ctx->spheres.p);
   a.X = static_cast<const float*>(ctx->X.p);
   a.nrm = static_cast<const float*>(ctx->nrm.p);
   a.nf = ctx->nf;
@@ -846,6 +848,17 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
     k_set_u64<<<1, 1, 0, st>>>(ctx->d_scal + SC_N, (uint64_t)N0);
     return k + 1;
   });
+  bool spheres = false;  // some block is walked for its mask only by the 3D point predicate
+  for (int L = 0; L < P.NL; ++L)
+    spheres |= D == 3 && P.pred == AMR_PRED_POINT && P.search == AMR_SEARCH_QUERY_BOX && P.walk_at[L] &&
+               (P.cont_after[L] || !P.adjacency);
+  if (spheres) {
+    if (eager) TRY(ensure(ctx, ctx->spheres, ctx->payload.cap / sizeof(Entry3) * sizeof(float4)));
+    timed(ctx, st, "entry_spheres", [&] {
+      return launch_entry_spheres(ctx->payload.p, static_cast<const uint32_t*>(ctx->offsets.p) + ctx->n_bins,
+                                  static_cast<float4*>(ctx->spheres.p), ctx->num_sms, st);
+    });
+  }
   int64_t N = N0;
   for (int L = 0; L < P.NL; ++L) {
     LevelBufs& lb = ctx->lv[L];

@@ -514,6 +514,7 @@ struct RefineLevel {
   const uint64_t* n_dev;       // device block count (nullable)
   const uint32_t* offsets;
   const void* payload;
+  const float4* spheres;       // per bin entry, 3D point predicate with mark-only blocks (launch_entry_spheres)
   const float* X;
   const float* nrm;
   int64_t nf;
@@ -540,6 +541,8 @@ struct RefineLevel {
 };
 constexpr int kMaxBatch = 8;
 int launch_refine(const RefineLevel& a, int num_sms, cudaStream_t st);
+// Spheres about the faces of all bin entries (their number on the device).
+int launch_entry_spheres(const void* payload, const uint32_t* n_entries, float4* out, int num_sms, cudaStream_t st);
 // Levels that launch_refine marks by parent groups (one warp per marked parent's 8
 // children): 3D box predicate, whole-query-box search, below the roots.  The
 // finest such level then always stages survivor records past shared memory in

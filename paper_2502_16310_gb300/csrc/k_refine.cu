@@ -698,14 +698,15 @@ __device__ __forceinline__ void issue_chunk(const E* payload, uint32_t s, uint32
   }
 }
 
-// Mark-only walk, point predicate: the cells of a block not yet marked (bits of um) that one of the ns faces in
-// sm.surv (vertices and normal at the front of each slot) reaches; returns what is left of um.  A lane per face, one
-// cell at a time: where some face's quick test is sure the cell is done; what the quick tests leave open is queued as
-// (face, cell) pairs in the record stage, which only runs the closest-point test, 32 pairs at a time, for cells that
-// nothing else has marked by then.  Bound by: issue slots.  3D, 112,500 faces, d = 0.05 (3 to 12 cells), the two
+// Mark-only walk, point predicate: the cells of a block not yet marked (bits of um) that one of the ns faces which
+// the warp gathered reaches (3D query box: their entries, listed in the entry buffer; else vertices at the front of
+// the slots); returns what is left of um.  A lane per face, a row of four cells at a time: where some face's quick
+// test is sure the cell is done; what the quick tests leave open is queued as (face, cell) pairs in the record stage,
+// which only runs the closest-point test, 32 pairs at a time, for cells that nothing else has marked by then.
+// Bound by: issue slots, at 16 warps per SM (128 registers).  3D, 112,500 faces, d = 0.05 (3 to 12 cells), the two
 // walked levels: 4.92 ms one face at a time over the lanes' cells (any open cell cost the whole warp a closest-point
 // test) -> 2.68 with 32 faces at a time -> 2.20 with the bins beyond d left out and the nearest rows first (90 -> 49
-// million candidates) -> 1.79 in rows of four cells; own-bin candidates 2.46 -> 0.87 ms.
+// million candidates) -> 1.79 in rows of four cells -> 1.57 with the cull by spheres; own-bin candidates 2.46 -> 0.87.
 template <int D, int PRED>
 __device__ __forceinline__ uint64_t mark_batch(const RefineLevel& a, uint32_t gid, const int* b, WarpSmem<D>& sm,
                                                uint32_t ns, uint64_t um, const BlockFrame<D>& F, const FastGeom& g,
@@ -721,20 +722,23 @@ __device__ __forceinline__ uint64_t mark_batch(const RefineLevel& a, uint32_t gi
   if (have) {
     Surv<D>& S = sm.surv[lane];
     float V[D * D], nh[3] = {0.f, 0.f, 0.f};
-    if constexpr (D == 3) {
-      const float4 v0 = S.t[0], v1 = S.t[1], v2 = S.t[2];
-      V[0] = v0.x, V[1] = v0.y, V[2] = v0.z, V[3] = v0.w, V[4] = v1.x, V[5] = v1.y, V[6] = v1.z, V[7] = v1.w, V[8] = v2.x;
-      nh[0] = v2.y, nh[1] = v2.z, nh[2] = v2.w;
+    float4 v0 = S.t[0], v1{}, v2{};
+    if constexpr (D == 3 && !kOwnBin) {
+      const float4* E = static_cast<const float4*>(a.payload) + 4ull * reinterpret_cast<const uint32_t*>(sm.buf)[lane];
+      v0 = __ldg(E), v1 = __ldg(E + 1), v2 = __ldg(E + 2);
+      S.face = __float_as_uint(__ldg(E + 3).x) & kIdMask;
     } else {
-      const float4 v0 = S.t[0];
-      V[0] = v0.x, V[1] = v0.y, V[2] = v0.z, V[3] = v0.w;
+      if constexpr (D == 3) v1 = S.t[1], v2 = S.t[2];
+      if constexpr (kOwnBin) bin = S.pad[0];
+      if constexpr (kOwnBin && D == 3) binz = S.pad[1];
+    }
+    V[0] = v0.x, V[1] = v0.y, V[2] = v0.z, V[3] = v0.w;
+    if constexpr (D == 3) {
+      V[4] = v1.x, V[5] = v1.y, V[6] = v1.z, V[7] = v1.w, V[8] = v2.x;
+      nh[0] = v2.y, nh[1] = v2.z, nh[2] = v2.w;
     }
     C = face_centre<D>(V, F, g.d);
     setup_point<D>(V, nh, F, S);
-    if constexpr (kOwnBin) {
-      bin = S.pad[0];
-      if constexpr (D == 3) binz = S.pad[1];
-    }
   }
   __syncwarp();
   auto place = [&](int l, int c) {  // of cell l along axis c
@@ -907,6 +911,7 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
   uint32_t ns = 0, most = kFirstBatch;
   const int64_t B = Bn;
   const E* payload = static_cast<const E*>(a.payload);
+  constexpr bool kSpheres = kMarkPoint && D == 3 && !kOwnBin;  // (own bin: most candidates stay, 1.38 / 1.40 ms)
   constexpr bool kTrim = kMarkPoint && !kOwnBin;  // (marks: a face may come twice)
   const int ny = qhi[1] - qlo[1] + 1;
   [[maybe_unused]] float bc[3] = {0.f, 0.f, 0.f};  // block centre relative to the domain's origin
@@ -916,6 +921,32 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
     bc[c] = fmaf(k, g.h_hi, k * g.h_lo);
   }
   const int nrows = ny * (D == 3 ? qhi[2] - qlo[2] + 1 : 1);
+  // the gathered faces against the unmarked cells; then the box of those that are left
+  [[maybe_unused]] auto work_off = [&]() {
+    um = mark_batch<D, PRED>(a, gid, b, sm, ns, um, F, g, shift, own0, own1, oz0, oz1, lane, wc);
+    ns = 0;
+    most = 32u;
+    if (!um) return;
+    // the box of the cells that are left
+    auto span = [&](uint32_t any, int c) {  // any: 4 bits, one per cell coordinate
+      const float lo = (float)(__ffs(any) - 1), hi = (float)(31 - __clz(any));
+      ctr[c] = fmaf(0.5f * (lo + hi + 1.0f), g.h_hi, shift[c]);
+      half[c] = 0.5f * (hi - lo) * g.h_hi;
+    };
+    const uint64_t pz = um | um >> 32, pl = pz | pz >> 16;      // over z
+    const uint32_t xy = (uint32_t)pl & 0xffffu, x2 = xy | xy >> 8;
+    span((x2 | x2 >> 4) & 15u, 0);
+    uint32_t any = 0;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) any |= ((xy >> (4 * l)) & 15u) ? 1u << l : 0u;
+    span(any, 1);
+    if constexpr (D == 3) {
+      any = 0;
+#pragma unroll
+      for (int l = 0; l < 4; ++l) any |= ((um >> (16 * l)) & 0xffffull) ? 1u << l : 0u;
+      span(any, 2);
+    }
+  };
   for (int rg = 0; rg < nrows; rg += 32) {
     // this group's rows: one lane each
     uint32_t rs = 0, rn = 0;
@@ -974,6 +1005,64 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
     const uint32_t rv = incl - rn;
     const uint32_t nch = (T + 31u) / 32u;
     if (nch == 0) continue;
+    if constexpr (kSpheres) {
+      uint32_t* list = reinterpret_cast<uint32_t*>(sm.buf);
+      // the group's item k: the last row that starts at or before it, and its place there
+      auto entry_of = [&](uint32_t k) {
+        int l = 0;
+#pragma unroll
+        for (int st = 16; st > 0; st >>= 1)
+          if (__shfl_sync(0xffffffffu, rv, l + st) <= k) l += st;
+        return __shfl_sync(0xffffffffu, rs, l) + k - __shfl_sync(0xffffffffu, rv, l);
+      };
+      uint32_t e = entry_of((uint32_t)lane);
+      float4 ball = (uint32_t)lane < T ? __ldg(a.spheres + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (uint32_t c = 0; c < nch; ++c) {
+        const bool more = c + 1 < nch;
+        const uint32_t e1 = entry_of(32u * (c + 1) + lane);
+        const float4 ball1 = 32u * (c + 1) + lane < T ? __ldg(a.spheres + e1) : make_float4(0.f, 0.f, 0.f, 0.f);
+        bool surv = false;
+        if (32u * c + lane < T) {
+          wc.cand++;
+          FaceCentre C;
+          C.c[0] = ball.x - F.Xb[0], C.c[1] = ball.y - F.Xb[1], C.c[2] = ball.z - F.Xb[2];
+          const float m = fmaxf(fmaxf(fabsf(C.c[0]), fabsf(C.c[1])), fabsf(C.c[2]));
+          const float out = g.d + ball.w + 16.0f * kU32 * (m + F.O) + 8.0f * kU32 * g.d;
+          surv = centre_to_box2<D>(C, ctr, half) <= fmaxf(out * out * (1.0f + 8.0f * kU32), 1e-30f);
+          if (surv && ball.w > 0.25f * F.rb) {
+            const E& ent = payload[e];
+            float V[9], nh[3];
+#pragma unroll
+            for (int j = 0; j < 9; ++j) V[j] = ent.v[j];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) nh[j] = ent.n[j];
+            surv = !face_beyond<D>(V, nh, F, g.d, m + 2.0f * ball.w, ctr, half);
+          }
+        }
+        unsigned left = __ballot_sync(0xffffffffu, surv);
+        wc.surv += __popc(left);
+        // into the free places; a full list (a short one at first: near faces settle whole blocks) is worked off
+        while (left || (!more && ns)) {
+          const uint32_t at = ns + __popc(left & ((1u << lane) - 1u));
+          const bool put = ((left >> lane) & 1u) && at < 32u;
+          if (put) list[at] = e;
+          const unsigned got = __ballot_sync(0xffffffffu, put);
+          left &= ~got;
+          ns += __popc(got);
+          __syncwarp();
+          if (ns < most && more) continue;
+          work_off();
+          if (!um) break;
+        }
+        if (!um) break;
+        e = e1;
+        ball = ball1;
+      }
+      h0 = !((um >> lane) & 1ull);
+      h1 = !((um >> (lane + 32)) & 1ull);
+      if (!um) return;
+      continue;
+    }
     int cb = 0;
     issue_chunk<E>(payload, rs, rn, rv, 0u, T, sm.buf[0], &sm.bar[0], lane);
     for (uint32_t c = 0; c < nch; ++c) {
@@ -1028,7 +1117,7 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
           }
         }
       }
-      if constexpr (kMarkPoint) {
+      if constexpr (kMarkPoint && !kSpheres) {
         // survivors into the free slots; a full set (a small one at first: near faces settle whole blocks) is worked off
         unsigned left = __ballot_sync(0xffffffffu, surv);
         wc.surv += __popc(left);
@@ -1054,29 +1143,8 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
           ns += __popc(got);
           __syncwarp();
           if (ns < most && more) continue;
-          um = mark_batch<D, PRED>(a, gid, b, sm, ns, um, F, g, shift, own0, own1, oz0, oz1, lane, wc);
-          ns = 0;
-          most = 32u;
+          work_off();
           if (!um) break;
-          // the box of the cells that are left
-          auto span = [&](uint32_t any, int c) {  // any: 4 bits, one per cell coordinate
-            const float lo = (float)(__ffs(any) - 1), hi = (float)(31 - __clz(any));
-            ctr[c] = fmaf(0.5f * (lo + hi + 1.0f), g.h_hi, shift[c]);
-            half[c] = 0.5f * (hi - lo) * g.h_hi;
-          };
-          const uint64_t pz = um | um >> 32, pl = pz | pz >> 16;      // over z
-          const uint32_t xy = (uint32_t)pl & 0xffffu, x2 = xy | xy >> 8;
-          span((x2 | x2 >> 4) & 15u, 0);
-          uint32_t any = 0;
-#pragma unroll
-          for (int l = 0; l < 4; ++l) any |= ((xy >> (4 * l)) & 15u) ? 1u << l : 0u;
-          span(any, 1);
-          if constexpr (D == 3) {
-            any = 0;
-#pragma unroll
-            for (int l = 0; l < 4; ++l) any |= ((um >> (16 * l)) & 0xffffull) ? 1u << l : 0u;
-            span(any, 2);
-          }
         }
         h0 = !((um >> lane) & 1ull) && lane_cell;
         h1 = D == 3 && !((um >> (lane + 32)) & 1ull);
@@ -1199,6 +1267,34 @@ __device__ __forceinline__ void store_records(const RefineLevel& a, WarpSmem<D>&
   }
   if (lane == 0) a.rec_desc[blk] = K == 0 ? 0ull : (base == ~0ull ? ~0ull : (base << kInfoShift) | K);
   __syncwarp();
+}
+
+// A sphere about every bin entry's face, in bin order: centroid (rounded; the radius is taken from the rounded one)
+// and a radius that covers the face.  The marks of the point predicate cull by it: 16 bytes and 15 operations per
+// candidate instead of the entry's 64 (read with bank conflicts) and about 90.  112,500 faces: built in
+// 7.5 us, and a pass of 2.36 ms took 2.17.
+__global__ void __launch_bounds__(256) k_entry_spheres(const Entry3* __restrict__ entries, const uint32_t* n_entries,
+                                                       float4* __restrict__ out) {
+  const uint32_t n = *n_entries;
+  for (uint64_t i = blockIdx.x * 256ull + threadIdx.x; i < n; i += gridDim.x * 256ull) {
+    const float4* E = reinterpret_cast<const float4*>(entries + i);
+    const float4 a = __ldg(E), b = __ldg(E + 1), c = __ldg(E + 2);
+    const float V[9] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x};
+    float m[3], r2 = 0.f, X = 0.f;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      m[q] = (V[q] + V[3 + q] + V[6 + q]) * (1.0f / 3.0f);
+      X = fmaxf(fmaxf(X, fabsf(V[q])), fmaxf(fabsf(V[3 + q]), fabsf(V[6 + q])));
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      float s = 0.f;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) s = fmaf(V[3 * k + q] - m[q], V[3 * k + q] - m[q], s);
+      r2 = fmaxf(r2, s);
+    }
+    out[i] = make_float4(m[0], m[1], m[2], sqrtf(r2) * (1.0f + 8.0f * kU32) + 8.0f * kU32 * X);
+  }
 }
 
 // ENDS: 0 no geometry of the launch ends at this level, 1 all do, 2 some may (the point predicate's two walks share
@@ -3146,6 +3242,11 @@ int launch_refine(const RefineLevel& a, int num_sms, cudaStream_t st) {
     else
       go(k_refine<2, 0, 2>);
   }
+  return 1;
+}
+
+int launch_entry_spheres(const void* payload, const uint32_t* n_entries, float4* out, int num_sms, cudaStream_t st) {
+  k_entry_spheres<<<num_sms * 8, 256, 0, st>>>(static_cast<const Entry3*>(payload), n_entries, out);
   return 1;
 }
 
