@@ -669,6 +669,8 @@ struct Plan {
   bool face_at[AMR_MAX_LEVELS];     // some geometry's blocks of the level are marked face by face
   bool unit_at[AMR_MAX_LEVELS];     // ... with d the cell size (kFaceUnit)
   bool plain_at[AMR_MAX_LEVELS];    // ... with another d or predicate
+  FaceRange marked[AMR_MAX_LEVELS]; // faces of the geometries marked face by face on the level
+  FaceRange ending[AMR_MAX_LEVELS]; // faces of the geometries that end there
   bool rec_at[AMR_MAX_LEVELS];      // the faces leave the records of every geometry that ends at the level
   bool walk_at[AMR_MAX_LEVELS];     // some geometry's blocks of the level are walked
   bool adjacency, links;
@@ -755,7 +757,16 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
     const bool unit = unit_of(g);
     if (bits && unit) bits |= kFaceUnit;
     g.face_levels = bits;
+    const int64_t f0 = ctx->multi ? g.face_base : 0;
+    const int64_t f1 = ctx->multi && gi + 1 < ctx->geoms.size() ? ctx->geoms[gi + 1].face_base : ctx->nf;
+    auto take = [&](FaceRange& r) {
+      r.begin = r.used ? std::min(r.begin, f0) : f0;
+      r.end = r.used ? std::max(r.end, f1) : f1;
+      r.used += f1 - f0;
+    };
+    take(P.ending[g.n_levels - 1]);
     for (int L = 0; L < g.n_levels; ++L) {
+      if ((bits >> L) & 1u) take(P.marked[L]);
       if ((bits >> L) & 1u) {
         P.face_at[L] = true;
         (unit ? P.unit_at : P.plain_at)[L] = true;
@@ -905,6 +916,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
       m.face_gid = ctx->multi ? static_cast<const uint32_t*>(ctx->face_gid.p) : nullptr;
       for (int l = 0; l < L; ++l) m.first_child[l] = static_cast<const int32_t*>(ctx->lv[l].first.p);
       m.unit = P.unit_at[L];
+      m.faces = P.marked[L];
       m.plain = P.plain_at[L];
       if (a.blockcnt) CK(cudaMemsetAsync(a.blockcnt, 0, sizeof(uint64_t) * (size_t)(lb.cap > 0 ? lb.cap : 1), st));
       if (a.info) CK(cudaMemsetAsync(a.info, 0, sizeof(uint64_t) * (size_t)(lb.cap > 0 ? lb.cap : 1), st));
@@ -1066,6 +1078,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         fl.face_gid = marks.face_gid;
         fl.rec = marks.rec;
         fl.nf = ctx->nf;
+        fl.faces = P.ending[L];
         for (int l = 0; l < L; ++l) fl.first_child[l] = marks.first_child[l];
         fl.n_blocks = lb.cap;
         fl.n_dev = a.n_dev;

@@ -243,10 +243,11 @@ __global__ void __launch_bounds__(kFWarps * 32, kFBlocks) k_face_links(FaceLinkA
     unsigned base = 0;
     if (lane == 0) base = atomicAdd(a.work, (unsigned)a.batch);
     base = __shfl_sync(0xffffffffu, base, 0);
-    if ((int64_t)base >= a.nf) break;
+    const int64_t first = a.faces.begin + base;
+    if (first >= a.faces.end) break;
     // a lane per face: its cells (down to one layer outside the domain), their frame, the groups in reach
-    const int64_t f = (int64_t)base + lane;
-    bool use = lane < a.batch && f < a.nf;
+    const int64_t f = first + lane;
+    bool use = lane < a.batch && f < a.faces.end;
     const uint32_t gid = MULTI && use ? __ldg(a.face_gid + f) : 0u;
     const GeomParams& P = geom_of<MULTI>(a, gid);
     use = use && P.n_levels - 1 == a.level;
@@ -822,8 +823,9 @@ int launch_face_links(const FaceLinkArgs& a0, void* scan_scratch, int num_sms, c
   cudaMemsetAsync(a.group_runs, 0, sizeof(uint64_t) * (size_t)groups, st);
   cudaMemsetAsync(a.work, 0, sizeof(unsigned), st);
   const int64_t grid = (int64_t)num_sms * kFBlocks;
-  a.batch = fetch_size(a.nf, grid * kFWarps, kFFaces);
-  const int64_t need = std::max<int64_t>(1, (a.nf + (int64_t)a.batch * kFWarps - 1) / ((int64_t)a.batch * kFWarps));
+  a.batch = a.faces.fetch(grid * kFWarps, kFFaces);
+  const int64_t nf = a.faces.end - a.faces.begin;
+  const int64_t need = std::max<int64_t>(1, (nf + (int64_t)a.batch * kFWarps - 1) / ((int64_t)a.batch * kFWarps));
   if (a.table)
     k_face_links<true><<<(unsigned)std::min(need, grid), kFWarps * 32, 0, st>>>(a);
   else

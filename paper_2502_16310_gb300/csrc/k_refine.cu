@@ -2423,10 +2423,11 @@ __global__ void __launch_bounds__(kMarkWarps * 32, 6) k_mark_faces(MarkArgs m) {
     unsigned base = 0;
     if (lane == 0) base = atomicAdd(a.work, (unsigned)batch);
     base = __shfl_sync(0xffffffffu, base, 0);
-    if ((int64_t)base >= a.nf) break;
+    const int64_t first = m.faces.begin + base;
+    if (first >= m.faces.end) break;
     for (int q = 0; q < batch; ++q) {
-      const int64_t f = (int64_t)base + q;
-      if (f >= a.nf) break;
+      const int64_t f = first + q;
+      if (f >= m.faces.end) break;
       // the face's geometry: only geometries marked face by face on this level (their blocks of the
       // level have the mask as the only output; the walk does the others)
       const uint32_t gid = MULTI ? __ldg(m.face_gid + f) : 0u;
@@ -2781,10 +2782,11 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
     unsigned base = 0;
     if (lane == 0) base = atomicAdd(a.work, (unsigned)batch);
     base = __shfl_sync(0xffffffffu, base, 0);
-    if ((int64_t)base >= a.nf) break;
+    const int64_t first = m.faces.begin + base;
+    if (first >= m.faces.end) break;
     // a lane per face: its cell range and thresholds
-    const int64_t f = (int64_t)base + lane;
-    bool use = lane < batch && f < a.nf;
+    const int64_t f = first + lane;
+    bool use = lane < batch && f < m.faces.end;
     const uint32_t gid = MULTI && use ? __ldg(m.face_gid + f) : 0u;
     const GeomParams& P = row<MULTI>(a, gid);
     use = use && ((P.face_levels >> a.level) & 1u) && (P.face_levels & kFaceUnit);
@@ -3284,22 +3286,23 @@ int launch_adjacency(const EmitArgs& a, int num_sms, cudaStream_t st) {
 }
 
 int launch_mark_faces(const MarkArgs& m, int num_sms, cudaStream_t st) {
-  if (m.lv.nf <= 0) return 0;
+  const int64_t nf = m.faces.end - m.faces.begin;
+  if (nf <= 0) return 0;
   const bool point = m.lv.pred == 1, multi = m.lv.table != nullptr;
   int k = 0;
   auto go = [&](auto kernel, int batch, int64_t resident, int warps) {
     MarkArgs x = m;
     x.batch = batch;
-    const int64_t need = (m.lv.nf + (int64_t)x.batch * warps - 1) / ((int64_t)x.batch * warps);
+    const int64_t need = (nf + (int64_t)x.batch * warps - 1) / ((int64_t)x.batch * warps);
     if (k++) cudaMemsetAsync(m.lv.work, 0, sizeof(unsigned), st);
     kernel<<<(unsigned)std::min<int64_t>(need, resident), warps * 32, 0, st>>>(x);
   };
   auto cells = [&](auto kernel) {
     const int64_t grid = (int64_t)num_sms * kCellBlocks;
-    go(kernel, fetch_size(m.lv.nf, grid * kCellWarps, kCellFaces), grid, kCellWarps);
+    go(kernel, m.faces.fetch(grid * kCellWarps, kCellFaces), grid, kCellWarps);
   };
   auto faces = [&](auto kernel) {
-    const int64_t few = m.lv.nf / ((int64_t)num_sms * 48);  // two fetches for each of 24 warps per SM
+    const int64_t few = m.faces.used / ((int64_t)num_sms * 48);  // two fetches for each of 24 warps per SM
     go(kernel, (int)std::max<int64_t>(1, std::min<int64_t>(kFaceBatch, few)), (int64_t)num_sms * 8, kMarkWarps);
   };
   if (m.unit) {
