@@ -671,6 +671,8 @@ struct Plan {
   bool plain_at[AMR_MAX_LEVELS];    // ... with another d or predicate
   FaceRange marked[AMR_MAX_LEVELS]; // faces of the geometries marked face by face on the level
   FaceRange ending[AMR_MAX_LEVELS]; // faces of the geometries that end there
+  bool lines_at[AMR_MAX_LEVELS];    // links of the level can be found from the faces (k_flinks.cu) ...
+  double reach[AMR_MAX_LEVELS];     // ... the smallest d / h of the geometries that end there
   bool rec_at[AMR_MAX_LEVELS];      // the faces leave the records of every geometry that ends at the level
   bool walk_at[AMR_MAX_LEVELS];     // some geometry's blocks of the level are walked
   bool adjacency, links;
@@ -695,7 +697,10 @@ constexpr double kAutoUnitCells = 8192.0;
 
 // Links from the faces (k_flinks.cu) from this many (cell, face) pairs on: its seven launches cost about 30 us
 // more than the pair kernel's four (0.5 M links of 20 K faces 0.113 / 0.088 ms), from about 8 M links on it is
-// the faster (8 K faces 0.39 / 0.38 ms, 32 K faces 0.41 / 0.46, 97 M links of 72 K faces 3.13 / 4.37).
+// the faster (8 K faces 0.39 / 0.38 ms, 32 K faces 0.41 / 0.46, 97 M links of 72 K faces 3.13 / 4.37).  The pair
+// kernel's time goes by pairs, this one's by links: where d is below the cell size (fewer pairs per link) the line
+// is three times higher (d = 0.75 h: 6.2 M pairs 0.46 / 0.42, 21.6 M 1.25 / 1.36, 327 M 15.4 / 20.3; d = 1.5 h:
+// 13.5 M 0.46 / 0.66, 47 M 1.25 / 2.18, 724 M 15.4 / 33.0).
 constexpr int64_t kFaceLinkPairs = 4 << 20;
 
 // Cells of level L in the range of a face of geometry g whose largest AABB side
@@ -725,6 +730,11 @@ Plan make_plan(const amr_ctx* ctx, const amr_refine_params* p) {
   return P;
 }
 
+// Smallest d_L / h_L for which every face a link segment (length up to sqrt(2) h)
+// can cross is in the cell's adjacency list: the inflated cell box contains the
+// segment once d_L >= h_L / 2; the ball of the point predicate once d_L >= sqrt(2) h_L.
+double link_reach(int pred) { return pred == AMR_PRED_POINT ? 1.4142135623730951 : 0.5; }
+
 // Per geometry and level: face by face or the block walk (face_levels bits of
 // the geometry rows, uploaded with the table); the plan's face_at / walk_at say
 // which of the two launches a level needs.  Returns a signature of the choice.
@@ -744,6 +754,20 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
   for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
     const int L = ctx->geoms[gi].n_levels - 1;
     if (P.rec_at[L]) P.rec_at[L] = unit_of(ctx->geoms[gi]) && small_faces(gi, L, kMaxFaceCells, kAutoUnitCells);
+  }
+  // links from the faces: every face that crosses a link has to be in the cell's list, by more than the band, and
+  // the widest face's cells within what a warp of k_face_links holds
+  for (int L = 0; L < P.NL; ++L) {
+    P.lines_at[L] = any && P.links && P.fin_at[L] && L > 0 && ctx->dom.dim == 3;
+    P.reach[L] = INFINITY;
+  }
+  for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
+    const GeomParams& g = ctx->geoms[gi];
+    const int L = g.n_levels - 1;
+    const double hL = std::ldexp(g.h0, -L), emax = gi < ctx->face_ext_max.size() ? ctx->face_ext_max[gi] : INFINITY;
+    P.reach[L] = std::min(P.reach[L], g.d_abs / hL + g.d_rel);
+    P.lines_at[L] = P.lines_at[L] && P.reach[L] >= 1.001 * link_reach(P.pred) &&
+                    std::pow(emax * std::ldexp(1.0, L) + 6.0, 3.0) <= kMaxFaceCells;
   }
   for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
     GeomParams& g = ctx->geoms[gi];
@@ -777,11 +801,6 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
   }
   return sig;
 }
-
-// Smallest d_L / h_L for which every face a link segment (length up to sqrt(2) h)
-// can cross is in the cell's adjacency list: the inflated cell box contains the
-// segment once d_L >= h_L / 2; the ball of the point predicate once d_L >= sqrt(2) h_L.
-double link_reach(int pred) { return pred == AMR_PRED_POINT ? 1.4142135623730951 : 0.5; }
 
 RefineLevel level_args(amr_ctx* ctx, const Plan& P, int L) {
   RefineLevel a{};
@@ -1068,18 +1087,18 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         return launch_advance(ctx->d_scal + SC_TOT + L, nullptr, ctx->d_scal + SC_RUN,
                               static_cast<uint32_t*>(ctx->adj_off.p), ctx->cap_cells, ctx->d_err, true, st);
       });
-      if (eager) ctx->face_links[L] = P.links && P.rec_at[L] && L > 0 && pairs >= kFaceLinkPairs;
+      if (eager) ctx->face_links[L] = P.lines_at[L] && pairs >= (P.reach[L] < 1.0 ? 3 : 1) * kFaceLinkPairs;
       if (P.links && ctx->face_links[L]) {  // (a capture follows the eager pass before it)
-        // the faces that left the records find the links too
+        // the links are found from the faces
         FaceLinkArgs fl{};
         fl.level = L;
         fl.g0 = ctx->geoms[0];
         fl.table = a.table;
-        fl.face_gid = marks.face_gid;
-        fl.rec = marks.rec;
+        fl.face_gid = ctx->multi ? static_cast<const uint32_t*>(ctx->face_gid.p) : nullptr;
+        fl.rec = static_cast<const FaceRec3*>(ctx->frec.p);
         fl.nf = ctx->nf;
         fl.faces = P.ending[L];
-        for (int l = 0; l < L; ++l) fl.first_child[l] = marks.first_child[l];
+        for (int l = 0; l < L; ++l) fl.first_child[l] = static_cast<const int32_t*>(ctx->lv[l].first.p);
         fl.n_blocks = lb.cap;
         fl.n_dev = a.n_dev;
         fl.mask = a.mask;
@@ -1095,10 +1114,12 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         fl.err = ctx->d_err;
         for (int attempt = 0; attempt < 2; ++attempt) {
           if (eager) {
-            // first guesses: a quarter more hits than (cell, face) pairs, two runs per record; a level
-            // with more of anything runs once more with room for its exact counts
+            // first guesses: a quarter more hits than (cell, face) pairs where d is the cell size (pairs go with
+            // 1 + 2 d / h, or its square for faces below a cell), two runs per record; a level with more of
+            // anything runs once more with room for its exact counts
             if (attempt == 0) {
-              ctx->cap_hits = std::max(ctx->cap_hits, pairs + pairs / 4 + 1024);
+              const double thin = 3.0 / (1.0 + 2.0 * P.reach[L]), hits = 1.25 * (thin > 1.0 ? thin * thin : thin);
+              ctx->cap_hits = std::max(ctx->cap_hits, (int64_t)(hits * (double)pairs) + 1024);
               ctx->cap_runs = std::max(ctx->cap_runs, 2 * n_rec + 4096);
             }
             const int64_t want = run_links + ctx->cap_hits;
