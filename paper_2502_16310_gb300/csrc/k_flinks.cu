@@ -20,9 +20,10 @@
 //   k_write_links   per group: every hit to its place in (cell, direction) order, the least (t, face)
 //                   where faces compete, through shared memory so that the output is written in runs.
 //
-// Bound by instructions (about 1,000 warp instructions per 32 links in all, half of them in
-// k_face_links, at 16 warps per SM) and by the latency of the group kernels' loads.  465 M links of
-// 1.3 M faces: 24.2 ms by pairs, 15.3 here; 31.5 M of 82 K: 1.61, 1.25; 9.5 M of 20 K: 0.49, 0.46.
+// Bound by instructions (about 700 warp instructions per 32 links in all, 400 of them in k_face_links, at 16
+// warps per SM) and by the latency of the group kernels' loads.  465 M links of 1.3 M faces: 24.2 ms by pairs,
+// 14.9 here; 31.5 M of 82 K: 1.61, 1.19; 9.5 M of 20 K: 0.49, 0.45.  k_write_links with a word less per cell, so
+// that 8 CTAs fit an SM instead of 6: 1.25 -> 1.19 (1.28 at 7).
 // Direction by direction over 16 faces, the hits of a (face, group) left in pieces: 19.7 and 1.54 ms;
 // each cell's position worked out per crossing instead of taken from a table: 1.54.  At 5 blocks per SM
 // (96 registers, spills) 16.7 and 1.34 ms.
@@ -658,7 +659,7 @@ __global__ void __launch_bounds__(256) k_place_runs(FaceLinkArgs a) {
 }
 
 constexpr int kGWarps = 4;       // warps per CTA of the group kernels
-constexpr int kGBlocks = 6;      // CTAs of k_write_links per SM (shared memory)
+constexpr int kGBlocks = 8;      // CTAs of k_write_links per SM (shared memory)
 constexpr int kGWindow = 448;    // links of a group gathered in shared memory at a time
 
 // Visit a group's hits, 4 a lane at a time (their loads overlap): fn(valid, code, q, face); returns their
@@ -737,8 +738,8 @@ __global__ void __launch_bounds__(kGWarps * 32) k_count_links(FaceLinkArgs a) {
 }
 
 struct WriteSmem {
-  uint32_t dirs[kGCells];                // per cell: directions hit
-  uint32_t info[kGCells];                // per cell: its first link in the group | its row in the group << 14
+  uint32_t dirs[kGCells];                // per cell: directions hit (1 to 18) << 13 | its first link in the group (14 bits)
+  uint32_t cells[32];                    // per lane's 16 cells: the adjacent ones | row of the first << 16
   unsigned long long key[kGWindow];      // q bits << 34 | direction << 29 | face
   uint16_t row[kGWindow];
 };
@@ -766,17 +767,15 @@ __global__ void __launch_bounds__(kGWarps * 32, kGBlocks) k_write_links(FaceLink
     const uint32_t rows = __popc(cells);
     const uint32_t cincl = warp_inclusive_scan<uint32_t>(c), rincl = warp_inclusive_scan<uint32_t>(rows);
     const uint32_t total = __shfl_sync(0xffffffffu, cincl, 31);
+    sm.cells[lane] = cells | (rincl - rows) << 16;
     {
-      uint32_t at = cincl - c, row = rincl - rows;
+      uint32_t at = cincl - c;
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
-        const bool adj = (cells >> i) & 1u;
-        if (!adj) sm.dirs[17 * lane + i] = 0u;  // (a hit cell is adjacent: such hits do not occur)
-        sm.info[17 * lane + i] = at | row << 14;
-        if (adj) {
-          at += __popc(sm.dirs[17 * lane + i]);
-          ++row;
-        }
+        // (a hit cell is adjacent: others have no hits)
+        const uint32_t d = (cells >> i) & 1u ? sm.dirs[17 * lane + i] : 0u;
+        sm.dirs[17 * lane + i] = d << 13 | at;
+        at += __popc(d);
       }
     }
     __syncwarp();
@@ -790,15 +789,16 @@ __global__ void __launch_bounds__(kGWarps * 32, kGBlocks) k_write_links(FaceLink
       }
       for_hits<true>(a, g, n_run, lane, [&](bool ok, uint32_t code, float q, uint32_t face) {
         if (!ok) return;
-        const uint32_t cell = code & 511u, dir = code >> 9, d = sm.dirs[cell_word(cell)], w = sm.info[cell_word(cell)];
+        const uint32_t cell = code & 511u, dir = code >> 9, w = sm.dirs[cell_word(cell)], d = (w >> 13) & ~1u;
         const uint32_t pos = (w & 0x3fffu) + __popc(d & ((1u << dir) - 1u)) - w0;
         if (pos >= nw0 || !((d >> dir) & 1u)) return;
+        const uint32_t t = sm.cells[cell >> 4];
         const unsigned long long k = (unsigned long long)__float_as_uint(q) << 34 | (unsigned long long)dir << 29 | face;
         if (once)
           sm.key[pos] = k;
         else
           atomicMin(&sm.key[pos], k);
-        sm.row[pos] = (uint16_t)(w >> 14);
+        sm.row[pos] = (uint16_t)((t >> 16) + __popc(t & ((1u << (cell & 15u)) - 1u)));
       });
       __syncwarp();
       for (uint32_t i = lane; i < nw0; i += 32) {
