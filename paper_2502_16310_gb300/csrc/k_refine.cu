@@ -2604,8 +2604,8 @@ __global__ void __launch_bounds__(kMarkWarps * 32, 6) k_mark_faces(MarkArgs m) {
 // is far beyond FP64's rounding, so the inflated boxes of its neighbours meet
 // the face; a face certified apart from all 3^D cells of an inflated box has a
 // distance from it that FP64 sees.  Where the test of a cell is not certified,
-// its 3^D neighbours are tested with their own inflated boxes, as everywhere
-// else (FP32, then FP64).  Cells of one layer outside the domain are tested as
+// those of its 3^D neighbours that no certified cell marks are tested with their
+// own inflated boxes, each once, as everywhere else (FP32, then FP64).  Cells of one layer outside the domain are tested as
 // well, for they widen into it.  A cell that a face meets lies in a block of
 // the level: the cell above it was marked.
 //
@@ -2645,6 +2645,10 @@ struct MarkFace {
 constexpr int kCellWarps = 4;    // warps per CTA of k_mark_cells
 constexpr int kCellBlocks = 5;   // CTAs per SM (shared memory)
 constexpr int kCellFaces = 16;   // faces a warp takes per work fetch
+// FP64 decisions of an open cell's neighbours that go one by one over the warp's lanes, at most (82 K faces with 70 K
+// exact contacts, five levels: marks 3.19 ms at 0, 2.62 at 2, 2.16 at 6, 2.45 at 12, 2.55 with all; 5.60 when every
+// open cell settled all its neighbours, covered or already settled, before the widening).
+constexpr int kFewFp64 = 6;
 constexpr int kCellPool = 160;   // blocks of the ranges of a group of faces
 constexpr uint32_t kCellRow = 3; // mean cells per x-row above which rows are cut first
 constexpr int kCellTile = 3;     // a face with more blocks is taken in tiles of 3 per axis and their rims
@@ -2656,7 +2660,7 @@ struct CellSmem {
   MarkFace<D> f[kCellFaces];
   alignas(8) uint32_t met[kCellPool][2];  // per block: its cells that the face meets, then widened
   uint64_t tmp[kCellPool];
-  uint32_t more[kCellPool][2];   // cells marked by their own test
+  uint32_t open[kCellPool][2];   // cells whose test was not certified
   int32_t bi[kCellPool];         // the block's index (-1: absent)
   uint8_t own[kCellPool];        // its face
   int whole[4][3];               // a face taken in tiles: lo, n, blo, nb of its range
@@ -2944,7 +2948,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
           sm.bi[s] = find(Q.gid, b);
           sm.own[s] = (uint8_t)j;
           sm.met[s][0] = sm.met[s][1] = 0u;
-          sm.more[s][0] = sm.more[s][1] = 0u;
+          sm.open[s][0] = sm.open[s][1] = 0u;
         }
       }
       __syncwarp();
@@ -2978,6 +2982,7 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
       const uint32_t rincl = warp_inclusive_scan<uint32_t>(nr);
       const uint32_t rfirst = rincl - nr, nrow = __shfl_sync(0xffffffffu, rincl, 31);
       const bool by_row = D == 3 && ncell > kCellRow * nrow;
+      bool any_open = false;
       for (uint32_t r0 = 0; r0 < (by_row ? nrow : 1u); r0 += 32) {
         int jr = 0, iy = 0, iz = 0, ix = 0;
         uint32_t rc = 0;  // cells of the lane's row, from ix on
@@ -3026,70 +3031,38 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
           if (D == 3 && __any_sync(0xffffffffu, !sep) && valid_cell) cell_axes_edges<D>(sm.surv[j], co, sep, in);
           if (!sep && in) atomicOr(&sm.met[slot_of(C, cx)][local_of(cx) >> 5], 1u << (local_of(cx) & 31));
           const bool unsure = !sep && !in;
-          const int idx = ci[0] + C.n0 * (ci[1] + C.n1 * ci[2]);
-          // a cell whose test is not certified: its neighbours by their own inflated boxes, a lane each;
-          // then FP64, by the whole warp in 3D
-          for (unsigned ub = __ballot_sync(0xffffffffu, unsure); ub; ub &= ub - 1) {
-            const int src = __ffs(ub) - 1;
-            const int ju = __shfl_sync(0xffffffffu, j, src), iu = __shfl_sync(0xffffffffu, idx, src);
-            const MarkFace<D>& Q = sm.f[ju];
-            int t = 0, x[3] = {0, 0, 0};
-            if (lane < (D == 3 ? 27 : 9)) {
-              int i[3];
-              float o[3];
-              cell_of(Q, iu, i);
-              centre(Q, i, lane % 3 - 1, lane / 3 % 3 - 1, D == 3 ? lane / 9 - 1 : 0, x, o);
-              const uint32_t s = slot_of(Q, x);
-              const int32_t bi = sm.bi[s];
-              if (bi >= 0) {
-                // (a record wants every cell of its face, a mask only the cells that are not marked yet)
-                const uint64_t now = REC ? 0ull : __ldcg(reinterpret_cast<const unsigned long long*>(a.mask + bi));
-                if (!((now >> local_of(x)) & 1ull)) t = cell_test_grown<D>(sm.surv[ju], o, Q.h_hi);
-              }
-              if (D == 2 && t == 2) {
-                const int b[3] = {x[0] >> 2, x[1] >> 2, 0};
-                t = resolve_fp64<D>(a, Q.gid, Q.face, b, local_of(x), &wc.fb, &wc.band) ? 1 : 0;
-              }
-              if (t == 1) atomicOr(&sm.more[s][local_of(x) >> 5], 1u << (local_of(x) & 31));
-            }
-            if constexpr (D == 3) {
-              for (unsigned vb = __ballot_sync(0xffffffffu, t == 2); vb; vb &= vb - 1) {
-                const int e = __ffs(vb) - 1;
-                int y[3];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) y[q] = __shfl_sync(0xffffffffu, x[q], e);
-                bool in_band;
-                const bool adj = resolve_sat_warp(a, Q.gid, Q.face, y[0] >> 2, y[1] >> 2, y[2] >> 2, local_of(y), &in_band);
-                if (lane == 0) {
-                  ++wc.fb;
-                  wc.band += in_band ? 1ull : 0ull;
-                  if (adj) atomicOr(&sm.more[slot_of(Q, y)][local_of(y) >> 5], 1u << (local_of(y) & 31));
-                }
-              }
-            }
-            __syncwarp();
-          }
+          // a cell whose test is not certified is settled after the widening
+          if (unsure) atomicOr(&sm.open[slot_of(C, cx)][local_of(cx) >> 5], 1u << (local_of(cx) & 31));
+          any_open |= __any_sync(0xffffffffu, unsure);
         }
       }
       __syncwarp();
       // widen along each axis, a lane per block (met -> tmp -> met -> tmp)
       uint64_t* met = reinterpret_cast<uint64_t*>(&sm.met[0][0]);
+      auto at_of = [&](uint32_t s, int* at) {  // a slot's place in its face's blocks
+        const MarkFace<D>& Q = sm.f[sm.own[s]];
+        const int k = (int)(s - Q.slot), k1 = divn(k, Q.inv_b0), k2 = divn(k1, Q.inv_b1);
+        at[0] = k - k1 * Q.nb0, at[1] = k1 - k2 * Q.nb1, at[2] = k2;
+      };
+      auto sends = [&](uint32_t s) {  // a block of the level, and of the tile itself
+        const MarkFace<D>& Q = sm.f[sm.own[s]];
+        int at[3];
+        at_of(s, at);
+        bool send = sm.bi[s] >= 0;
+#pragma unroll
+        for (int q = 0; q < D; ++q) send = send && at[q] >= Q.c0[q] && at[q] < Q.c1[q];
+        return send;
+      };
       auto pass = [&](auto ax, const uint64_t* in, uint64_t* out, bool last) {
         constexpr int AX = decltype(ax)::value;
         for (uint32_t s = lane; s < nsl; s += 32) {
           const MarkFace<D>& Q = sm.f[sm.own[s]];
-          const int k = (int)(s - Q.slot), k1 = divn(k, Q.inv_b0), k2 = divn(k1, Q.inv_b1);
-          const int at[3] = {k - k1 * Q.nb0, k1 - k2 * Q.nb1, k2};
+          int at[3];
+          at_of(s, at);
           const int n = AX == 0 ? Q.nb0 : (AX == 1 ? Q.nb1 : Q.nb2);
           const int step = AX == 0 ? 1 : (AX == 1 ? Q.nb0 : Q.nb0 * Q.nb1);
           uint64_t w = widen<AX>(in[s], at[AX] > 0 ? in[s - step] : 0ull, at[AX] + 1 < n ? in[s + step] : 0ull);
-          if (last) {
-            w = (w | sm.more[s][0] | ((uint64_t)sm.more[s][1] << 32)) & (D == 3 ? ~0ull : 0xffffull);
-            bool send = sm.bi[s] >= 0;
-#pragma unroll
-            for (int q = 0; q < D; ++q) send = send && at[q] >= Q.c0[q] && at[q] < Q.c1[q];
-            if (!send) w = 0ull;
-          }
+          if (last) w = sends(s) ? w & (D == 3 ? ~0ull : 0xffffull) : 0ull;
           out[s] = w;
         }
         __syncwarp();
@@ -3097,7 +3070,60 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
       pass(std::integral_constant<int, 0>{}, met, sm.tmp, false);
       pass(std::integral_constant<int, 1>{}, sm.tmp, met, D == 2);
       if constexpr (D == 3) pass(std::integral_constant<int, 2>{}, met, sm.tmp, true);
-      const uint64_t* res = D == 3 ? sm.tmp : met;
+      uint64_t* res = D == 3 ? sm.tmp : met;
+      if (any_open) {
+        // the neighbours of open cells that no certain cell has marked: each once, by its own inflated box, a lane
+        // per neighbour; then FP64, in 3D a few by the whole warp, more of them a lane each
+        uint32_t* out = reinterpret_cast<uint32_t*>(res);
+        uint32_t* seen = reinterpret_cast<uint32_t*>(D == 3 ? met : sm.tmp);
+        for (uint32_t k = lane; k < 2 * nsl; k += 32) seen[k] = 0u;
+        __syncwarp();
+        for (uint32_t s = 0; s < nsl; ++s) {
+          for (uint64_t u = sm.open[s][0] | (uint64_t)sm.open[s][1] << 32; u; u &= u - 1) {
+            const int cell = __ffsll((long long)u) - 1;
+            const MarkFace<D>& Q = sm.f[sm.own[s]];
+            int t = 0, x[3] = {0, 0, 0};
+            uint32_t y = 0;
+            if (lane < (D == 3 ? 27 : 9)) {
+              int at[3], i[3] = {0, 0, 0};
+              float o[3];
+              at_of(s, at);
+#pragma unroll
+              for (int q = 0; q < D; ++q) i[q] = 4 * (Q.blo[q] + at[q]) + ((cell >> (2 * q)) & 3) - Q.lo[q];
+              centre(Q, i, lane % 3 - 1, lane / 3 % 3 - 1, D == 3 ? lane / 9 - 1 : 0, x, o);
+              const uint32_t sy = slot_of(Q, x);
+              y = 2 * sy + (local_of(x) >> 5);
+              const uint32_t bit = 1u << (local_of(x) & 31);
+              if (sends(sy) && !(out[y] & bit) && !(atomicOr(seen + y, bit) & bit)) {
+                // (a record wants every cell of its face, a mask only the cells that are not marked yet)
+                const uint64_t now = REC ? 0ull : __ldcg(reinterpret_cast<const unsigned long long*>(a.mask + sm.bi[sy]));
+                if (!((now >> local_of(x)) & 1ull)) t = cell_test_grown<D>(sm.surv[sm.own[s]], o, Q.h_hi);
+              }
+            }
+            const unsigned vb = __ballot_sync(0xffffffffu, t == 2);
+            if (D == 2 || __popc(vb) > kFewFp64) {
+              const int b[3] = {x[0] >> 2, x[1] >> 2, D == 3 ? x[2] >> 2 : 0};
+              if (t == 2) t = resolve_fp64<D>(a, Q.gid, Q.face, b, local_of(x), &wc.fb, &wc.band) ? 1 : 0;
+            } else if constexpr (D == 3) {
+              for (unsigned v = vb; v; v &= v - 1) {
+                const int e = __ffs(v) - 1;
+                int z[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) z[q] = __shfl_sync(0xffffffffu, x[q], e);
+                bool in_band;
+                const bool adj = resolve_sat_warp(a, Q.gid, Q.face, z[0] >> 2, z[1] >> 2, z[2] >> 2, local_of(z), &in_band);
+                if (lane == 0) {
+                  ++wc.fb;
+                  wc.band += in_band ? 1ull : 0ull;
+                }
+                if (lane == e) t = adj ? 1 : 0;
+              }
+            }
+            if (t == 1) atomicOr(out + y, 1u << (local_of(x) & 31));
+            __syncwarp();
+          }
+        }
+      }
       // a block's new marks with one atomic; a face of a geometry that ends here leaves a record for the block
       auto ends_here = [&](uint32_t s) {
         return !MULTI || row<MULTI>(a, sm.f[sm.own[s]].gid).n_levels - 1 == a.level;
