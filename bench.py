@@ -44,11 +44,12 @@ OPS_FACE_SETUP = 400.0        # face-by-face marking, per (face, level): cell ra
 OPS_LINK_DIR = 40.0           # per (adjacent cell, face, lattice direction): one watertight segment-triangle test
 OPS_LINK_FACE = 150.0         # per (adjacent cell, face), executed on top: double-float offsets, plane offset,
                               # cross products and the line filters (reported beside the roofline, not in it)
+OPS_LINK_LINE = 60.0          # per link found from the faces: half a lattice line's three edge functions, one plane
+                              # offset in double-float
+FACE_LINK_PAIRS = 4 << 20     # from this many pairs on a 3D level's links are found from the faces (csrc/api.cu)
 # DRAM bytes (read + write) per launch of the current kernels, from one ncu capture each
 # (dram__bytes_read.sum + dram__bytes_write.sum, one pass) of the named workload; others report null
-MEASURED_TRAFFIC = {("c4", "refine_level"): 393028096 + 2277046272,
-                    # the link step: k_links, the scan of its tile counts, k_links_place
-                    ("c4", "links"): 3768263936 + 4520397312 + 12329216 + 5083136000 + 6614900736}
+MEASURED_TRAFFIC = {}
 
 
 def parse_args(argv=None):
@@ -261,7 +262,8 @@ def run_ours(args, rank, world, local):
     t_refine = kern.get("refine_level", {}).get("ms_per_step", 0.0)
     t_mark = kern.get("mark_faces", {}).get("ms_per_step", 0.0)
     dom = max(kern.items(), key=lambda kv: kv[1]["ms_per_step"])
-    roof = roofline(dom[0], dom[1], w, kern, n_cand, n_surv, n_adj, n_pairs, blocks, clocks, n_fsetup, n_ftest)
+    roof = roofline(dom[0], dom[1], w, kern, n_cand, n_surv, n_adj, n_pairs, blocks, clocks, n_fsetup, n_ftest,
+                    n_links)
     roof["traffic"] = MEASURED_TRAFFIC.get((args.workload, dom[0]))
     NCe = 64 if w.dim == 3 else 16
     n_tests = n_surv * NCe + n_ftest  # block-walk cell tests + face-by-face (face, cell) tests
@@ -624,7 +626,7 @@ def run_paper_setups(args, dev, flush, bins=(1, 2, 4, 6, 7, 8, 9, 10, 12, 14, 16
     return out
 
 
-def roofline(name, k, w, kern, n_cand, n_surv, n_adj, n_pairs, blocks, clocks, n_fsetup=0, n_ftest=0):
+def roofline(name, k, w, kern, n_cand, n_surv, n_adj, n_pairs, blocks, clocks, n_fsetup=0, n_ftest=0, n_links=0):
     """Roofline entry for the dominant kernel: algorithmic work per launch / average launch time."""
     hbm, src = measured_peaks()
     launches = max(k["launches_per_step"], 1e-9)
@@ -644,6 +646,12 @@ def roofline(name, k, w, kern, n_cand, n_surv, n_adj, n_pairs, blocks, clocks, n
         a = ops / t / 1e12
         return {"kernel": name, "bound": "alu", "achieved": a, "peak": alu_peak, "unit": "Tops/s (FP32 pipe)",
                 "frac": a / alu_peak, "traffic": None, "peak_source": "152 SM x 128 FP32 lanes x 2070 MHz"}
+    if name == "links" and w.dim == 3 and n_pairs >= FACE_LINK_PAIRS:
+        ops = n_links * OPS_LINK_LINE / launches  # lattice line by lattice line: each link is computed once
+        a = ops / t / 1e12
+        return {"kernel": name, "bound": "alu", "achieved": a, "peak": alu_peak, "unit": "Tops/s (FP32 pipe)",
+                "frac": a / alu_peak, "traffic": None, "peak_source": "152 SM x 128 FP32 lanes x 2070 MHz",
+                "ops_per_launch": ops, "links_per_s": n_links / launches / t}
     if name == "links":
         # algorithmic work: one ~40-op watertight test per (adjacent cell, adjacent face, lattice direction)
         Q1 = 18 if w.dim == 3 else 8

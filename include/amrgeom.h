@@ -247,9 +247,9 @@ AMR_API amr_status amr_refine_near_wall(amr_ctx* ctx, const amr_refine_params* p
  * overwritten: [n_verts][dim] when the geometry was loaded as an index list,
  * else [n_faces][dim][dim].  Gradients flow through q of the hit face only
  * (dt/dv of the plane / line through that face); flags, masks and adjacency are
- * not differentiated.  Deterministic: links are grouped by face with a stable
- * radix sort and summed in ascending link order, face corners by vertex in
- * ascending (face, corner) order, without float atomics, so repeated calls give
+ * not differentiated.  Deterministic: links are grouped by face within tiles, the tiles' sums added per
+ * face as 64-bit integers at a scale of the face, face corners by vertex in ascending (face, corner)
+ * order, without float atomics, so repeated calls give
  * bitwise identical results.  ESTATE without links; EINVAL for host pointers. */
 AMR_API amr_status amr_q_backward(amr_ctx* ctx, const float* grad_q, float* grad_out);
 
@@ -258,8 +258,8 @@ AMR_API amr_status amr_q_backward(amr_ctx* ctx, const float* grad_q, float* grad
  * exactly binned single-geometry context: for every adjacent cell of the finest
  * level (row i of adj_cell), *cell_solid[i] = 1 when its centre lies inside the
  * closed boundary mesh, else 0 (fluid).  Decided by the parity of the faces a ray
- * from the centre along +x crosses (each face once; FP32 box cull, FP64 crossing
- * test); a ray through an edge or vertex, or a centre on a face, falls back to the
+ * from the centre along +x crosses (each face once; crossings certified in FP32, else
+ * FP64); a ray through an edge or vertex, or a centre on a face, falls back to the
  * generalized winding number of the whole mesh (|w| > 1/2 = solid), counted in
  * *n_fallback (nullable).  The mesh must be closed (either orientation).
  * cell_solid: BORROWED device u8 [n_adj_cells], valid until the next refinement.
