@@ -599,6 +599,12 @@ __device__ __noinline__ bool resolve_fp64(const RefineLevel& a, uint32_t gid, ui
   return m <= 0.0;
 }
 
+// FP64 decisions that go one by one by the whole warp (resolve_sat_warp), at most; more of them go a lane each (a
+// warp's DP instructions serve 13 axes of one pair there, and here 32 pairs).  A box of 49,152 faces on cell planes,
+// 4 levels, 21 M pairs, nearly all exact contacts: marks 146 ms one by one, 26.5 so (walk and marks before: 53.6);
+// 768 wide faces of the same box: walk 35.4 and 16.1.  82 K faces with 70 K exact contacts: marks 2.16 and 1.21.
+constexpr int kFewFp64 = 6;
+
 // sat_adjacent_fp64_3 by a whole warp, an axis per lane (the same operations in the same order per axis,
 // so the same decision and band): an FP64 operation takes tens of cycles here, and one pair's 13 axes in
 // a row held its warp for tens of microseconds, which on a small mesh is longer than the rest of a level.
@@ -1175,9 +1181,10 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
           cell_test2<D>(S, o0, o1, t0, t1);
         }
         if constexpr (D == 3 && !kPoint) {
-          for (uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h0) && t0 == 2) |
-                            ((uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h1) && t1 == 2) << 32);
-               u; u &= u - 1) {
+          uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h0) && t0 == 2) |
+                       ((uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h1) && t1 == 2) << 32);
+          if (__popcll(u) > kFewFp64) u = 0;  // (a lane each, below)
+          for (; u; u &= u - 1) {
             const int cell = __ffsll((long long)u) - 1;
             bool in_band;
             const int t = resolve_sat_warp(a, gid, S.face, b[0], b[1], b[2], cell, &in_band) ? 1 : 0;
@@ -1596,10 +1603,18 @@ __device__ __forceinline__ void walk_group(const RefineLevel& a, const GeomParam
           int t0 = 0, t1 = 0;
           cell_test2<3>(S, o0, o1, t0, t1);
           const int bj[3] = {c0[0] + cx, c0[1] + cy, c0[2] + cz};  // child j's block coordinates
-          // pairs not certified in FP32, one after another by the whole warp
-          for (uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !m0 && t0 == 2) |
-                            ((uint64_t)__ballot_sync(0xffffffffu, !m1 && t1 == 2) << 32);
-               u; u &= u - 1) {
+          // pairs not certified in FP32: many a lane each, a few one after another by the whole warp
+          uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !m0 && t0 == 2) |
+                       ((uint64_t)__ballot_sync(0xffffffffu, !m1 && t1 == 2) << 32);
+          if (__popcll(u) > kFewFp64) {
+            unsigned long long nf = 0, nb = 0;
+            if (!m0 && t0 == 2) t0 = resolve_fp64<3>(a, gid, S.face, bj, lane, &nf, &nb) ? 1 : 0;
+            if (!m1 && t1 == 2) t1 = resolve_fp64<3>(a, gid, S.face, bj, lane + 32, &nf, &nb) ? 1 : 0;
+            wc.fb += (unsigned)nf;
+            wc.band += (unsigned)nb;
+            u = 0;
+          }
+          for (; u; u &= u - 1) {
             const int cell = __ffsll((long long)u) - 1;
             bool in_band;
             const int t = resolve_sat_warp(a, gid, S.face, bj[0], bj[1], bj[2], cell, &in_band) ? 1 : 0;
@@ -2645,10 +2660,6 @@ struct MarkFace {
 constexpr int kCellWarps = 4;    // warps per CTA of k_mark_cells
 constexpr int kCellBlocks = 5;   // CTAs per SM (shared memory)
 constexpr int kCellFaces = 16;   // faces a warp takes per work fetch
-// FP64 decisions of an open cell's neighbours that go one by one over the warp's lanes, at most (82 K faces with 70 K
-// exact contacts, five levels: marks 3.19 ms at 0, 2.62 at 2, 2.16 at 6, 2.45 at 12, 2.55 with all; 5.60 when every
-// open cell settled all its neighbours, covered or already settled, before the widening).
-constexpr int kFewFp64 = 6;
 constexpr int kCellPool = 160;   // blocks of the ranges of a group of faces
 constexpr uint32_t kCellRow = 3; // mean cells per x-row above which rows are cut first
 constexpr int kCellTile = 3;     // a face with more blocks is taken in tiles of 3 per axis and their rims
@@ -3078,6 +3089,42 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
         uint32_t* seen = reinterpret_cast<uint32_t*>(D == 3 ? met : sm.tmp);
         for (uint32_t k = lane; k < 2 * nsl; k += 32) seen[k] = 0u;
         __syncwarp();
+        uint32_t pend = 0;  // lane i: the i-th neighbour (slot << 6 | cell) left to FP64
+        int np = 0;
+        auto decide = [&]() {
+          auto cell_at = [&](uint32_t e, int* z) {
+            const MarkFace<D>& Q = sm.f[sm.own[e >> 6]];
+            int at[3];
+            at_of(e >> 6, at);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) z[q] = q < D ? 4 * (Q.blo[q] + at[q]) + (int)((e >> (2 * q)) & 3u) : 0;
+            return &Q;
+          };
+          if (D == 2 || np > kFewFp64) {
+            if (lane < np) {
+              int z[3];
+              const MarkFace<D>& Q = *cell_at(pend, z);
+              const int b[3] = {z[0] >> 2, z[1] >> 2, z[2] >> 2};
+              if (resolve_fp64<D>(a, Q.gid, Q.face, b, (int)(pend & 63u), &wc.fb, &wc.band))
+                atomicOr(out + 2 * (pend >> 6) + ((pend >> 5) & 1u), 1u << (pend & 31u));
+            }
+          } else if constexpr (D == 3) {
+            for (int k = 0; k < np; ++k) {
+              const uint32_t e = __shfl_sync(0xffffffffu, pend, k);
+              int z[3];
+              const MarkFace<D>& Q = *cell_at(e, z);
+              bool in_band;
+              const bool adj = resolve_sat_warp(a, Q.gid, Q.face, z[0] >> 2, z[1] >> 2, z[2] >> 2, (int)(e & 63u), &in_band);
+              if (lane == 0) {
+                ++wc.fb;
+                wc.band += in_band ? 1ull : 0ull;
+                if (adj) atomicOr(out + 2 * (e >> 6) + ((e >> 5) & 1u), 1u << (e & 31u));
+              }
+            }
+          }
+          np = 0;
+          __syncwarp();
+        };
         for (uint32_t s = 0; s < nsl; ++s) {
           for (uint64_t u = sm.open[s][0] | (uint64_t)sm.open[s][1] << 32; u; u &= u - 1) {
             const int cell = __ffsll((long long)u) - 1;
@@ -3100,29 +3147,16 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
                 if (!((now >> local_of(x)) & 1ull)) t = cell_test_grown<D>(sm.surv[sm.own[s]], o, Q.h_hi);
               }
             }
-            const unsigned vb = __ballot_sync(0xffffffffu, t == 2);
-            if (D == 2 || __popc(vb) > kFewFp64) {
-              const int b[3] = {x[0] >> 2, x[1] >> 2, D == 3 ? x[2] >> 2 : 0};
-              if (t == 2) t = resolve_fp64<D>(a, Q.gid, Q.face, b, local_of(x), &wc.fb, &wc.band) ? 1 : 0;
-            } else if constexpr (D == 3) {
-              for (unsigned v = vb; v; v &= v - 1) {
-                const int e = __ffs(v) - 1;
-                int z[3];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) z[q] = __shfl_sync(0xffffffffu, x[q], e);
-                bool in_band;
-                const bool adj = resolve_sat_warp(a, Q.gid, Q.face, z[0] >> 2, z[1] >> 2, z[2] >> 2, local_of(z), &in_band);
-                if (lane == 0) {
-                  ++wc.fb;
-                  wc.band += in_band ? 1ull : 0ull;
-                }
-                if (lane == e) t = adj ? 1 : 0;
-              }
-            }
             if (t == 1) atomicOr(out + y, 1u << (local_of(x) & 31));
+            for (unsigned vb = __ballot_sync(0xffffffffu, t == 2); vb; vb &= vb - 1) {
+              const uint32_t e = __shfl_sync(0xffffffffu, (y >> 1) << 6 | (uint32_t)local_of(x), __ffs(vb) - 1);
+              if (lane == np) pend = e;
+              if (++np == 32) decide();
+            }
             __syncwarp();
           }
         }
+        if (np) decide();
       }
       // a block's new marks with one atomic; a face of a geometry that ends here leaves a record for the block
       auto ends_here = [&](uint32_t s) {
