@@ -1049,7 +1049,8 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
       }
       if (P.rec_at[L])
         timed(ctx, st, "place_records", [&] {
-          return launch_place_records(a, static_cast<const uint64_t*>(lb.rfirst.p), ctx->num_sms, st);
+          return launch_place_records(a, static_cast<const uint64_t*>(lb.rfirst.p), ctx->d_scal + SC_TOT + L,
+                                      ctx->num_sms, st);
         });
       if (eager) {
         cells = (int64_t)(tot >> 32);

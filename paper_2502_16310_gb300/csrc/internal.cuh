@@ -584,9 +584,11 @@ constexpr int kFaceBatch = 8;  // most faces a warp of the general kernel takes 
 int launch_mark_faces(const MarkArgs& m, int num_sms, cudaStream_t st);
 // A level whose records the faces left (lv.staged): blockcnt and the blocks' record counts; then, with
 // first = the exclusive scan of n_rec, the records by block and their descriptors (ERR_OVERFLOW when
-// more were left than cap_recs).
+// more were left than cap_recs: no block has records then, and level_tot, the level's pairs | cells << 32,
+// is set to zero).
 int launch_record_counts(const RefineLevel& a, uint64_t* n_rec, int num_sms, cudaStream_t st);
-int launch_place_records(const RefineLevel& a, const uint64_t* first, int num_sms, cudaStream_t st);
+int launch_place_records(const RefineLevel& a, const uint64_t* first, uint64_t* level_tot, int num_sms,
+                         cudaStream_t st);
 
 // The algorithmic cell-face test count of one level (single geometry): per cell
 // of its blocks, the distinct faces in the bins its inflated box overlaps,

@@ -3232,10 +3232,19 @@ __global__ void __launch_bounds__(256) k_record_counts(RefineLevel a, uint64_t* 
 }
 
 // The staged records into their blocks' runs (first[b] = scan of the counts), and each block's descriptor.
-__global__ void __launch_bounds__(256) k_place_records(RefineLevel a, const uint64_t* first) {
+// More records than were staged (a replay whose capacities were outgrown; the caller runs again with more
+// room): the level is left without records, cells and pairs, so that the kernels after this one find nothing
+// to read (rows without their offsets would lead the link kernel out of its tables).
+__global__ void __launch_bounds__(256) k_place_records(RefineLevel a, const uint64_t* first, uint64_t* level_tot) {
   const int64_t n = (int64_t)*a.rec_count;
-  if (n > a.cap_recs) {  // some were not staged: the caller runs again with more room
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.err, ERR_OVERFLOW);
+  if (n > a.cap_recs) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      *level_tot = 0;
+      atomicOr(a.err, ERR_OVERFLOW);
+    }
+    const int64_t nb = launch_count(a.n_blocks, a.n_dev, a.err);
+    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nb; b += (int64_t)gridDim.x * blockDim.x)
+      a.rec_desc[b] = 0ull;
     return;
   }
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -3390,9 +3399,10 @@ int launch_record_counts(const RefineLevel& a, uint64_t* n_rec, int num_sms, cud
   return 1;
 }
 
-int launch_place_records(const RefineLevel& a, const uint64_t* first, int num_sms, cudaStream_t st) {
+int launch_place_records(const RefineLevel& a, const uint64_t* first, uint64_t* level_tot, int num_sms,
+                         cudaStream_t st) {
   const int64_t g = std::min<int64_t>((a.cap_recs + 255) / 256, (int64_t)num_sms * 8);
-  k_place_records<<<(unsigned)std::max<int64_t>(1, g), 256, 0, st>>>(a, first);
+  k_place_records<<<(unsigned)std::max<int64_t>(1, g), 256, 0, st>>>(a, first, level_tot);
   return 1;
 }
 
