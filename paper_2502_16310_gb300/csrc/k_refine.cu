@@ -2234,7 +2234,8 @@ __global__ void __launch_bounds__(kChThreads) k_children(ChildrenArgs a, uint64_
         if (j < n) {
           const uint64_t o = kk * NCH;
           if (fl[i] && o >= 0x7fffffffull) atomicOr(a.err, ERR_OVERFLOW);
-          a.first_child[j] = fl[i] ? (int32_t)o : -1;
+          // children past the level's capacity (reported below) do not exist: the block lookups descend by this index
+          a.first_child[j] = fl[i] && (int64_t)(o + NCH) <= a.cap_out ? (int32_t)o : -1;
         }
         kk += fl[i];
       }

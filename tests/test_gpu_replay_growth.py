@@ -50,3 +50,13 @@ def test_more_records_than_staged():
     small = np.concatenate([inside, _tiny(rng, 3500, 1.5, 1.9)]).astype(np.float32)
     large = np.concatenate([inside, _tiny(rng, 3500, 0.3, 0.5)]).astype(np.float32)
     _grow(small, large, 4, 2, 1)
+
+
+@pytest.mark.parametrize("levels", [2, 4])
+def test_more_blocks_than_captured(levels):
+    """600 faces in one corner, then all over the domain: every level below the roots has many times its blocks, and
+    the faces look their blocks up through the levels above."""
+    rng = np.random.default_rng(2)
+    small = _tiny(rng, 600, 0.02, 0.1).astype(np.float32)
+    large = _tiny(rng, 600, 0.02, 0.98).astype(np.float32)
+    _grow(small, large, 8, 2, levels)
