@@ -573,8 +573,8 @@ amr_status amr_bin_all(amr_ctx* ctx) {
   TRY(ensure(ctx, ctx->count, sizeof(uint32_t) * (size_t)nb));
   if (!ctx->count_clean) {
     CK(cudaMemsetAsync(ctx->count.p, 0, ctx->count.cap, st));
-    ctx->count_clean = true;
   }
+  ctx->count_clean = false;  // until the scatter has counted every bin back to zero
   TRY(ensure(ctx, ctx->offsets, sizeof(uint32_t) * (size_t)(nb + 1)));
   TRY(ensure(ctx, ctx->frange, sizeof(uint32_t) * 3 * (size_t)(nf > 0 ? nf : 1)));
   TRY(ensure(ctx, ctx->scratch, scan_u32_scratch_bytes(nb)));
@@ -634,14 +634,9 @@ amr_status amr_bin_all(amr_ctx* ctx) {
     ctx->face_ext_max[g] = f1 > f0 ? (double)mx : 0.0;
     ctx->face_ext_mean[g] = f1 > f0 ? (double)hs[2 * g + 1] / 65536.0 / (double)(f1 - f0) : 0.0;
   }
-  if (e) {
-    ctx->count_clean = false;
-    return device_error(ctx, e);
-  }
-  if (tot > 0xffffffffull) {
-    ctx->count_clean = false;
+  if (e) return device_error(ctx, e);
+  if (tot > 0xffffffffull)
     return fail(ctx, AMR_EOVERFLOW, "%llu (face, bin) entries exceed 2^32 - 1", (unsigned long long)tot);
-  }
   const size_t esz = D == 3 ? sizeof(Entry3) : sizeof(Entry2);
   TRY(ensure(ctx, ctx->ids, sizeof(uint32_t) * (size_t)tot));
   TRY(ensure(ctx, ctx->payload, esz * (size_t)tot));
@@ -653,6 +648,7 @@ amr_status amr_bin_all(amr_ctx* ctx) {
   sa.rec = static_cast<const FaceRec3*>(ctx->frec.p);
   timed(ctx, st, "bin_scatter", [&] { return launch_scatter(sa, st); });
   CK(cudaGetLastError());
+  ctx->count_clean = true;
   ctx->n_bins = nb;
   ctx->nnz = (int64_t)tot;
   ctx->binned = true;
