@@ -847,6 +847,15 @@ __global__ void k_set_u64(uint64_t* p, uint64_t v) { *p = v; }
 // room for the sizes to drift between calls (a moving wall) without an overflow.
 int64_t with_slack(int64_t n) { return n + n / 8 + 256; }
 
+// Room for n survivor records.  The capacity is stated only once the buffer is there: after a failed allocation
+// the next pass asks again (the faces' records are placed without a test for the buffer).
+amr_status grow_records(amr_ctx* ctx, int64_t n) {
+  ctx->cap_recs = 0;
+  TRY(ensure(ctx, ctx->recs, sizeof(SurvRec) * (size_t)n));
+  ctx->cap_recs = n;
+  return AMR_OK;
+}
+
 // One pass over all levels.  eager: learn sizes with read-backs and grow
 // buffers (with slack when a graph is captured next); otherwise (capture) use
 // the capacities as they are.
@@ -901,10 +910,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         TRY(ensure(ctx, lb.desc, sizeof(uint64_t) * n1));
         // record staging: what the last pass needed, at least a few per block
         int64_t want = ctx->want_recs > 4 * lb.cap + 1024 ? ctx->want_recs : 4 * lb.cap + 1024;
-        if (want > ctx->cap_recs) {
-          TRY(ensure(ctx, ctx->recs, sizeof(SurvRec) * (size_t)want));
-          ctx->cap_recs = want;
-        }
+        if (want > ctx->cap_recs) TRY(grow_records(ctx, want));
         if (P.rec_at[L]) {
           TRY(ensure(ctx, ctx->staged, sizeof(StagedRec) * (size_t)ctx->cap_recs));
           TRY(ensure(ctx, lb.info, sizeof(uint64_t) * n1));
@@ -1033,8 +1039,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         TRY(device_error(ctx, e));
         if (!P.rec_at[L] || n_rec <= ctx->cap_recs) break;
         // the faces left more records than there was room for: again, with room for all
-        ctx->cap_recs = n_rec + n_rec / 4 + 1024;
-        TRY(ensure(ctx, ctx->recs, sizeof(SurvRec) * (size_t)ctx->cap_recs));
+        TRY(grow_records(ctx, n_rec + n_rec / 4 + 1024));
         TRY(ensure(ctx, ctx->staged, sizeof(StagedRec) * (size_t)ctx->cap_recs));
         a = level_args(ctx, P, L);
         marks.lv = a;
@@ -1194,6 +1199,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         la.n_links = ctx->d_scal + SC_NL + L;
         la.counters = ctx->counters;
         la.err = ctx->d_err;
+        int64_t exact = 0;  // links up to and with this level, once counted
         for (int attempt = 0; attempt < 2; ++attempt) {
           if (eager) {
             // first guess: a quarter more links than (cell, face) pairs (the synthetic spheres have
@@ -1201,7 +1207,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
             const int64_t guess = pairs + pairs / 4 + 1024;
             const int64_t want = run_links + (guess > cells ? guess : cells);
             if (want > ctx->cap_links || attempt > 0) {
-              const int64_t nc = attempt > 0 ? ctx->cap_links : want;
+              const int64_t nc = attempt > 0 ? exact : want;
               const size_t keep = (size_t)run_links;
               TRY(ensure_keep(ctx, ctx->link_cell, sizeof(uint32_t) * (size_t)(nc + 1), sizeof(uint32_t) * keep));
               TRY(ensure_keep(ctx, ctx->link_dir, (size_t)(nc + 1), keep));
@@ -1232,7 +1238,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
           }
           // too small: grow to the exact count and run the level's links again
           CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(unsigned), st));
-          ctx->cap_links = run_links + (int64_t)nl;
+          exact = run_links + (int64_t)nl;
         }
       }
       timed(ctx, st, "advance", [&] {

@@ -6,6 +6,9 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
+KEYS = ("adj_cell", "adj_off", "adj_ids", "link_cell", "link_dir", "link_q", "link_face")
+
+
 def _mesh(kind):
     """cluster: more records than a block's usual share; wide: more links than a quarter above the pairs."""
     if kind == "cluster":
@@ -74,5 +77,19 @@ def test_binning(kind):
         torch.cuda.synchronize()
         bins = torch.bucketize(torch.arange(b["nnz"], device="cuda"), b["offsets"][1:].long(), right=True)
         return [b["offsets"].clone(), torch.sort(bins * (1 << 29) + b["ids"].long())[0]]
+
+    _each_fails_once(kind, call)
+
+
+@pytest.mark.parametrize("kind", ["cluster", "wide"])
+def test_refinement(kind):
+    import torch
+
+    def call(g, dev):
+        g.load(dev)
+        g.bin(8)
+        r = g.refine(2, 0.0, 1.0, 19, True, True)
+        torch.cuda.synchronize()
+        return [lv["mask"].clone() for lv in r["levels"]] + [r[k].clone() for k in KEYS]
 
     _each_fails_once(kind, call)
