@@ -781,7 +781,8 @@ struct FaceLinkArgs {
   unsigned* err;
   int batch;                   // faces per work fetch (set by the launcher)
 };
-// ERR_OVERFLOW where hits, runs or links exceed their capacity (their counts are right then).
+// ERR_OVERFLOW where hits, runs or links exceed their capacity.  The counts of hits and runs are right then; with
+// more of them than there is room for no links are counted or written (n_links = 0).
 int launch_face_links(const FaceLinkArgs& a, void* scan_scratch, int num_sms, cudaStream_t st);
 
 size_t links_scratch_bytes(int64_t n_adj);

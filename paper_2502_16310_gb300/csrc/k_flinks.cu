@@ -721,11 +721,12 @@ __global__ void __launch_bounds__(kGWarps * 32) k_count_links(FaceLinkArgs a) {
   const int lane = threadIdx.x & 31;
   uint32_t* dirs = s_dirs[threadIdx.x >> 5];
   const int64_t n = (int64_t)*a.n_groups, nw = (int64_t)gridDim.x * kGWarps;
-  if ((int64_t)*a.run_count > a.cap_runs || (int64_t)*a.hit_count > a.cap_hits) return;  // reported by k_place_runs
+  // not all were kept (reported by k_place_runs): the level has no links then
+  const bool kept = (int64_t)*a.run_count <= a.cap_runs && (int64_t)*a.hit_count <= a.cap_hits;
   for (int64_t g = (int64_t)blockIdx.x * kGWarps + (threadIdx.x >> 5); g < n; g += nw) {
     const uint32_t n_run = (uint32_t)a.group_runs[g];
     uint32_t c = 0;
-    if (n_run) {
+    if (n_run && kept) {
       mark_hits(a, g, n_run, dirs, lane);
       const uint32_t cells = lane_cells(a, g, lane);
 #pragma unroll
@@ -750,7 +751,7 @@ __global__ void __launch_bounds__(kGWarps * 32, kGBlocks) k_write_links(FaceLink
   WriteSmem& sm = s_all[threadIdx.x >> 5];
   const int64_t n = (int64_t)*a.n_groups, nw = (int64_t)gridDim.x * kGWarps;
   const uint64_t row0 = a.run[0], link0 = a.run[2];
-  if ((int64_t)(link0 + *a.n_links) > a.link_cap) {
+  if (link0 + *a.n_links > (uint64_t)a.link_cap) {
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.err, ERR_OVERFLOW);
     return;
   }

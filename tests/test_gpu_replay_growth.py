@@ -60,3 +60,14 @@ def test_more_blocks_than_captured(levels):
     small = _tiny(rng, 600, 0.02, 0.1).astype(np.float32)
     large = _tiny(rng, 600, 0.02, 0.98).astype(np.float32)
     _grow(small, large, 8, 2, levels)
+
+
+def test_more_hits_than_captured():
+    """Links found from the faces (over 4 M pairs): a sphere beside a copy of itself outside the domain, then on top of
+    it.  The cells stay, every link is hit twice."""
+    from synth import geometry as G
+
+    v, f = G.jittered_sphere(6, radius=0.3, centre=(0.5, 0.49, 0.51), sigma=1e-4, seed=9)
+    t = v[f]
+    small, large = np.concatenate([t, t + np.float32(2.0)]), np.concatenate([t, t])
+    _grow(small.astype(np.float32), large.astype(np.float32), 32, 8, 3)
