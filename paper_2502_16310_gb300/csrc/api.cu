@@ -708,6 +708,16 @@ double face_cells(const amr_ctx* ctx, const GeomParams& g, int L, double ext, do
   return std::pow(ext * std::ldexp(1.0, L) + 2.0 * dh + pad, (double)ctx->dom.dim);
 }
 
+// Cells of level L by which the kernels widen a face's range, over both sides, for the rounding of its coordinates
+// (16 u (|v| + |origin|) / h a side; k_mark_faces, k_mark_cells, k_face_links): next to nothing, but some cells from
+// about a million cells away from the coordinates' origin on.
+double range_margin(const amr_ctx* ctx, const GeomParams& g, int L, double ext) {
+  double m = 0.0;
+  for (int a = 0; a < ctx->dom.dim; ++a)
+    m = std::max(m, 2.0 * std::fabs(g.origin[a]) + (4.0 * g.root[a] + ext) * g.h0);
+  return 2.0 * 16.0 * std::ldexp(1.0, -24) * m / std::ldexp(g.h0, -L);
+}
+
 Plan make_plan(const amr_ctx* ctx, const amr_refine_params* p) {
   Plan P{};
   for (const auto& g : ctx->geoms) P.NL = g.n_levels > P.NL ? g.n_levels : P.NL;
@@ -741,7 +751,7 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
   auto small_faces = [&](size_t gi, int L, double most, double mean) {
     const double emax = gi < ctx->face_ext_max.size() ? ctx->face_ext_max[gi] : INFINITY;
     const double emean = gi < ctx->face_ext_mean.size() ? ctx->face_ext_mean[gi] : INFINITY;
-    return face_cells(ctx, ctx->geoms[gi], L, emax, 4.0) <= most &&
+    return face_cells(ctx, ctx->geoms[gi], L, emax, 4.0 + range_margin(ctx, ctx->geoms[gi], L, emax)) <= most &&
            (p->face_pass != AMR_FACE_PASS_AUTO || face_cells(ctx, ctx->geoms[gi], L, emean, 1.0) <= mean);
   };
   const bool any = p->face_pass != AMR_FACE_PASS_OFF && P.search == AMR_SEARCH_QUERY_BOX;
@@ -763,7 +773,7 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
     const double hL = std::ldexp(g.h0, -L), emax = gi < ctx->face_ext_max.size() ? ctx->face_ext_max[gi] : INFINITY;
     P.reach[L] = std::min(P.reach[L], g.d_abs / hL + g.d_rel);
     P.lines_at[L] = P.lines_at[L] && P.reach[L] >= 1.001 * link_reach(P.pred) &&
-                    std::pow(emax * std::ldexp(1.0, L) + 6.0, 3.0) <= kMaxFaceCells;
+                    std::pow(emax * std::ldexp(1.0, L) + 6.0 + range_margin(ctx, g, L, emax), 3.0) <= kMaxFaceCells;
   }
   for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
     GeomParams& g = ctx->geoms[gi];
