@@ -671,6 +671,7 @@ struct Plan {
   double reach[AMR_MAX_LEVELS];     // ... the smallest d / h of the geometries that end there
   bool rec_at[AMR_MAX_LEVELS];      // the faces leave the records of every geometry that ends at the level
   bool walk_at[AMR_MAX_LEVELS];     // some geometry's blocks of the level are walked
+  bool gather_at[AMR_MAX_LEVELS];   // mark-only walks of the point predicate gather faces (mark_batch)
   bool adjacency, links;
   int lattice, warps, pred, search, propagate;
   int64_t n_roots;
@@ -741,6 +742,33 @@ Plan make_plan(const amr_ctx* ctx, const amr_refine_params* p) {
 // segment once d_L >= h_L / 2; the ball of the point predicate once d_L >= sqrt(2) h_L.
 double link_reach(int pred) { return pred == AMR_PRED_POINT ? 1.4142135623730951 : 0.5; }
 
+// Mark-only walks of the point predicate: gather the faces and test a lane per face (mark_batch), or take them one
+// at a time over the lanes' cells.  Gathering pays where many small faces reach a block and most cells are settled by
+// a face's sphere; it takes an entry for every bin that a face lies in and 64 steps per batch however few its faces.
+//
+// Query box: at least 16 (2D: 32) faces across the reach of a block, (4 h + 2 d) / e to the power D - 1 with e the
+// mean face's side, and at most two bins per face.  Sums over 1,008 levels of spheres of 80 to 112,500 faces, d
+// from 0.75 to 32 cells, 8 to 256 bins per axis (0.671 s one at a time): 0.622 s by this rule, 0.615 the better of
+// both everywhere, 3.35 s gathered everywhere; worst call 0.98 of one at a time, best 2.35.  2D, 720 levels: 87.8
+// ms one at a time, 39.8 by the rule, 46.8 gathered.
+// Own bin: 3D blocks at least two faces across and bins from three cells to no less than d (1,296 levels: 0.492 s
+// one at a time, 0.410 by the rule, 0.422 gathered; worst 0.98), 2D blocks at least 16 faces across (74.6, 41.0 and
+// 40.0 ms; worst 1.00, gathered 0.80).
+bool gather_pays(const amr_ctx* ctx, const Plan& P, size_t gi, int L) {
+  const GeomParams& g = ctx->geoms[gi];
+  const int D = ctx->dom.dim;
+  const double h = std::ldexp(g.h0, -L), d = g.d_abs + g.d_rel * h;
+  const double e = gi < ctx->face_ext_mean.size() ? ctx->face_ext_mean[gi] * g.h0 : INFINITY;
+  if (P.search == AMR_SEARCH_OWN_BIN) {
+    if (D == 2) return 4.0 * h >= 16.0 * e;
+    double bin = INFINITY;
+    for (int a = 0; a < D; ++a) bin = std::min(bin, 1.0 / g.bin_scale[a]);
+    return 4.0 * h >= 2.0 * e && bin >= 3.0 * h && bin >= d;
+  }
+  const double across = (4.0 * h + 2.0 * d) / e;
+  return (D == 2 ? across >= 32.0 : across * across >= 16.0) && ctx->nnz <= 2 * ctx->nf;
+}
+
 // Per geometry and level: face by face or the block walk (face_levels bits of
 // the geometry rows, uploaded with the table); the plan's face_at / walk_at say
 // which of the two launches a level needs.  Returns a signature of the choice.
@@ -775,6 +803,7 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
     P.lines_at[L] = P.lines_at[L] && P.reach[L] >= 1.001 * link_reach(P.pred) &&
                     std::pow(emax * std::ldexp(1.0, L) + 6.0 + range_margin(ctx, g, L, emax), 3.0) <= kMaxFaceCells;
   }
+  for (int L = 0; L < P.NL; ++L) P.gather_at[L] = P.pred == AMR_PRED_POINT;  // where it pays for every geometry's walk
   for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
     GeomParams& g = ctx->geoms[gi];
     uint32_t bits = 0;
@@ -800,8 +829,10 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
       if ((bits >> L) & 1u) {
         P.face_at[L] = true;
         (unit ? P.unit_at : P.plain_at)[L] = true;
-      } else
+      } else {
         P.walk_at[L] = true;
+        if (L < g.n_levels - 1 || !P.adjacency) P.gather_at[L] = P.gather_at[L] && gather_pays(ctx, P, gi, L);
+      }
     }
     sig = (sig ^ bits) * 1099511628211ull;
   }
@@ -844,6 +875,7 @@ RefineLevel level_args(amr_ctx* ctx, const Plan& P, int L) {
   a.warps = P.warps;
   a.pred = P.pred;
   a.search = P.search;
+  a.gather = P.gather_at[L];
   // blocks per work fetch: batches hide the fetch latency where every warp has many blocks;
   // single blocks keep the load balanced where there are few (and heavy ones cluster)
   const int64_t per_warp = ctx->lv[L].cap / ((int64_t)ctx->num_sms * 16);
@@ -895,7 +927,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
   });
   bool spheres = false;  // some block is walked for its mask only by the 3D point predicate
   for (int L = 0; L < P.NL; ++L)
-    spheres |= D == 3 && P.pred == AMR_PRED_POINT && P.search == AMR_SEARCH_QUERY_BOX && P.walk_at[L] &&
+    spheres |= D == 3 && P.pred == AMR_PRED_POINT && P.search == AMR_SEARCH_QUERY_BOX && P.gather_at[L] && P.walk_at[L] &&
                (P.cont_after[L] || !P.adjacency);
   if (spheres) {
     if (eager) TRY(ensure(ctx, ctx->spheres, ctx->payload.cap / sizeof(Entry3) * sizeof(float4)));

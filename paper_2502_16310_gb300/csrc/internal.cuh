@@ -541,6 +541,7 @@ struct RefineLevel {
   StagedRec* staged;           // nullable: records left by the faces, capacity cap_recs; then also:
   uint64_t* info;              // per block: its records | pairs << kInfoShift (zeroed before)
   SurvRec* spill;              // nullable: kSpillCap records per warp of the launch (records past kRecCap)
+  bool gather;                 // point predicate, mark-only blocks: faces gathered 32 at a time (mark_batch)
   unsigned long long* counters;
   unsigned* work;              // dynamic work counter (zeroed before launch)
   unsigned* err;

@@ -713,6 +713,7 @@ __device__ __forceinline__ void issue_chunk(const E* payload, uint32_t s, uint32
 // walked levels: 4.92 ms one face at a time over the lanes' cells (any open cell cost the whole warp a closest-point
 // test) -> 2.68 with 32 faces at a time -> 2.20 with the bins beyond d left out and the nearest rows first (90 -> 49
 // million candidates) -> 1.79 in rows of four cells -> 1.57 with the cull by spheres; own-bin candidates 2.46 -> 0.87.
+// Few or wide faces, and faces in many bins, are better taken one at a time (gather_pays in api.cu).
 template <int D, int PRED>
 __device__ __forceinline__ uint64_t mark_batch(const RefineLevel& a, uint32_t gid, const int* b, WarpSmem<D>& sm,
                                                uint32_t ns, uint64_t um, const BlockFrame<D>& F, const FastGeom& g,
@@ -837,7 +838,7 @@ __device__ __forceinline__ uint64_t mark_batch(const RefineLevel& a, uint32_t gi
 // 32, double-buffered: the next chunk is requested before the warp tests the
 // current one.
 constexpr uint32_t kFirstBatch = 8;  // faces of a block's first mark_batch
-template <int D, int PRED, bool kMarkOnly, typename OnSurv>
+template <int D, int PRED, bool kMarkOnly, bool kGather, typename OnSurv>
 __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParams& P, uint32_t gid, const int* b,
                                            WarpSmem<D>& sm, uint32_t& phase, int lane, WarpCounters& wc, bool& h0,
                                            bool& h1, OnSurv on_surv) {
@@ -911,7 +912,7 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
     }
   }
   // marks of the point predicate: the unmarked cells, their centres' box, the faces gathered for mark_batch
-  constexpr bool kMarkPoint = kPoint && kMarkOnly;
+  constexpr bool kMarkPoint = kPoint && kMarkOnly && kGather;
   uint64_t um = D == 3 ? ~0ull : 0xffffull;
   float ctr[3] = {F.cB[0], F.cB[1], D == 3 ? F.cB[D - 1] : 0.f}, half[3] = {1.5f * hf, 1.5f * hf, 1.5f * hf};
   uint32_t ns = 0, most = kFirstBatch;
@@ -1306,7 +1307,7 @@ __global__ void __launch_bounds__(256) k_entry_spheres(const Entry3* __restrict_
 
 // ENDS: 0 no geometry of the launch ends at this level, 1 all do, 2 some may (the point predicate's two walks share
 // no code: one kernel with both held 112 registers, and the walk that keeps records took 0.386 instead of 0.341 ms).
-template <int D, int PRED, int ENDS>
+template <int D, int PRED, int ENDS, bool GATHER>
 __global__ void __launch_bounds__(256) k_refine(RefineLevel a) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   WarpSmem<D>& sm = reinterpret_cast<WarpSmem<D>*>(s_raw)[threadIdx.x >> 5];
@@ -1344,7 +1345,7 @@ __global__ void __launch_bounds__(256) k_refine(RefineLevel a) {
     if (ENDS == 1 || (ENDS == 2 && fin)) {
       if constexpr (ENDS != 0) {
       uint32_t K = 0;  // records of this block (warp-uniform); past kRecCap into the warp's spill area
-      walk_block<D, PRED, false>(a, P, gid, b, sm, phase, lane, wc, h0, h1, [&](uint32_t f, bool r0, bool r1) {
+      walk_block<D, PRED, false, false>(a, P, gid, b, sm, phase, lane, wc, h0, h1, [&](uint32_t f, bool r0, bool r1) {
         cnt0 += r0 ? 1u : 0u;
         cnt1 += r1 ? 1u : 0u;
         if (a.recs) {
@@ -1369,7 +1370,7 @@ __global__ void __launch_bounds__(256) k_refine(RefineLevel a) {
       }
       }
     } else if constexpr (ENDS != 1) {
-      walk_block<D, PRED, true>(a, P, gid, b, sm, phase, lane, wc, h0, h1, [](uint32_t, bool, bool) {});
+      walk_block<D, PRED, true, GATHER>(a, P, gid, b, sm, phase, lane, wc, h0, h1, [](uint32_t, bool, bool) {});
       cnt0 = h0 ? 1u : 0u;
       cnt1 = h1 ? 1u : 0u;
     }
@@ -2097,7 +2098,7 @@ __device__ __forceinline__ void emit_block(const EmitArgs& a, unsigned blk, uint
       return;
     }
     bool h0 = false, h1 = false;
-    walk_block<D, PRED, false>(a.lv, P, gid, b, sm, phase, lane, wc, h0, h1,
+    walk_block<D, PRED, false, false>(a.lv, P, gid, b, sm, phase, lane, wc, h0, h1,
                          [&](uint32_t fc, bool r0, bool r1) { put(r0, r1, fc); });
     if (bad || c0 != n0 || c1 != n1) atomicOr(a.lv.err, ERR_OVERFLOW);
     if (!__all_sync(0xffffffffu, can0 && can1)) return;  // lists beyond the capacity (reported)
@@ -3298,21 +3299,27 @@ int launch_refine(const RefineLevel& a, int num_sms, cudaStream_t st) {
   }
   // one geometry: every block ends here or none does
   const int ends = mode == 0 ? 2 : (!a.blockcnt ? 0 : (a.table ? 2 : 1));
-  auto pick = [&](auto k0, auto k1, auto k2) { ends == 0 ? go(k0) : (ends == 1 ? go(k1) : go(k2)); };
+  auto pick = [&](auto k0, auto g0, auto k1, auto k2, auto g2) {
+    ends == 0 ? (a.gather ? go(g0) : go(k0)) : (ends == 1 ? go(k1) : (a.gather ? go(g2) : go(k2)));
+  };
   if (a.dim == 3) {
     if (mode == 2)
-      pick(k_refine<3, 2, 0>, k_refine<3, 2, 1>, k_refine<3, 2, 2>);
+      pick(k_refine<3, 2, 0, false>, k_refine<3, 2, 0, true>, k_refine<3, 2, 1, false>, k_refine<3, 2, 2, false>,
+           k_refine<3, 2, 2, true>);
     else if (mode == 1)
-      pick(k_refine<3, 1, 0>, k_refine<3, 1, 1>, k_refine<3, 1, 2>);
+      pick(k_refine<3, 1, 0, false>, k_refine<3, 1, 0, true>, k_refine<3, 1, 1, false>, k_refine<3, 1, 2, false>,
+           k_refine<3, 1, 2, true>);
     else
-      go(k_refine<3, 0, 2>);
+      go(k_refine<3, 0, 2, false>);
   } else {
     if (mode == 2)
-      pick(k_refine<2, 2, 0>, k_refine<2, 2, 1>, k_refine<2, 2, 2>);
+      pick(k_refine<2, 2, 0, false>, k_refine<2, 2, 0, true>, k_refine<2, 2, 1, false>, k_refine<2, 2, 2, false>,
+           k_refine<2, 2, 2, true>);
     else if (mode == 1)
-      pick(k_refine<2, 1, 0>, k_refine<2, 1, 1>, k_refine<2, 1, 2>);
+      pick(k_refine<2, 1, 0, false>, k_refine<2, 1, 0, true>, k_refine<2, 1, 1, false>, k_refine<2, 1, 2, false>,
+           k_refine<2, 1, 2, true>);
     else
-      go(k_refine<2, 0, 2>);
+      go(k_refine<2, 0, 2, false>);
   }
   return 1;
 }
