@@ -685,12 +685,21 @@ constexpr double kMaxFaceCells = 32768.0;
 // Automatic choice: face by face where the geometry's mean face covers at most
 // this many cells of the level (the block walk is cheaper once faces span many cells).
 constexpr double kAutoFaceCells = 1024.0;
-// The same in 3D where d is the cell size, for mask-only levels and for the records of a last level
-// (k_mark_cells: a face of 17 cells across takes as long as the walk; measured on 32^3 roots, 4 levels,
-// last level by faces / by the walk: 2.2 cells 1.06 / 1.94 ms for the refinement, 8.6 cells 0.48 / 0.61,
-// 13.8 cells 0.41 / 0.51, 19.6 cells 0.54 / 0.52).  In 2D the walk of the last level is never dearer than
-// the records' launches (0.33 / 0.35 ms for 20,000 edges).
+// The same in 3D where d is the cell size (k_mark_cells), for mask-only levels.
 constexpr double kAutoUnitCells = 8192.0;
+// The last level's records from the faces (3D, d the cell size) against the parents' walk, whole passes:
+//   mean face on 32^3 roots, 4 levels, refinement alone: 2.2 cells 1.06 / 1.94 ms, 8.6 cells 0.48 / 0.61, 13.8
+//     cells 0.41 / 0.51, 19.6 cells 0.54 / 0.52; 3,000 scattered faces of 15 cells 0.65 / 0.56: up to this many cells;
+//   the records' four launches cost about 15 us, so from 4,096 faces on, or 2,048 of two cells and more (10 faces
+//     0.236 / 0.219, 1,000 of 0.3 cells 0.278 / 0.264, 3,000 0.319 / 0.308 on average, 10,000 0.38 / 0.42; 3,000 of
+//     four cells 0.39 / 0.43);
+//   a warp takes a face, and up to 16 in a row, alone: one of 25 cells among 20,000 of two cells 0.81 / 0.84, twenty
+//     of 16 cells 1.06 / 0.88, of 20 cells 1.59 / 0.89, 400 of 12 cells 0.81 / 0.90.  So the widest face may have 13
+//     cells, or 1.75 times the mean (then all warps take as long).
+// In 2D the walk of the last level is never dearer than the records' launches (0.33 / 0.35 ms for 20,000 edges).
+constexpr double kAutoRecordCells = 5000.0;
+constexpr int64_t kRecordFaces = 4096;
+constexpr double kRecordWidest = 13.0, kRecordSpread = 1.75;
 
 // Links from the faces (k_flinks.cu) from this many (cell, face) pairs on: its seven launches cost about 30 us
 // more than the pair kernel's four (0.5 M links of 20 K faces 0.113 / 0.088 ms), from about 8 M links on it is
@@ -785,9 +794,23 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
   const bool any = p->face_pass != AMR_FACE_PASS_OFF && P.search == AMR_SEARCH_QUERY_BOX;
   // levels where geometries end: from the faces when that suits every one of them
   for (int L = 0; L < P.NL; ++L) P.rec_at[L] = any && P.adjacency && P.fin_at[L] && ctx->dom.dim == 3;
+  auto faces_of = [&](size_t gi) {
+    if (!ctx->multi) return ctx->nf;
+    return (gi + 1 < ctx->geoms.size() ? ctx->geoms[gi + 1].face_base : ctx->nf) - ctx->geoms[gi].face_base;
+  };
+  auto records_pay = [&](size_t gi, int L, int64_t n) {  // n: faces of all geometries that end at L
+    const double emax = gi < ctx->face_ext_max.size() ? std::ldexp(ctx->face_ext_max[gi], L) : INFINITY;
+    const double emean = gi < ctx->face_ext_mean.size() ? std::ldexp(ctx->face_ext_mean[gi], L) : INFINITY;
+    return n >= (emean >= 2.0 ? kRecordFaces / 2 : kRecordFaces) &&
+           emax <= std::max(kRecordWidest, kRecordSpread * emean);
+  };
+  int64_t n_end[AMR_MAX_LEVELS] = {};
+  for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) n_end[ctx->geoms[gi].n_levels - 1] += faces_of(gi);
   for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
     const int L = ctx->geoms[gi].n_levels - 1;
-    if (P.rec_at[L]) P.rec_at[L] = unit_of(ctx->geoms[gi]) && small_faces(gi, L, kMaxFaceCells, kAutoUnitCells);
+    if (P.rec_at[L])
+      P.rec_at[L] = unit_of(ctx->geoms[gi]) && small_faces(gi, L, kMaxFaceCells, kAutoRecordCells) &&
+                    (p->face_pass != AMR_FACE_PASS_AUTO || records_pay(gi, L, n_end[L]));
   }
   // links from the faces: every face that crosses a link has to be in the cell's list, by more than the band, and
   // the widest face's cells within what a warp of k_face_links holds

@@ -88,7 +88,7 @@ def test_refinement(kind):
     def call(g, dev):
         g.load(dev)
         g.bin(8)
-        r = g.refine(2, 0.0, 1.0, 19, True, True)
+        r = g.refine(2, 0.0, 1.0, 19, True, True, face_pass=2)
         torch.cuda.synchronize()
         return [lv["mask"].clone() for lv in r["levels"]] + [r[k].clone() for k in KEYS]
 

@@ -15,7 +15,7 @@ def _call(g, verts, bins, levels, graph):
     before = g.launch_count()
     g.load(torch.from_numpy(verts).cuda())
     g.bin(bins)
-    r = g.refine(levels, 0.0, 1.0, 19, True, True, use_graph=graph)
+    r = g.refine(levels, 0.0, 1.0, 19, True, True, use_graph=graph, face_pass=2)
     out = [lv[k].clone() for lv in r["levels"] for k in ("blocks", "mask", "flag")] + [r[k].clone() for k in KEYS]
     return out, r["graph_replay"], g.launch_count() - before
 
