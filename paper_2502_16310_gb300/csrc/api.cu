@@ -778,6 +778,17 @@ bool gather_pays(const amr_ctx* ctx, const Plan& P, size_t gi, int L) {
   return (D == 2 ? across >= 32.0 : across * across >= 16.0) && ctx->nnz <= 2 * ctx->nf;
 }
 
+// Marks where d is the cell size: widen the cells that a face meets (k_mark_cells: 16 faces per warp in packed steps),
+// or a warp per face over every inflated cell it reaches (k_mark_faces).  The steps cost about 2.5 us more than a
+// small face's test, so few small faces go the second way.  L: the geometry's last marked level.  us a level, warp
+// per face / widening, by the mean face's side in cells there: 3D, 10 to 300 faces, up to 0.9 cells 10.4 / 12.4, 1.9
+// cells 12.5 / 12.8, 3 cells 16 / 14; 1,000 faces 0.3 cells 15 / 16, 0.9 cells 42 / 18; 3,000 of 0.1 cells 18.0 / 21.2,
+// 4,000 of 0.3 22 / 17.  2D, up to 2,000 edges of 5 cells 9.3 / 10.6 to 17.0 / 17.9, 300 of 9 cells 17.9 / 14.8, 4,000 18 / 15.
+bool widening_pays(const amr_ctx* ctx, size_t gi, int L) {
+  const double side = gi < ctx->face_ext_mean.size() ? std::ldexp(ctx->face_ext_mean[gi], L > 0 ? L : 0) : INFINITY;
+  return ctx->nf > 3072 || side > (ctx->dom.dim == 2 ? 8.0 : ctx->nf > 512 ? 0.75 : 1.5);
+}
+
 // Per geometry and level: face by face or the block walk (face_levels bits of
 // the geometry rows, uploaded with the table); the plan's face_at / walk_at say
 // which of the two launches a level needs.  Returns a signature of the choice.
@@ -836,7 +847,8 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
       if (mask_only ? small_faces(gi, L, kMaxFaceCells, mean) : P.rec_at[L]) bits |= 1u << L;
     }
     // the inflated box is the 3^D cells around a cell exactly when d is the cell size on every level
-    const bool unit = unit_of(g);
+    const bool unit = unit_of(g) && (p->face_pass != AMR_FACE_PASS_AUTO || P.rec_at[g.n_levels - 1] ||
+                                     widening_pays(ctx, gi, g.n_levels - (P.adjacency ? 2 : 1)));
     if (bits && unit) bits |= kFaceUnit;
     g.face_levels = bits;
     const int64_t f0 = ctx->multi ? g.face_base : 0;
