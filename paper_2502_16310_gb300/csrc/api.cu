@@ -61,11 +61,12 @@ constexpr int SC_TOT = 16;   // [16] adjacency totals per level (pairs | cells <
 constexpr int SC_NL = 32;    // [16] links per level
 constexpr int SC_RUN = 48;   // [3] running cells, pairs, links
 constexpr int SC_REC = 52;   // [16] survivor records handed out per level
-constexpr int SC_RTOT = 68;    // records placed (the record scan's total)
+constexpr int SC_PLACED = 68;  // survivor records placed (zero between levels)
 constexpr int SC_HITS = 69;    // links from the faces: hits, runs, groups
 constexpr int SC_RUNS = 70;
 constexpr int SC_NGRP = 71;
-constexpr int SC_WORDS = 72;
+constexpr int SC_RTOT = 72;    // their runs (the run scan's total)
+constexpr int SC_WORDS = 74;
 
 // A captured graph stays valid while no buffer it uses was reallocated
 // (layout generation) and its by-value kernel arguments are unchanged.
@@ -1095,13 +1096,9 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
       uint64_t tot = 0;
       for (int attempt = 0; attempt < 2; ++attempt) {
         timed(ctx, st, "adj_scan", [&] {
-          int k = 0;
-          uint64_t* n_rec = static_cast<uint64_t*>(lb.desc.p);  // (the descriptors take their place)
-          if (P.rec_at[L]) {
-            k += launch_record_counts(a, n_rec, ctx->num_sms, st);
-            k += launch_scan_u64(n_rec, static_cast<uint64_t*>(lb.rfirst.p), lb.cap, ctx->d_scal + SC_N + L,
-                                 ctx->d_scal + SC_RTOT, ctx->scratch.p, ctx->d_err, ctx->num_sms, st);
-          }
+          const int k = P.rec_at[L] ? launch_record_counts(a, static_cast<uint64_t*>(lb.rfirst.p), ctx->d_scal + SC_PLACED,
+                                                           ctx->num_sms, st)
+                                    : 0;
           return k + launch_scan_u64(static_cast<const uint64_t*>(lb.blockcnt.p), static_cast<uint64_t*>(lb.base.p),
                                      lb.cap, ctx->d_scal + SC_N + L, ctx->d_scal + SC_TOT + L, ctx->scratch.p,
                                      ctx->d_err, ctx->num_sms, st);
@@ -1122,13 +1119,14 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         marks.lv = a;
         CK(cudaMemsetAsync(a.info, 0, sizeof(uint64_t) * (size_t)(lb.cap > 0 ? lb.cap : 1), st));
         CK(cudaMemsetAsync(a.rec_count, 0, sizeof(uint64_t), st));
+        CK(cudaMemsetAsync(ctx->d_scal + SC_PLACED, 0, sizeof(uint64_t), st));
         CK(cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned), st));
         timed(ctx, st, "mark_faces", [&] { return launch_mark_faces(marks, ctx->num_sms, st); });
       }
       if (P.rec_at[L])
         timed(ctx, st, "place_records", [&] {
-          return launch_place_records(a, static_cast<const uint64_t*>(lb.rfirst.p), ctx->d_scal + SC_TOT + L,
-                                      ctx->num_sms, st);
+          return launch_place_records(a, static_cast<const uint64_t*>(lb.rfirst.p), ctx->d_scal + SC_PLACED,
+                                      ctx->d_scal + SC_TOT + L, ctx->num_sms, st);
         });
       if (eager) {
         cells = (int64_t)(tot >> 32);

@@ -583,13 +583,13 @@ struct MarkArgs {
 };
 constexpr int kFaceBatch = 8;  // most faces a warp of the general kernel takes per work fetch
 int launch_mark_faces(const MarkArgs& m, int num_sms, cudaStream_t st);
-// A level whose records the faces left (lv.staged): blockcnt and the blocks' record counts; then, with
-// first = the exclusive scan of n_rec, the records by block and their descriptors (ERR_OVERFLOW when
-// more were left than cap_recs: no block has records then, and level_tot, the level's pairs | cells << 32,
-// is set to zero).
-int launch_record_counts(const RefineLevel& a, uint64_t* n_rec, int num_sms, cudaStream_t st);
-int launch_place_records(const RefineLevel& a, const uint64_t* first, uint64_t* level_tot, int num_sms,
-                         cudaStream_t st);
+// A level whose records the faces left (lv.staged): blockcnt and the place of each block's records (placed, a device
+// word that is zero before, hands them out); then the records by block and their descriptors, and placed zero again
+// (ERR_OVERFLOW when more were left than cap_recs: no block has records then, and level_tot, the level's pairs |
+// cells << 32, is set to zero).
+int launch_record_counts(const RefineLevel& a, uint64_t* first, uint64_t* placed, int num_sms, cudaStream_t st);
+int launch_place_records(const RefineLevel& a, const uint64_t* first, uint64_t* placed, uint64_t* level_tot,
+                         int num_sms, cudaStream_t st);
 
 // The algorithmic cell-face test count of one level (single geometry): per cell
 // of its blocks, the distinct faces in the bins its inflated box overlaps,
