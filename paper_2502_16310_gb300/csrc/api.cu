@@ -691,16 +691,17 @@ constexpr double kAutoUnitCells = 8192.0;
 // The last level's records from the faces (3D, d the cell size) against the parents' walk, whole passes:
 //   mean face on 32^3 roots, 4 levels, refinement alone: 2.2 cells 1.06 / 1.94 ms, 8.6 cells 0.48 / 0.61, 13.8
 //     cells 0.41 / 0.51, 19.6 cells 0.54 / 0.52; 3,000 scattered faces of 15 cells 0.65 / 0.56: up to this many cells;
-//   the records' four launches cost about 15 us, so from 4,096 faces on, or 2,048 of two cells and more (10 faces
-//     0.236 / 0.219, 1,000 of 0.3 cells 0.278 / 0.264, 3,000 0.319 / 0.308 on average, 10,000 0.38 / 0.42; 3,000 of
-//     four cells 0.39 / 0.43);
+//   the records' launches cost about 11 us, which 10 to 60 faces scattered over the domain do not give back (0.228 /
+//     0.215 ms a pass), 1,000 do (0.26 / 0.27), and closed surfaces, whose blocks have many faces, do from 80 on (0.160
+//     / 0.324; 320 faces 0.168 / 0.403): from 64 faces on;
 //   a warp takes a face, and up to 16 in a row, alone: one of 25 cells among 20,000 of two cells 0.81 / 0.84, twenty
-//     of 16 cells 1.06 / 0.88, of 20 cells 1.59 / 0.89, 400 of 12 cells 0.81 / 0.90.  So the widest face may have 13
-//     cells, or 1.75 times the mean (then all warps take as long).
+//     of 16 cells 1.06 / 0.88, of 20 cells 1.59 / 0.89, 400 of 12 cells 0.81 / 0.90; among 80,000 twenty of 16 cells 1.83 /
+//     2.02, of 20 cells 2.77 / 2.24.  So the widest face may have 13 cells, or 1.75 times the mean (then all warps take as
+//     long: a bumpy body of 46 K faces, mean 13.9, widest 20.6 cells 1.41 / 2.15), or 400 times its square are the faces.
 // In 2D the walk of the last level is never dearer than the records' launches (0.33 / 0.35 ms for 20,000 edges).
 constexpr double kAutoRecordCells = 5000.0;
-constexpr int64_t kRecordFaces = 4096;
-constexpr double kRecordWidest = 13.0, kRecordSpread = 1.75;
+constexpr int64_t kRecordFaces = 64;
+constexpr double kRecordWidest = 13.0, kEvenSpread = 1.75, kRecordMany = 400.0;
 
 // Links from the faces (k_flinks.cu) from this many (cell, face) pairs on: its seven launches cost about 30 us
 // more than the pair kernel's four (0.5 M links of 20 K faces 0.113 / 0.088 ms), from about 8 M links on it is
@@ -810,19 +811,24 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
     if (!ctx->multi) return ctx->nf;
     return (gi + 1 < ctx->geoms.size() ? ctx->geoms[gi + 1].face_base : ctx->nf) - ctx->geoms[gi].face_base;
   };
-  auto records_pay = [&](size_t gi, int L, int64_t n) {  // n: faces of all geometries that end at L
-    const double emax = gi < ctx->face_ext_max.size() ? std::ldexp(ctx->face_ext_max[gi], L) : INFINITY;
-    const double emean = gi < ctx->face_ext_mean.size() ? std::ldexp(ctx->face_ext_mean[gi], L) : INFINITY;
-    return n >= (emean >= 2.0 ? kRecordFaces / 2 : kRecordFaces) &&
-           emax <= std::max(kRecordWidest, kRecordSpread * emean);
-  };
+  // the faces of all geometries that end at a level: their number, and the widest of those geometries whose faces are
+  // uneven (its side in cells of the level)
   int64_t n_end[AMR_MAX_LEVELS] = {};
-  for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) n_end[ctx->geoms[gi].n_levels - 1] += faces_of(gi);
+  double uneven[AMR_MAX_LEVELS] = {};
   for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
     const int L = ctx->geoms[gi].n_levels - 1;
+    const bool known = gi < ctx->face_ext_max.size();
+    n_end[L] += faces_of(gi);
+    if (!known || ctx->face_ext_max[gi] > kEvenSpread * ctx->face_ext_mean[gi])
+      uneven[L] = std::max(uneven[L], known ? std::ldexp(ctx->face_ext_max[gi], L) : 1e6);
+  }
+  for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
+    const int L = ctx->geoms[gi].n_levels - 1;
+    const bool pays = n_end[L] >= kRecordFaces && (uneven[L] <= kRecordWidest ||
+                                                   (double)n_end[L] >= kRecordMany * uneven[L] * uneven[L]);
     if (P.rec_at[L])
       P.rec_at[L] = unit_of(ctx->geoms[gi]) && small_faces(gi, L, kMaxFaceCells, kAutoRecordCells) &&
-                    (p->face_pass != AMR_FACE_PASS_AUTO || records_pay(gi, L, n_end[L]));
+                    (p->face_pass != AMR_FACE_PASS_AUTO || pays);
   }
   // links from the faces: every face that crosses a link has to be in the cell's list, by more than the band, and
   // the widest face's cells within what a warp of k_face_links holds
