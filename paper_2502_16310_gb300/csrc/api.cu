@@ -670,6 +670,7 @@ struct Plan {
   FaceRange ending[AMR_MAX_LEVELS]; // faces of the geometries that end there
   bool lines_at[AMR_MAX_LEVELS];    // links of the level can be found from the faces (k_flinks.cu) ...
   double reach[AMR_MAX_LEVELS];     // ... the smallest d / h of the geometries that end there
+  int64_t line_pairs[AMR_MAX_LEVELS];  // ... and are from this many (cell, face) pairs on
   bool rec_at[AMR_MAX_LEVELS];      // the faces leave the records of every geometry that ends at the level
   bool walk_at[AMR_MAX_LEVELS];     // some geometry's blocks of the level are walked
   bool gather_at[AMR_MAX_LEVELS];   // mark-only walks of the point predicate gather faces (mark_batch)
@@ -704,11 +705,16 @@ constexpr int64_t kRecordFaces = 64;
 constexpr double kRecordWidest = 13.0, kEvenSpread = 1.75, kRecordMany = 400.0;
 
 // Links from the faces (k_flinks.cu) from this many (cell, face) pairs on: its seven launches cost about 30 us
-// more than the pair kernel's four (0.5 M links of 20 K faces 0.113 / 0.088 ms), from about 8 M links on it is
-// the faster (8 K faces 0.39 / 0.38 ms, 32 K faces 0.41 / 0.46, 97 M links of 72 K faces 3.13 / 4.37).  The pair
-// kernel's time goes by pairs, this one's by links: where d is below the cell size (fewer pairs per link) the line
-// is three times higher (d = 0.75 h: 6.2 M pairs 0.46 / 0.42, 21.6 M 1.25 / 1.36, 327 M 15.4 / 20.3; d = 1.5 h:
-// 13.5 M 0.46 / 0.66, 47 M 1.25 / 2.18, 724 M 15.4 / 33.0).
+// more than the pair kernel's four (0.5 M links of 20 K faces 0.113 / 0.088 ms), but where d is the cell size or more
+// it is the faster from 2 to 3 M pairs on (us by faces / by pairs: 2.5 M pairs of 6 cell faces 131 to 183 / 188, 3.2 M
+// of 2 cells 150 / 225, 3.7 M of 12 cells 183 / 262; 29 M 1,190 / 1,610, 424 M 14,900 / 24,200).  The pair kernel's
+// time goes by pairs, this one's by links: where d is below the cell size (fewer pairs per link) the line is three
+// times higher (d = 0.75 h: 6.2 M pairs 0.46 / 0.42 ms, 21.6 M 1.25 / 1.36, 327 M 15.4 / 20.3; d = 1.5 h: 13.5 M 0.46 /
+// 0.66, 47 M 1.25 / 2.18, 724 M 15.4 / 33.0).
+// A warp works on up to eight faces in a row alone, 1.35 us times the square of their side in cells when they are
+// wide, and the faces' way is some 25 us sooner for 2^20 pairs: where the widest face is well above the mean, the line
+// lies at side^2 / 20 2^20 pairs (twenty faces of 16 cells among 120 K of two: 6.5 M pairs 543 / 422 us, 13 M 0.53 / 0.70
+// ms; 400 of 12 cells 7.1 M 417 / 428 us; 400 of 20 cells 7.2 M 890 / 470, 14 M 0.91 / 0.75 ms).
 constexpr int64_t kFaceLinkPairs = 4 << 20;
 
 // Cells of level L in the range of a face of geometry g whose largest AABB side
@@ -843,6 +849,11 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
     P.reach[L] = std::min(P.reach[L], g.d_abs / hL + g.d_rel);
     P.lines_at[L] = P.lines_at[L] && P.reach[L] >= 1.001 * link_reach(P.pred) &&
                     std::pow(emax * std::ldexp(1.0, L) + 6.0 + range_margin(ctx, g, L, emax), 3.0) <= kMaxFaceCells;
+  }
+  for (int L = 0; L < P.NL; ++L) {
+    P.line_pairs[L] = (P.reach[L] < 1.0 ? 3 : 1) * kFaceLinkPairs;
+    if (p->face_pass == AMR_FACE_PASS_AUTO && P.lines_at[L])
+      P.line_pairs[L] = std::max(P.line_pairs[L], (int64_t)(uneven[L] * uneven[L] / 20.0 * 1048576.0));
   }
   for (int L = 0; L < P.NL; ++L) P.gather_at[L] = P.pred == AMR_PRED_POINT;  // where it pays for every geometry's walk
   for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
@@ -1170,7 +1181,7 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         return launch_advance(ctx->d_scal + SC_TOT + L, nullptr, ctx->d_scal + SC_RUN,
                               static_cast<uint32_t*>(ctx->adj_off.p), ctx->cap_cells, ctx->d_err, true, st);
       });
-      if (eager) ctx->face_links[L] = P.lines_at[L] && pairs >= (P.reach[L] < 1.0 ? 3 : 1) * kFaceLinkPairs;
+      if (eager) ctx->face_links[L] = P.lines_at[L] && pairs >= P.line_pairs[L];
       if (P.links && ctx->face_links[L]) {  // (a capture follows the eager pass before it)
         // the links are found from the faces
         FaceLinkArgs fl{};
