@@ -110,7 +110,7 @@ struct amr_ctx {
   bool multi = false;
   DevBuf table, face_gid;
   // buffers
-  DevBuf X, nrm, frec, recs, staged, hkeys, hvals, mkeys, mvals, cls, flbase, tl_cell, tl_dir, tl_q, tl_face, stage_a, stage_b, frange, count, offsets, ids, payload, scratch, misc, scal;
+  DevBuf X, nrm, frec, recs, staged, hkeys, hvals, mkeys, mvals, cls, cls_open, flbase, tl_cell, tl_dir, tl_q, tl_face, stage_a, stage_b, frange, count, offsets, ids, payload, scratch, misc, scal;
   LevelBufs lv[AMR_MAX_LEVELS];
   DevBuf adj_cell, adj_off, adj_ids, link_cell, link_dir, link_q, link_face, link_stage;
   DevBuf hit_q, hit_code, run_staged, runs, grp_runs, grp_first, grp_links, grp_base;  // links from the faces
@@ -523,7 +523,7 @@ amr_status amr_ctx_init(amr_ctx* ctx) {
 void amr_ctx_free(amr_ctx* ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   drop_graph(ctx);
-  DevBuf* all[] = {&ctx->X, &ctx->frec, &ctx->recs, &ctx->staged, &ctx->hkeys, &ctx->hvals, &ctx->mkeys, &ctx->mvals, &ctx->cls, &ctx->flbase,
+  DevBuf* all[] = {&ctx->X, &ctx->frec, &ctx->recs, &ctx->staged, &ctx->hkeys, &ctx->hvals, &ctx->mkeys, &ctx->mvals, &ctx->cls, &ctx->cls_open, &ctx->flbase,
                    &ctx->tl_cell, &ctx->tl_dir, &ctx->tl_q, &ctx->tl_face, &ctx->nrm,          &ctx->stage_a,    &ctx->stage_b,    &ctx->frange,
                    &ctx->count,     &ctx->offsets,      &ctx->ids,        &ctx->payload,    &ctx->scratch,
                    &ctx->misc,      &ctx->scal,         &ctx->adj_cell,   &ctx->adj_off,    &ctx->adj_ids,
@@ -1815,6 +1815,8 @@ amr_status amr_classify_nodes(amr_ctx* ctx, const uint8_t** cell_solid, int64_t*
   const int64_t n = r.n_adj_cells;
   cudaStream_t st = ctx->stream;
   TRY(ensure(ctx, ctx->cls, (size_t)(n > 0 ? n : 1)));
+  const int64_t open_cap = std::min<int64_t>(n, 1 << 20);
+  TRY(ensure_aux(ctx, ctx->cls_open, sizeof(uint32_t) * (size_t)open_cap));
   CK(cudaMemsetAsync(ctx->counters + CNT_CLASS_FALLBACK, 0, sizeof(unsigned long long), st));
   ClassifyArgs a{};
   a.dim = ctx->dom.dim;
@@ -1832,6 +1834,8 @@ amr_status amr_classify_nodes(amr_ctx* ctx, const uint8_t** cell_solid, int64_t*
   a.X = static_cast<const float*>(ctx->X.p);
   a.nf = ctx->nf;
   a.cls = static_cast<uint8_t*>(ctx->cls.p);
+  a.open_rows = static_cast<uint32_t*>(ctx->cls_open.p);
+  a.open_cap = open_cap;
   a.counters = ctx->counters;
   a.err = ctx->d_err;
   timed(ctx, st, "classify", [&] { return launch_classify(a, st); });

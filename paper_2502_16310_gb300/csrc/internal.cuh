@@ -667,6 +667,8 @@ struct ClassifyArgs {
   const float* X;              // faces (SoA), for the winding-number fallback
   int64_t nf;
   uint8_t* cls;
+  uint32_t* open_rows;         // 3D: rows of cells left to the winding number, room for open_cap
+  int64_t open_cap;
   unsigned long long* counters;
   unsigned* err;
 };
