@@ -225,15 +225,25 @@ __global__ void __launch_bounds__(kKWarps * 32) k_classify_3(ClassifyArgs a) {
     int xb[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) xb[i] = __shfl_sync(0xffffffffu, my_xb, i);
-    const int y0 = __shfl_sync(0xffffffffu, yb, 0), y1 = __shfl_sync(0xffffffffu, yb, 3);
-    const int z0 = __shfl_sync(0xffffffffu, zb, 0), z1 = __shfl_sync(0xffffffffu, zb, 12);
     const float by0 = __shfl_sync(0xffffffffu, pyh, 0), by1 = __shfl_sync(0xffffffffu, pyh, 3);
     const float bz0 = __shfl_sync(0xffffffffu, pzh, 0), bz1 = __shfl_sync(0xffffffffu, pzh, 12);
     const float tol = 1e-6f * (fmaxf(fabsf(by0), fabsf(by1)) + fmaxf(fabsf(bz0), fabsf(bz1)) + 1.0f);
     const float d0 = 5.7e-14f * (fabsf(pyh) + fabsf(pzh) + fabsf(P.org_hi[1]) + fabsf(P.org_hi[2]));  // 2^-44: hi + lo
     uint32_t solid = 0, open = 0;  // of the lane's line, from its half of the entries: parity, undecided
-    for (int z = z0; z <= z1; ++z)
-      for (int y = y0; y <= y1; ++y) {
+    // the rows of bins that hold a ray, each once (where bins are finer than cells, most rows between them hold none:
+    // 180 faces on 16^3 cells, 128^3 bins 0.69 ms with all rows walked, now 0.07)
+    int zp = -1;
+#pragma unroll 1
+    for (int iz = 0; iz < 4; ++iz) {
+      const int z = __shfl_sync(0xffffffffu, zb, 4 * iz);
+      if (z == zp) continue;
+      zp = z;
+      int yp = -1;
+#pragma unroll 1
+      for (int iy = 0; iy < 4; ++iy) {
+        const int y = __shfl_sync(0xffffffffu, yb, iy);
+        if (y == yp) continue;
+        yp = y;
         const int64_t bin = P.bin_base + (int64_t)P.B * (y + (int64_t)P.B * z);
         const uint32_t j0 = a.offsets[bin + xb[0]], j1 = a.offsets[bin + P.B];
         const bool mine = yb == y && zb == z;  // the lane's ray lies in this row of bins
@@ -317,6 +327,7 @@ __global__ void __launch_bounds__(kKWarps * 32) k_classify_3(ClassifyArgs a) {
           __syncwarp();  // the next entries reuse the places
         }
       }
+    }
     solid ^= __shfl_xor_sync(0xffffffffu, solid, 16);
     open |= __shfl_xor_sync(0xffffffffu, open, 16);
     // the lane's half of its line: cells 2 half and 2 half + 1
