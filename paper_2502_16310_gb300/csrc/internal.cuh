@@ -800,7 +800,7 @@ int launch_advance(const uint64_t* level_tot, const uint64_t* n_links, uint64_t*
 // What a face's links share in the adjoint (see k_face_lines).
 struct __align__(16) FaceLines {
   float v0[3];
-  int extent;
+  uint32_t scale;              // bytes: exponent + 126 of the bound on w per axis; bits of the number of links
   float inv[9];
   float pad[3];
 };

@@ -121,11 +121,12 @@ __device__ __forceinline__ void acc2(float& hi, float& lo, float x) {
 // face ids, ranks by __match_any_sync), adds each face's terms in double-float
 // and sends one set of sums per face to global memory.  There the sums of a
 // face's tiles are added as integers: the terms are fixed point with a scale per
-// face (the largest |grad_q / (c . n)| of its links, which a first kernel finds,
-// and the face's extent), so the result does not depend on the order of the
-// tiles.  The spacing is 2^-30 of the face's largest term for 2^32 links (2^-33
-// for 5e8), below the FP32 rounding of that term itself.  What depends on the
-// face alone (the 9 lines' 1 / (c . n), the extent) is worked out once per face.
+// face and axis (the largest |grad_q / (c . n)| of its links, which a first kernel finds, the face's extent
+// along the axis and a bound on its number of links), so the result does not depend on the order of the
+// tiles.  With b bits for the number the spacing is 2^-(62 - b) of the bound: 2^-51 for a face of 10 cells
+// across (b = 11; 22 for one of 600 cells).  With the number of all links and the largest axis for every face it was
+// 2^-33 at 5e8 links: less than the double-float sums of a tile hold.  What depends on the face alone (the 9
+// lines' 1 / (c . n), the bounds) is worked out once per face.
 //
 // Bound by instructions (the grouping, the positions, the double-float sums), at
 // 9 bytes a link in the first kernel and 17 and the cell's in the second.  Before,
@@ -187,8 +188,11 @@ __device__ __forceinline__ const GeomParams& face_geom(const AdjointArgs& a, int
 }
 
 // Per face what its links' terms need: v0, the lines' 1 / (c . n) of the scaled normal (0: parallel,
-// no link), and the exponent r with |v0 - x - t d| < 2^r for every point x + t d of the face (twice
-// its extent, since a certified hit may lie outside it by its rounding, and the rounding of t d).
+// no link), per axis the exponent r with |v0 - x - t d| < 2^r for every point x + t d of the face (twice its
+// extent, since a certified hit may lie outside it by its rounding, and the rounding of t d), and the bits b
+// of its number of links: a lattice line meets the face in at most four (the cells before and after the
+// crossing, two of each where it is a node), and a convex region of area A and perimeter U holds at most
+// A + U / 2 + 1 points of a unit lattice (Nosarzewska's bound; the face projected along the line, in units of h).
 template <int D, bool MULTI>
 __global__ void __launch_bounds__(256) k_face_lines(AdjointArgs a) {
   for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < a.nf; f += (int64_t)gridDim.x * blockDim.x) {
@@ -203,14 +207,20 @@ __global__ void __launch_bounds__(256) k_face_lines(AdjointArgs a) {
       lo[c] *= scale;
     }
     FaceLines L{};
-    float m = 0.f;
+    float e[2][3] = {};  // the edges from v0
 #pragma unroll
     for (int c = 0; c < D; ++c) {
       L.v0[c] = a.X[(int64_t)c * a.nf + f];
+      float m = 0.f;
 #pragma unroll
-      for (int k = 1; k < D; ++k) m = fmaxf(m, fabsf(a.X[(int64_t)(D * k + c) * a.nf + f] - L.v0[c]));
+      for (int k = 1; k < D; ++k) {
+        e[k - 1][c] = a.X[(int64_t)(D * k + c) * a.nf + f] - L.v0[c];
+        m = fmaxf(m, fabsf(e[k - 1][c]));
+      }
+      L.scale |= (__float_as_uint(fmaf(3.8e-6f, h, 2.0f * m)) >> 23) << (8 * c);
     }
-    L.extent = (int)(__float_as_uint(fmaf(3.8e-6f, h, 2.0f * m)) >> 23) - 126;
+    const float ih = 1.0f / h;
+    float lines = 0.f;  // lattice lines through the face
     constexpr int kPlus3[9] = {1, 3, 5, 7, 9, 11, 13, 15, 17}, kPlus2[4] = {1, 2, 5, 6};
 #pragma unroll
     for (int l = 0; l < (D == 3 ? 9 : 4); ++l) {
@@ -220,7 +230,22 @@ __global__ void __launch_bounds__(256) k_face_lines(AdjointArgs a) {
         c[q] = D == 3 ? (float)d3q19_c(kPlus3[l], q) : (q < 2 ? (float)d2q9_c(kPlus2[l < 4 ? l : 0], q) : 0.f);
       const float den = (c[0] * hi[0] + c[1] * hi[1] + c[2] * hi[2]) + (c[0] * lo[0] + c[1] * lo[1] + c[2] * lo[2]);
       L.inv[l] = den == 0.f ? 0.f : 1.0f / den;
+      // the projection along the line: axes i < j with a part of c (i: the first of them or the only one), w the third
+      if constexpr (D == 3) {
+        const int n_axes = (c[0] != 0.f) + (c[1] != 0.f) + (c[2] != 0.f);
+        const int i = c[0] != 0.f ? 0 : (c[1] != 0.f ? 1 : 2);
+        const int j = n_axes == 2 ? (c[2] != 0.f ? 2 : 1) : (i + 1) % 3, w = 3 - i - j;
+        const float s = n_axes == 2 ? c[i] * c[j] : 0.f;
+        const float p0 = e[0][j] - s * e[0][i], p1 = e[1][j] - s * e[1][i], q0 = e[0][w], q1 = e[1][w];
+        const float area = 0.5f * fabsf(p0 * q1 - q0 * p1), rim = fabsf(p0) + fabsf(q0) + fabsf(p1) + fabsf(q1) +
+                                                                  fabsf(p1 - p0) + fabsf(q1 - q0);
+        lines += area * ih * ih + 0.5f * rim * ih + 1.0f;
+      } else if (l < 4) {
+        lines += fabsf(c[0] * e[0][1] - c[1] * e[0][0]) * ih + 1.0f;
+      }
     }
+    const int bits = (int)(__float_as_uint(4.1f * lines + 4.0f) >> 23) - 126;
+    L.scale |= (uint32_t)min(a.count_bits, bits) << 24;
     reinterpret_cast<FaceLines*>(a.face_lines)[f] = L;
   }
 }
@@ -441,12 +466,17 @@ __global__ void __launch_bounds__(kSWarps * 32, kSBlocks) k_face_sums(AdjointArg
         if (ok && (lane == 0 || ((heads >> lane) & 1u))) {
           const uint32_t f = sm.face[g0 + j], key = __ldg(a.face_key + f);
           if (key != 0u && key != kNonFinite) {
-            const int k = 62 - a.count_bits, r = __ldg(&a.face_lines[f].extent);
+            const uint32_t sc = __ldg(&a.face_lines[f].scale);
+            const int b = (int)(sc >> 24), k = 62 - b;
+            // no more than so many bounds (t of a face nearly along its line may be off): the sums stay below 2^63
+            const uint32_t cnt = min((uint32_t)(sm.at[g0 + j + 1] - sm.at[g0 + j]), 1u << min(b, 16));
+            const long long lim = (long long)cnt << k;
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-              // terms below 1 (W: below 2^extent): the sums stay below 2^62
-              const double x = ((double)hi[v] + (double)lo[v]) * __hiloint2double((1023 + k - (v < D ? r : 0)) << 20, 0);
-              const long long n = __double2ll_rn(x);
+              // terms below 1 (W: below 2^r)
+              const int r = v < D ? (int)((sc >> (8 * v)) & 255u) - 126 : 0;
+              const double x = ((double)hi[v] + (double)lo[v]) * __hiloint2double((1023 + k - r) << 20, 0);
+              const long long n = min(max(__double2ll_rn(x), -lim), lim);
               if (n) atomicAdd(a.face_acc + (int64_t)f * NV + v, (unsigned long long)n);
             }
           }
@@ -476,13 +506,14 @@ __global__ void __launch_bounds__(256) k_face_grad(AdjointArgs a) {
     const float scale = normal_scale(fmaxf(fmaxf(fabsf(nh[0]), fabsf(nh[1])), fabsf(nh[2])));
     // grad_q / (d . n) of the sums: the terms left out h, the power of two of the scaled normal and the key's
     const double unit = scalbn((double)scale / ((double)fg.h_hi + (double)fg.h_lo), (int)key - 253);
-    const int kS = 62 - a.count_bits;
-    const int kW = kS - a.face_lines[f].extent;
+    const uint32_t sc = a.face_lines[f].scale;
+    const int k = 62 - (int)(sc >> 24);
     double v[4];
 #pragma unroll
-    for (int j = 0; j < NV; ++j)
-      v[j] = (double)(long long)a.face_acc[f * NV + j] *
-             __hiloint2double((1023 - (j < D ? kW : kS)) << 20, 0) * unit;
+    for (int j = 0; j < NV; ++j) {
+      const int r = j < D ? (int)((sc >> (8 * j)) & 255u) - 126 : 0;
+      v[j] = (double)(long long)a.face_acc[f * NV + j] * __hiloint2double((1023 - k + r) << 20, 0) * unit;
+    }
     double X[D][D];
 #pragma unroll
     for (int k = 0; k < D; ++k)
