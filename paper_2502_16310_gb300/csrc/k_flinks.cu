@@ -421,8 +421,11 @@ __global__ void __launch_bounds__(kFWarps * 32, kFBlocks) k_face_links(FaceLinkA
           const float Pb = ob - ln.sg * oa;
           T.Pb = Pb;
           T.Qb = ow;
-          // (an edge function beyond this is beyond k_links' own bound, too: 8 u |c|_1 M, M <= 2 L^2)
-          T.e = 64.0f * kU32 * F.L * F.L;
+          // Beyond this k_links certifies the edge, too.  Offsets of a line inside the projection are at most 2 L in P
+          // and L in Q, and within 8.2 u L (a difference of two vertex coordinates, the line's place, their difference,
+          // each rounded) and 3 u L of their values, so an edge function is within 2 (2 L 3 u L + L 8.2 u L) + 6 u L^2 <
+          // 35 u L^2.  k_links asks for 8 u |c|_1 M and is itself within 4 u |c|_1 M, M <= 2 L^2: 48 u L^2 more.
+          T.e = 96.0f * kU32 * F.L * F.L;
           // c . n and the crossing's place along line (u, v)
           float dh, de;
           df_two_sum(F.nh[ln.a], ln.sg * F.nh[ln.b], dh, de);
