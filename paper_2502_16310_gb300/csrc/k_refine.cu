@@ -608,9 +608,9 @@ constexpr int kFewFp64 = 6;
 // sat_adjacent_fp64_3 by a whole warp, an axis per lane (the same operations in the same order per axis,
 // so the same decision and band): an FP64 operation takes tens of cycles here, and one pair's 13 axes in
 // a row held its warp for tens of microseconds, which on a small mesh is longer than the rest of a level.
-// Every lane passes the same arguments and gets the decision.
-__device__ __noinline__ bool resolve_sat_warp(const RefineLevel& a, uint32_t gid, uint32_t face, int b0, int b1, int b2,
-                                              int cell_local, bool* band) {
+// Every lane passes the same arguments and gets the decision (bit 0; bit 1: in the band).
+__device__ __noinline__ uint32_t resolve_sat_warp(const RefineLevel& a, uint32_t gid, uint32_t face, int b0, int b1,
+                                                  int b2, int cell_local) {
   const int lane = threadIdx.x & 31;
   const GeomParams& P = a.table ? a.table[gid] : a.g0;
   const double h = scalbn(P.h0, -a.level);
@@ -659,8 +659,7 @@ __device__ __noinline__ bool resolve_sat_warp(const RefineLevel& a, uint32_t gid
   const unsigned sep = __ballot_sync(0xffffffffu, axis && g > 0.0);
   const unsigned big = __ballot_sync(0xffffffffu, axis && g > 0.0 && !small);
   const unsigned near0 = __ballot_sync(0xffffffffu, axis && !(g > 0.0) && small);
-  *band = sep ? big == 0u : near0 != 0u;
-  return sep == 0u;
+  return (sep == 0u ? 1u : 0u) | ((sep ? big == 0u : near0 != 0u) ? 2u : 0u);
 }
 
 // Per-warp shared memory of the walk: survivor data, a double buffer of bin
@@ -1182,19 +1181,20 @@ __device__ __forceinline__ void walk_block(const RefineLevel& a, const GeomParam
           cell_test2<D>(S, o0, o1, t0, t1);
         }
         if constexpr (D == 3 && !kPoint) {
-          uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h0) && t0 == 2) |
-                       ((uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h1) && t1 == 2) << 32);
-          if (__popcll(u) > kFewFp64) u = 0;  // (a lane each, below)
-          for (; u; u &= u - 1) {
-            const int cell = __ffsll((long long)u) - 1;
-            bool in_band;
-            const int t = resolve_sat_warp(a, gid, S.face, b[0], b[1], b[2], cell, &in_band) ? 1 : 0;
-            if (lane == 0) {
-              ++wc.fb;
-              wc.band += in_band ? 1ull : 0ull;
+          if (__any_sync(0xffffffffu, (!(kMarkOnly && h0) && t0 == 2) || (!(kMarkOnly && h1) && t1 == 2))) {
+            uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h0) && t0 == 2) |
+                         ((uint64_t)__ballot_sync(0xffffffffu, !(kMarkOnly && h1) && t1 == 2) << 32);
+            if (__popcll(u) > kFewFp64) u = 0;  // (a lane each, below)
+            for (; u; u &= u - 1) {
+              const int cell = __ffsll((long long)u) - 1;
+              const uint32_t w = resolve_sat_warp(a, gid, S.face, b[0], b[1], b[2], cell);
+              if (lane == 0) {
+                ++wc.fb;
+                wc.band += w >> 1;
+              }
+              if (cell == lane) t0 = (int)(w & 1u);
+              if (cell == lane + 32) t1 = (int)(w & 1u);
             }
-            if (cell == lane) t0 = t;
-            if (cell == lane + 32) t1 = t;
           }
         }
         bool r0 = false, r1 = false;
@@ -1468,6 +1468,16 @@ struct GroupCounters {
   uint32_t fb = 0, band = 0, cand = 0, surv = 0, big = 0;
 };
 
+// FP64 decision of one (cell, face) pair of a group (the per-block walk's resolution).
+__device__ __noinline__ bool resolve_group(const RefineLevel& a, uint32_t gid, uint32_t face, const int* b,
+                                           int cell_local, GroupCounters& wc) {
+  unsigned long long fb = 0, band = 0;
+  const bool r = resolve_fp64<3>(a, gid, face, b, cell_local, &fb, &band);
+  wc.fb += (uint32_t)fb;
+  wc.band += (uint32_t)band;
+  return r;
+}
+
 // One parent group: walk, culls and cell tests.  kMark: only the masks are
 // wanted (the walk ends once every cell of the 8 children is marked); else the
 // per-cell counts and the survivor records of the finest level are kept.
@@ -1604,27 +1614,26 @@ __device__ __forceinline__ void walk_group(const RefineLevel& a, const GeomParam
           int t0 = 0, t1 = 0;
           cell_test2<3>(S, o0, o1, t0, t1);
           const int bj[3] = {c0[0] + cx, c0[1] + cy, c0[2] + cz};  // child j's block coordinates
-          // pairs not certified in FP32: many a lane each, a few one after another by the whole warp
-          uint64_t u = (uint64_t)__ballot_sync(0xffffffffu, !m0 && t0 == 2) |
-                       ((uint64_t)__ballot_sync(0xffffffffu, !m1 && t1 == 2) << 32);
-          if (__popcll(u) > kFewFp64) {
-            unsigned long long nf = 0, nb = 0;
-            if (!m0 && t0 == 2) t0 = resolve_fp64<3>(a, gid, S.face, bj, lane, &nf, &nb) ? 1 : 0;
-            if (!m1 && t1 == 2) t1 = resolve_fp64<3>(a, gid, S.face, bj, lane + 32, &nf, &nb) ? 1 : 0;
-            wc.fb += (unsigned)nf;
-            wc.band += (unsigned)nb;
-            u = 0;
-          }
-          for (; u; u &= u - 1) {
-            const int cell = __ffsll((long long)u) - 1;
-            bool in_band;
-            const int t = resolve_sat_warp(a, gid, S.face, bj[0], bj[1], bj[2], cell, &in_band) ? 1 : 0;
-            if (lane == 0) {
-              ++wc.fb;
-              wc.band += in_band ? 1u : 0u;
+          // pairs not certified in FP32: many a lane each, a few one after another by the whole warp (one vote first,
+          // for few faces have any; by value, for the walk's registers are full)
+          if (__any_sync(0xffffffffu, (!m0 && t0 == 2) || (!m1 && t1 == 2))) {
+            uint32_t u0 = __ballot_sync(0xffffffffu, !m0 && t0 == 2), u1 = __ballot_sync(0xffffffffu, !m1 && t1 == 2);
+            if (__popc(u0) + __popc(u1) > kFewFp64) {
+              if (!m0 && t0 == 2) t0 = resolve_group(a, gid, S.face, bj, lane, wc) ? 1 : 0;
+              if (!m1 && t1 == 2) t1 = resolve_group(a, gid, S.face, bj, lane + 32, wc) ? 1 : 0;
+            } else {
+              while (u0 | u1) {
+                const int cell = u0 ? __ffs(u0) - 1 : 31 + __ffs(u1);
+                if (u0) u0 &= u0 - 1; else u1 &= u1 - 1;
+                const uint32_t w = resolve_sat_warp(a, gid, S.face, bj[0], bj[1], bj[2], cell);
+                if (lane == 0) {
+                  ++wc.fb;
+                  wc.band += w >> 1;
+                }
+                if (cell == lane) t0 = (int)(w & 1u);
+                if (cell == lane + 32) t1 = (int)(w & 1u);
+              }
             }
-            if (cell == lane) t0 = t;
-            if (cell == lane + 32) t1 = t;
           }
           const bool r0 = !m0 && t0 != 0, r1 = !m1 && t1 != 0;
           hb0 |= (uint32_t)r0 << j;
@@ -3115,12 +3124,11 @@ __global__ void __launch_bounds__(kCellWarps * 32, kCellBlocks) k_mark_cells(Mar
               const uint32_t e = __shfl_sync(0xffffffffu, pend, k);
               int z[3];
               const MarkFace<D>& Q = *cell_at(e, z);
-              bool in_band;
-              const bool adj = resolve_sat_warp(a, Q.gid, Q.face, z[0] >> 2, z[1] >> 2, z[2] >> 2, (int)(e & 63u), &in_band);
+              const uint32_t w = resolve_sat_warp(a, Q.gid, Q.face, z[0] >> 2, z[1] >> 2, z[2] >> 2, (int)(e & 63u));
               if (lane == 0) {
                 ++wc.fb;
-                wc.band += in_band ? 1ull : 0ull;
-                if (adj) atomicOr(out + 2 * (e >> 6) + ((e >> 5) & 1u), 1u << (e & 31u));
+                wc.band += w >> 1;
+                if (w & 1u) atomicOr(out + 2 * (e >> 6) + ((e >> 5) & 1u), 1u << (e & 31u));
               }
             }
           }
