@@ -687,21 +687,24 @@ constexpr double kMaxFaceCells = 32768.0;
 // Automatic choice: face by face where the geometry's mean face covers at most
 // this many cells of the level (the block walk is cheaper once faces span many cells).
 constexpr double kAutoFaceCells = 1024.0;
-// The same in 3D where d is the cell size (k_mark_cells), for mask-only levels.
+// The same in 3D where d is the cell size (k_mark_cells), for mask-only levels; fewer than 64 faces are too few warps for
+// it (a box of 12 faces on cell planes, 8 to 16 cells wide 1.24 ms on two levels, 0.85 by the walk).
 constexpr double kAutoUnitCells = 8192.0;
+constexpr int64_t kUnitFaces = 64;
 // The last level's records from the faces (3D, d the cell size) against the parents' walk, whole passes:
 //   mean face on 32^3 roots, 4 levels, refinement alone: 2.2 cells 1.06 / 1.94 ms, 8.6 cells 0.48 / 0.61, 13.8
-//     cells 0.41 / 0.51, 19.6 cells 0.54 / 0.52; 3,000 scattered faces of 15 cells 0.65 / 0.56: up to this many cells;
+//     cells 0.41 / 0.51, 19.6 cells 0.54 / 0.52; of 15 cells 3,700 close together 0.71 / 1.01, 3,000 scattered 0.65 /
+//     0.56, but 100 to 1,000 scattered 0.42 / 0.30 and 0.54 / 0.42: kAutoUnitCells from 2,048 faces on, this below;
 //   the records' launches cost about 11 us, which 10 to 60 faces scattered over the domain do not give back (0.228 /
-//     0.215 ms a pass), 1,000 do (0.26 / 0.27), and closed surfaces, whose blocks have many faces, do from 80 on (0.160
-//     / 0.324; 320 faces 0.168 / 0.403): from 64 faces on;
+//     0.215 ms a pass), but closed surfaces, whose blocks have many faces, do (a box of 12 faces 0.33 / 0.53, 80 faces 0.160 /
+//     0.324, 320 0.168 / 0.403), and 1,000 scattered ones (0.26 / 0.27);
 //   a warp takes a face, and up to 16 in a row, alone: one of 25 cells among 20,000 of two cells 0.81 / 0.84, twenty
 //     of 16 cells 1.06 / 0.88, of 20 cells 1.59 / 0.89, 400 of 12 cells 0.81 / 0.90; among 80,000 twenty of 16 cells 1.83 /
 //     2.02, of 20 cells 2.77 / 2.24.  So the widest face may have 13 cells, or 1.75 times the mean (then all warps take as
 //     long: a bumpy body of 46 K faces, mean 13.9, widest 20.6 cells 1.41 / 2.15), or 400 times its square are the faces.
 // In 2D the walk of the last level is never dearer than the records' launches (0.33 / 0.35 ms for 20,000 edges).
 constexpr double kAutoRecordCells = 5000.0;
-constexpr int64_t kRecordFaces = 64;
+constexpr int64_t kRecordFaces = 2048;
 constexpr double kRecordWidest = 13.0, kEvenSpread = 1.75, kRecordMany = 400.0;
 
 // Links from the faces (k_flinks.cu) from this many (cell, face) pairs on: its seven launches cost about 30 us
@@ -788,13 +791,14 @@ bool gather_pays(const amr_ctx* ctx, const Plan& P, size_t gi, int L) {
 
 // Marks where d is the cell size: widen the cells that a face meets (k_mark_cells: 16 faces per warp in packed steps),
 // or a warp per face over every inflated cell it reaches (k_mark_faces).  The steps cost about 2.5 us more than a
-// small face's test, so few small faces go the second way.  L: the geometry's last marked level.  us a level, warp
-// per face / widening, by the mean face's side in cells there: 3D, 10 to 300 faces, up to 0.9 cells 10.4 / 12.4, 1.9
-// cells 12.5 / 12.8, 3 cells 16 / 14; 1,000 faces 0.3 cells 15 / 16, 0.9 cells 42 / 18; 3,000 of 0.1 cells 18.0 / 21.2,
-// 4,000 of 0.3 22 / 17.  2D, up to 2,000 edges of 5 cells 9.3 / 10.6 to 17.0 / 17.9, 300 of 9 cells 17.9 / 14.8, 4,000 18 / 15.
+// small face's test, so few small faces go the second way; among more there is often one with a pair for FP64, which
+// holds its warp there for 20 to 60 us.  L: the geometry's last marked level.  us a level, warp per face / widening, by
+// the mean face's side in cells there: 3D, 10 to 500 faces up to 0.9 cells 10.2 / 12.4 (with a pair for FP64 29), 1.9 cells
+// 12.5 / 12.8, 3 cells 16 / 14; 1,000 of 0.9 cells 42 / 18; 2,000 of 0.3 cells 14 / 17 to 46 / 25.  2D, up to 2,000 edges of 5
+// cells 9.3 / 10.6 to 17.0 / 17.9, 300 of 9 cells 17.9 / 14.8, 4,000 18 / 15.
 bool widening_pays(const amr_ctx* ctx, size_t gi, int L) {
   const double side = gi < ctx->face_ext_mean.size() ? std::ldexp(ctx->face_ext_mean[gi], L > 0 ? L : 0) : INFINITY;
-  return ctx->nf > 3072 || side > (ctx->dom.dim == 2 ? 8.0 : ctx->nf > 512 ? 0.75 : 1.5);
+  return ctx->dom.dim == 2 ? ctx->nf > 3072 || side > 8.0 : ctx->nf > 512 || side > 1.5;
 }
 
 // Per geometry and level: face by face or the block walk (face_levels bits of
@@ -830,10 +834,10 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
   }
   for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
     const int L = ctx->geoms[gi].n_levels - 1;
-    const bool pays = n_end[L] >= kRecordFaces && (uneven[L] <= kRecordWidest ||
-                                                   (double)n_end[L] >= kRecordMany * uneven[L] * uneven[L]);
+    const bool pays = uneven[L] <= kRecordWidest || (double)n_end[L] >= kRecordMany * uneven[L] * uneven[L];
+    const double mean = n_end[L] >= kRecordFaces ? kAutoUnitCells : kAutoRecordCells;
     if (P.rec_at[L])
-      P.rec_at[L] = unit_of(ctx->geoms[gi]) && small_faces(gi, L, kMaxFaceCells, kAutoRecordCells) &&
+      P.rec_at[L] = unit_of(ctx->geoms[gi]) && small_faces(gi, L, kMaxFaceCells, mean) &&
                     (p->face_pass != AMR_FACE_PASS_AUTO || pays);
   }
   // links from the faces: every face that crosses a link has to be in the cell's list, by more than the band, and
@@ -861,7 +865,7 @@ uint64_t assign_face_levels(amr_ctx* ctx, Plan& P, const amr_refine_params* p) {
     uint32_t bits = 0;
     for (int L = 0; any && L < g.n_levels; ++L) {
       const bool mask_only = L < g.n_levels - 1 || !P.adjacency;
-      const double mean = unit_of(g) && ctx->dom.dim == 3 ? kAutoUnitCells : kAutoFaceCells;
+      const double mean = unit_of(g) && ctx->dom.dim == 3 && ctx->nf >= kUnitFaces ? kAutoUnitCells : kAutoFaceCells;
       if (mask_only ? small_faces(gi, L, kMaxFaceCells, mean) : P.rec_at[L]) bits |= 1u << L;
     }
     // the inflated box is the 3^D cells around a cell exactly when d is the cell size on every level

@@ -16,7 +16,7 @@ def _soup(n, cells, wide, width):
     return np.concatenate([t, rng.uniform(0.2, 0.8, (wide, 1, 3)) + w]).astype(np.float32)
 
 
-@pytest.mark.parametrize("n,cells,wide,width,by_faces", [(40, 2, 0, 0, False), (100, 2, 0, 0, True),
+@pytest.mark.parametrize("n,cells,wide,width,by_faces", [(40, 2, 0, 0, True), (300, 25, 0, 0, False),
                                                          (5000, 2, 10, 12, True), (5000, 2, 10, 20, False),
                                                          (60000, 1, 2, 20, False), (170000, 1, 2, 20, True)])
 def test_route(n, cells, wide, width, by_faces):
