@@ -185,11 +185,12 @@ typedef struct {
                                  neighbour blocks (3^D - 1) of every marked block; single-geometry only */
   int keep_previous;          /* 1: keep the previous call's block lists for amr_adapt_diff (re-adaptation of
                                  a moving or changing geometry); single-geometry only */
-  int face_pass;              /* levels whose only output is the mask (every level above the finest, and the
-                                 finest without adjacency): AMR_FACE_PASS_AUTO (0) marks them face by face where
-                                 that is expected to be cheaper than the block walk, _OFF (1) never, _ON (2)
-                                 wherever it applies (single geometry, AMR_SEARCH_QUERY_BOX, block coordinates
-                                 below 2^21).  Results are identical either way. */
+  int face_pass;              /* whether the faces do the work of a level: marks of levels whose only output is the mask
+                                 (every level above the finest, and the finest without adjacency), in 3D with d the
+                                 cell size the finest level's lists too, and the links of 3D levels with millions of
+                                 (cell, face) pairs.  AMR_FACE_PASS_AUTO (0): where that is expected to be cheaper
+                                 than the block walk and the pair kernel, _OFF (1) never, _ON (2) wherever it applies
+                                 (AMR_SEARCH_QUERY_BOX, faces up to 32,768 cells).  Results are identical either way. */
 } amr_refine_params;
 enum { AMR_PRED_BOX = 0, AMR_PRED_POINT = 1 };
 enum { AMR_SEARCH_QUERY_BOX = 0, AMR_SEARCH_OWN_BIN = 1 };
@@ -209,8 +210,10 @@ enum { AMR_FACE_PASS_AUTO = 0, AMR_FACE_PASS_OFF = 1, AMR_FACE_PASS_ON = 2 };
  *   link_dir   device u8  [n_links]: lattice direction 1..Q-1
  *   link_q     device f32 [n_links]: smallest t in [0,1] with centre + t*c_i*h on a face
  *   link_face  device u32 [n_links]: the face hit at q (smallest id on ties)
- * Diagnostics: n_fallback = close decisions re-evaluated in FP64; n_band = those
- * whose FP64 margin was within 1e-6*h (adjacency) or 1e-6 (links) of the boundary. */
+ * Diagnostics (of the work that ran, so they depend on how a level was marked and its links were found, and on the
+ * order of concurrent marks): n_fallback = close decisions re-evaluated in FP64; n_band = those whose FP64 margin
+ * was within 1e-6*h (adjacency) or 1e-6 (links) of the boundary.  A close pair that a certain neighbour settles is in
+ * neither. */
 typedef struct {
   int n_levels;
   int64_t n_blocks[AMR_MAX_LEVELS];
@@ -230,9 +233,11 @@ typedef struct {
   const uint32_t* link_face;
   int64_t n_fallback;
   int64_t n_band;
-  int64_t n_candidates;       /* (block, face) candidate pairs read from the bins, all levels */
+  int64_t n_candidates;       /* (block, face) candidate pairs read from the bins, all walked levels (0 on levels marked
+                                 from the faces; the point predicate's gathered walk counts a face once per bin) */
   int64_t n_survivors;        /* candidates that passed the block-level test */
-  int64_t n_link_candidates;  /* (cell, face, direction) triples that passed the plane-range filter */
+  int64_t n_link_candidates;  /* (cell, face, direction) triples that passed the plane-range filter; where a level's
+                                 links are found from the faces, the hits (3D) */
   int64_t n_face_setups;      /* faces set up by the face-by-face marking (face_pass), all its levels */
   int64_t n_face_tests;       /* (face, cell) tests it ran */
   int graph_replay;           /* 1: the level loop ran as a replay of the captured graph; 0: eagerly (first

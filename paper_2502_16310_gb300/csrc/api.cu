@@ -1194,7 +1194,6 @@ amr_status engine_pass(amr_ctx* ctx, const Plan& P, bool eager, bool slack, cuda
         fl.table = a.table;
         fl.face_gid = ctx->multi ? static_cast<const uint32_t*>(ctx->face_gid.p) : nullptr;
         fl.rec = static_cast<const FaceRec3*>(ctx->frec.p);
-        fl.nf = ctx->nf;
         fl.faces = P.ending[L];
         for (int l = 0; l < L; ++l) fl.first_child[l] = static_cast<const int32_t*>(ctx->lv[l].first.p);
         fl.n_blocks = lb.cap;

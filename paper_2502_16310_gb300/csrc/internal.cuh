@@ -734,8 +734,8 @@ struct LinkArgs {
   unsigned* err;
 };
 
-// Links found from the faces (k_flinks.cu): 3D, a level below the roots whose survivor records the
-// faces left.  Hits leave as runs, one per (face, group), a group being the 8 blocks of one parent.
+// Links found from the faces (k_flinks.cu): 3D, a level below the roots.  Hits leave as runs, one per
+// (face, group), a group being the 8 blocks of one parent.
 struct StagedRun {
   unsigned long long start;    // first hit
   uint32_t n, face;
@@ -751,7 +751,6 @@ struct FaceLinkArgs {
   const GeomParams* table;
   const uint32_t* face_gid;
   const FaceRec3* rec;
-  int64_t nf;
   FaceRange faces;             // of the geometries that end at the level
   const int32_t* first_child[kMaxLevels];
   int64_t n_blocks;            // capacity of the level (n_dev: its count)

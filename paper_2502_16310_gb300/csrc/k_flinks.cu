@@ -1,5 +1,5 @@
-// k_flinks.cu — wall links of a level whose survivor records the faces left (3D, box predicate, d the
-// cell size): the links are found from the faces too.
+// k_flinks.cu — wall links found from the faces: a 3D level below the roots, either predicate, any d that puts every
+// face a link can cross into its cell's list (0.5 h; point predicate sqrt(2) h), faces up to 26 cells wide.
 //
 // A lattice line (a row of cell centres along one of the 9 lines of D3Q19) that crosses a face at one
 // point gives at most two links of the face: the cell before the point links forward across it with

@@ -198,7 +198,7 @@ struct BlockFrame {
 // the block frame, the cell-level intervals [tmin - r|a|_1, tmax + r|a|_1] and
 // their error bounds.  Returns false when some axis certifiably separates the
 // face from the whole inflated block.  Without kCull (face-by-face marking, which has no block) the face is
-// kept whatever the block would say; returns 16 u (P + O + r) then, the error bound of a unit axis.
+// kept whatever the block would say.
 //
 // Error bound per axis a: every computed projection, interval end and cell
 // coordinate differs from its exact value by at most a few unit roundoffs of
@@ -206,8 +206,7 @@ struct BlockFrame {
 // covers the rounding of the frame origin, of the edges when they are not
 // exact and of the FP32 normal relative to the FP64 one).  eps = 16 u (P+O+r)|a|_1.
 template <int D, bool kCull = true>
-__device__ __forceinline__ auto setup_face(const float* V, const float* nh, const BlockFrame<D>& F, Surv<D>& S)
-    -> std::conditional_t<kCull, bool, float> {
+__device__ __forceinline__ bool setup_face(const float* V, const float* nh, const BlockFrame<D>& F, Surv<D>& S) {
   float p[3][3];
   float P = 0.f;
 #pragma unroll
@@ -276,10 +275,7 @@ __device__ __forceinline__ auto setup_face(const float* V, const float* nh, cons
     S.e[0] = e0;
     S.e[1] = e1;
   }
-  if constexpr (kCull)
-    return true;
-  else
-    return scale;
+  return true;
 }
 
 // Cell tests of the lane's two cells against one survivor: 0 = separated,
