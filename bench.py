@@ -46,7 +46,8 @@ OPS_LINK_FACE = 150.0         # per (adjacent cell, face), executed on top: doub
                               # cross products and the line filters (reported beside the roofline, not in it)
 OPS_LINK_LINE = 60.0          # per link found from the faces: half a lattice line's three edge functions, one plane
                               # offset in double-float
-FACE_LINK_PAIRS = 4 << 20     # from this many pairs on a 3D level's links are found from the faces (csrc/api.cu)
+FACE_LINK_PAIRS = 4 << 20     # from this many pairs on a 3D level's links are found from the faces: csrc/api.cu's rule
+                              # for even meshes with d the cell size or more, which the 3D workloads here all are
 # DRAM bytes (read + write) per launch of the current kernels, from one ncu capture each
 # (dram__bytes_read.sum + dram__bytes_write.sum, one pass) of the named workload; others report null
 MEASURED_TRAFFIC = {}
